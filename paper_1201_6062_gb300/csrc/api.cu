@@ -19,6 +19,7 @@
 #include "batch.h"
 #include "plan.h"
 #include "tc.h"
+#include "dig.h"
 #include "lanczos.h"
 #include "sync.cuh"
 #include "rkf.h"
@@ -130,6 +131,15 @@ struct tdse_ctx {
     int nb = 0, ldb = 0;
     int tc_B = 0;                       // batch size the plane buffers / maps were built for
     tdse::TcMaps tc_maps{};
+    // digit-sliced batches on the tensor cores (FP64 / FP32 / float-float contexts):
+    // row exponents and digits of the dipole blocks (built by the first such
+    // batch), the maxima and digits of the states and the field values
+    DevBuf dgE, dgU, dgmax, dgX, dgF;
+    bool dg_ready = false;
+    DevBuf dgscr;
+    int dg_B = 0;                       // batch size the state digits / maps were built for
+    tdse::DigTile dg_tile{};
+    tdse::DigMaps dg_maps{};
     int tc_persistent = 1;              // all stages of a batch in one launch (tdse_set_batch_persistent)
     MvPlan plan;
     SysDesc desc{};                    // host copy of the descriptor (static fields filled)
@@ -428,6 +438,118 @@ static tdse_status propagate_batch_tc(tdse_ctx *ctx, double *c, const double *fi
     }
     CUDA_TRY(tdse::launch_tc_out(ctx->tc_c.as<float4>(), (double2 *)c, N * B, s));
     ctx->launches += 1;
+    return TDSE_OK;
+}
+
+// ------------------------------------------- digit-sliced batches (dig.cuh) --
+// Whether a batch of B pulses runs as digit-sliced products on the tensor
+// cores.  Against the FMA-pipe GEMMs (FP32, float-float) they win at every
+// measured shape (1.1x-6.7x a stage: lmax=15, n=1000, 256 pulses 546 against
+// 3645 us float-float, 388 against 945 us FP32) but short rows with many
+// pulses, where most of a 128-row tile is padding (n=40, 200 pulses: 50
+// against 36 us; n=60: 45 against 48).  FP64 batches otherwise run pulse by
+// pulse: one stage of lmax=7, n=301 takes 29 us a pulse, 67 us for 2 and 70 us
+// for 4 pulses here.
+static bool dig_wanted(const tdse_ctx *ctx, int B)
+{
+    if (ctx->lmax < 1) return false;
+    return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
+}
+
+// Device storage, dipole digits and tensor maps of a digit-sliced batch; false
+// when they cannot be had (memory, or a stream under capture before the
+// digits exist): the caller then takes the FMA-pipe path.
+static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
+{
+    const int S = tdse::dig_slices(ctx->prec), L = ctx->lmax + 1, n = ctx->n;
+    const int ldb = (n + 7) & ~7, nb = (n + 63) & ~63;
+    const tdse::DigTile tile = tdse::dig_tile(S, n, B);
+    const long long plane = (long long)L * nb;
+    const size_t ub = sizeof(__nv_bfloat16) * 2 * S * (size_t)ctx->lmax * n * ldb;
+    const size_t xb = sizeof(__nv_bfloat16) * S * 2 * (size_t)B * plane;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
+    const bool grown = ctx->dgX.bytes < xb || ctx->bx.bytes < sizeof(double2) * (size_t)B * ctx->N ||
+                       ctx->dgF.bytes < sizeof(double) * 3 * (size_t)B * nsteps;
+    if (cap != cudaStreamCaptureStatusNone && (!ctx->dg_ready || ctx->dg_B != B || grown)) return false;
+    bool ok = ctx->bx.ensure(sizeof(double2) * (size_t)B * ctx->N) == cudaSuccess &&
+              ctx->bacc.ensure(sizeof(double2) * (size_t)B * ctx->N) == cudaSuccess &&
+              ctx->dgmax.ensure(sizeof(int) * 2 * 2 * (size_t)B * L) == cudaSuccess &&
+              ctx->dgF.ensure(sizeof(double) * 3 * (size_t)B * nsteps) == cudaSuccess;
+    if (ok && !ctx->dg_ready) {
+        ok = ctx->dgE.ensure(sizeof(int) * 2 * (size_t)ctx->lmax * n) == cudaSuccess &&
+             ctx->dgU.ensure(ub) == cudaSuccess &&
+             tdse::launch_dig_u(ctx->prec, ctx->U.p, ctx->bstride, ctx->ld, n, ctx->lmax, ldb, ctx->dgE.as<int>(),
+                                ctx->dgU.as<__nv_bfloat16>(), s) == cudaSuccess;
+        const cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)(2 * S * ctx->lmax)};
+        const cuuint64_t strides[2] = {(cuuint64_t)ldb * 2, (cuuint64_t)n * ldb * 2};
+        const cuuint32_t box[3] = {64, 128, 1};
+        ok = ok && make_map(&ctx->dg_maps.U, ctx->dgU.p, 3, dims, strides, box) == TDSE_OK;
+        ctx->dg_ready = ok;
+        ctx->launches += 3;
+    }
+    if (ok && ctx->dg_B != B) {
+        ok = ctx->dgX.ensure(xb) == cudaSuccess && ctx->dgscr.ensure(tdse::dig_scratch_bytes(tile)) == cudaSuccess &&
+             cudaMemsetAsync(ctx->dgX.p, 0, xb, s) == cudaSuccess;   // padding columns stay zero
+        const cuuint64_t dims[3] = {(cuuint64_t)plane, (cuuint64_t)(2 * B), (cuuint64_t)S};
+        const cuuint64_t strides[2] = {(cuuint64_t)plane * 2, (cuuint64_t)(2 * B) * plane * 2};
+        const cuuint32_t box[3] = {64, (cuuint32_t)(tile.bn / tile.cg), 1};
+        ok = ok && make_map(&ctx->dg_maps.X, ctx->dgX.p, 3, dims, strides, box) == TDSE_OK;
+        ctx->dg_B = ok ? B : 0;
+        ctx->dg_tile = tile;
+    }
+    if (!ok) {
+        (void)cudaGetLastError();
+        g_err.clear();
+        if (!ctx->dg_ready) { ctx->dgU.release(); ctx->dgE.release(); }
+        ctx->dgX.release();
+        ctx->dg_B = 0;
+    }
+    return ok;
+}
+
+static tdse_status propagate_batch_dig(tdse_ctx *ctx, double *c, const double *field, int B, int sps, double dt,
+                                       long nsteps, tdse_scheme scheme, int order, int hold, cudaStream_t s)
+{
+    const int S = tdse::dig_slices(ctx->prec), L = ctx->lmax + 1, n = ctx->n, nb = (n + 63) & ~63;
+    int *xm = ctx->dgmax.as<int>();
+    const size_t slot = (size_t)L * 2 * B;
+    CUDA_TRY(cudaMemsetAsync(xm, 0, sizeof(int) * slot, s));
+    CUDA_TRY(tdse::launch_dig_field(field, (int)((long)sps * nsteps + 1), sps, nsteps, B, ctx->dgF.as<double>(), s));
+    CUDA_TRY(tdse::launch_dig_max((const double2 *)c, n, ctx->lmax, B, xm, s));
+    ctx->launches += 2;
+    tdse::DigArgs A{};
+    A.n = n;
+    A.lmax = ctx->lmax;
+    A.B = B;
+    A.nb = nb;
+    A.N = ctx->N;
+    A.E = ctx->E.as<double>();
+    A.eu = ctx->dgE.as<int>();
+    A.c = (double2 *)c;
+    A.x = ctx->bx.as<double2>();
+    A.acc = ctx->bacc.as<double2>();
+    A.mode = scheme == TDSE_RK4 ? tdse::EPI_RK4 : tdse::EPI_TAYLOR;
+    A.order = order;
+    A.gauge = ctx->desc.gauge;
+    A.scratch = ctx->dgscr.p;
+    A.err = ctx->errw.as<int>();
+    const int q0 = scheme == TDSE_RK4 ? 0 : 1, q1 = scheme == TDSE_RK4 ? 3 : order;
+    long t = 0;
+    for (long k = 0; k < nsteps; ++k) {
+        for (int q = q0; q <= q1; ++q, ++t) {
+            const int h = scheme == TDSE_RK4 ? (q == 0 ? 0 : (q == 3 ? 2 : 1)) : (hold ? 1 : 0);
+            A.stage = q;
+            A.step = scheme == TDSE_RK4 ? (q == 3 ? dt / 6.0 : (q == 2 ? dt : 0.5 * dt)) : dt / (double)q;
+            A.fval = ctx->dgF.as<double>() + ((size_t)k * 3 + h) * B;
+            A.xmax = xm + (t & 1) * slot;
+            A.xmax_next = xm + ((t + 1) & 1) * slot;
+            CUDA_TRY(tdse::launch_dig_x(S, q == q0 ? A.c : A.x, n, nb, ctx->lmax, B, A.xmax, A.xmax_next,
+                                        ctx->dgX.as<__nv_bfloat16>(), s));
+            CUDA_TRY(tdse::launch_dig(S, ctx->dg_tile, ctx->dg_maps, A, s));
+            ctx->launches += 2;
+        }
+    }
     return TDSE_OK;
 }
 
@@ -1173,6 +1295,8 @@ tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, 
         if (nsteps == 0) return TDSE_OK;
         return propagate_batch_tc(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, s);
     }
+    if (scheme != TDSE_LANCZOS && nsteps > 0 && dig_wanted(ctx, B) && dig_prepare(ctx, B, nsteps, s))
+        return propagate_batch_dig(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, s);
     if (ctx->prec == TDSE_DF32 && scheme != TDSE_LANCZOS) {
         if (nsteps == 0) return TDSE_OK;
         return propagate_batch_df(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, s);

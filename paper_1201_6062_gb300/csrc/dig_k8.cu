@@ -1,0 +1,14 @@
+// Digit-sliced batched products of FP64 contexts: 8 digits per operand (dig.cuh).
+#include "dig.cuh"
+
+namespace tdse {
+
+const void *dig_fn8(int cg, int bn)
+{
+    if (cg == 1 && bn == 32) return (const void *)dig_kernel<8, 32, 1>;
+    if (cg == 1 && bn == 64) return (const void *)dig_kernel<8, 64, 1>;
+    if (cg == 2 && bn == 64) return (const void *)dig_kernel<8, 64, 2>;
+    return nullptr;
+}
+
+}  // namespace tdse

@@ -1,0 +1,159 @@
+"""The digit-sliced batched products (csrc/dig.cuh) at the edges of their
+tiles: rows (128, 256), K rounds (64, 512), pulses per tile (16, 32, 64), end
+blocks, both gauges, graded and zero states, non-finite states, and the path
+that takes over when their storage cannot be had."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1201_6062_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+DIGITS = {"fp32": 4, "df32": 6, "fp64": 8}
+# error of the products, relative 2-norm, that the FMA- and FP64-pipe kernels show at these sizes
+NORM = {"fp32": 6e-7, "df32": 1e-11, "fp64": 2e-15}
+# state arithmetic (float-float sums of the products: 2^-46 of the largest; FP64 elsewhere)
+SUM = {"fp32": 2.0 ** -46, "df32": 2.0 ** -46, "fp64": 2.0 ** -50}
+
+
+def product(T, prec, lmax, n, U, C, gauge="length"):
+    """(1 - i D) c - c for every state: one Taylor term of order 1, E = 0, f = dt = 1."""
+    B = len(C)
+    H = T.Hamiltonian(np.zeros((lmax + 1) * n), U, lmax, n, prec)
+    if gauge != "length":
+        H.set_gauge(gauge)
+    c = torch.from_numpy(C.copy()).cuda()
+    H.propagate_batch(c, torch.ones(B, 2, dtype=torch.float64, device="cuda"), B, 1.0, 1, "taylor", order=1)
+    H.sync()
+    H.close()
+    return c.cpu().numpy() - C
+
+
+def draw(lmax, n, B, seed, graded=False):
+    rng = np.random.default_rng(seed)
+    U = rng.standard_normal((lmax, n, n)) / np.sqrt(n)
+    C = rng.standard_normal((B, (lmax + 1) * n)) + 1j * rng.standard_normal((B, (lmax + 1) * n))
+    if graded:
+        # every block and pulse on a scale of its own
+        C *= np.exp(rng.uniform(-40, 10, (B, lmax + 1))).repeat(n, axis=1)
+        U *= np.exp(rng.uniform(-20, 5, (lmax, n, 1)))
+    return U, C
+
+
+def check(prec, lmax, n, U, C, k, gauge="length"):
+    S = DIGITS[prec]
+    x = C.reshape(len(C), lmax + 1, n)
+    k = k.reshape(x.shape)
+    amax = np.maximum(np.abs(x.real).max(2), np.abs(x.imag).max(2))          # [B, L]
+    for l in range(lmax + 1):
+        ref = np.zeros((len(C), n), np.complex128)
+        bound = np.zeros((len(C), n))
+        if l < lmax:
+            ref += (1j if gauge == "velocity" else 1.0) * (x[:, l + 1] @ U[l].T)
+            bound += amax[:, l + 1, None] * np.abs(U[l]).max(1)[None]
+        if l >= 1:
+            ref += (-1j if gauge == "velocity" else 1.0) * (x[:, l - 1] @ U[l - 1])
+            bound += amax[:, l - 1, None] * np.abs(U[l - 1]).max(0)[None]
+        # digits left out: S - 1 pairs of weight S and half a unit of either operand's last
+        # digit, against maxima rounded up to powers of two (one bit more for S = 8)
+        bound = n * bound * (S * 2.0 ** (4 - 8 * S) + SUM[prec]) + 2.0 ** -51 * (np.abs(x[:, l]) + np.abs(ref))
+        err = np.abs(k[:, l] - -1j * ref)
+        assert np.all(err <= 2 * bound), (l, float((err / np.maximum(bound, 1e-300)).max()))
+        # relative to each pulse's block; the subtraction of c costs FP64 rounding of c
+        nrm = np.linalg.norm(err, axis=1) - 2.0 ** -52 * np.linalg.norm(x[:, l], axis=1)
+        assert np.all(nrm <= NORM[prec] * np.linalg.norm(ref, axis=1) + 1e-300), (l, nrm / np.linalg.norm(ref, axis=1))
+
+
+SHAPES = [(1, 64, 1), (2, 65, 16), (1, 127, 17), (3, 128, 32), (1, 129, 33), (2, 200, 64), (1, 256, 65), (1, 257, 3),
+          (2, 513, 9), (1, 640, 40)]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+@pytest.mark.parametrize("lmax,n,B", SHAPES)
+def test_products_at_tile_edges(tdse_lib, prec, lmax, n, B):
+    U, C = draw(lmax, n, B, 11 * n + B)
+    C *= 1e3                                      # the products, not c, set the size of the result
+    check(prec, lmax, n, U * 1e3, C, product(tdse_lib, prec, lmax, n, U * 1e3, C))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+@pytest.mark.parametrize("gauge", ["length", "velocity"])
+def test_graded_blocks_keep_their_own_scale(tdse_lib, prec, gauge):
+    lmax, n, B = 3, 150, 20
+    U, C = draw(lmax, n, B, 5, graded=True)
+    C[3] = 0.0
+    C[4, n:2 * n] = 0.0
+    k = product(tdse_lib, prec, lmax, n, U, C, gauge)
+    assert not np.any(k[3])
+    x = C.reshape(B, lmax + 1, n)
+    S = DIGITS[prec]
+    for l in range(lmax + 1):
+        up, dn = np.zeros((B, n), np.complex128), np.zeros((B, n), np.complex128)
+        bound = 2.0 ** -50 * np.abs(x[:, l])
+        if l < lmax:
+            up = (1j if gauge == "velocity" else 1.0) * (x[:, l + 1] @ U[l].T)
+            bound = bound + (S * 2.0 ** (4 - 8 * S) + SUM[prec]) * n * np.abs(x[:, l + 1]).max(1)[:, None] * np.abs(U[l]).max(1)
+        if l >= 1:
+            dn = (-1j if gauge == "velocity" else 1.0) * (x[:, l - 1] @ U[l - 1])
+            bound = bound + (S * 2.0 ** (4 - 8 * S) + SUM[prec]) * n * np.abs(x[:, l - 1]).max(1)[:, None] * np.abs(U[l - 1]).max(0)
+        err = np.abs(k.reshape(x.shape)[:, l] - -1j * (up + dn))
+        assert np.all(err <= 2 * (bound + 2.0 ** -50 * (np.abs(up) + np.abs(dn)))), l
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_non_finite_pulse_stays_alone(tdse_lib, prec, bad):
+    lmax, n, B = 2, 140, 18
+    U, C = draw(lmax, n, B, 6)
+    clean = product(tdse_lib, prec, lmax, n, U, C)
+    C2 = C.copy()
+    C2[7, n + 5] = bad
+    k = product(tdse_lib, prec, lmax, n, U, C2)
+    assert not np.any(np.isfinite(k[7, :n].real) & np.isfinite(k[7, :n].imag))
+    assert np.array_equal(np.delete(k, 7, 0), np.delete(clean, 7, 0))
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("df32", 1e-10), ("fp64", 1e-10)])
+@pytest.mark.parametrize("scheme,order,sps", [("rk4", 4, 2), ("taylor", 3, 1)])
+def test_windows_match_the_oracle(tdse_lib, prec, tol, scheme, order, sps):
+    lmax, n, B, dt, steps = 3, 140, 19, 0.02, 12
+    E, U = inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8)
+    C = np.stack([inputs.random_state((lmax + 1) * n, b) for b in range(B)])
+    F = np.stack([inputs.field_samples(0.1 + 0.01 * b, 0.5, dt, steps, sps, cycles=3, t0=3.0) for b in range(B)])
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, prec)
+    c = torch.from_numpy(C.copy()).cuda()
+    H.propagate_batch(c, torch.from_numpy(F).cuda(), B, dt, steps, scheme, order=order, samples_per_step=sps)
+    H.sync()
+    # again on the same context with fewer pulses (other digit planes and tiles)
+    c2 = torch.from_numpy(C[:3].copy()).cuda()
+    H.propagate_batch(c2, torch.from_numpy(F[:3].copy()).cuda(), 3, dt, steps, scheme, order=order, samples_per_step=sps)
+    H.sync()
+    H.close()
+    for b in range(B):
+        args = (lmax, n, E, U, C[b], F[b], dt, steps)
+        ref, _ = oracle.rk4(*args, samples_per_step=sps) if scheme == "rk4" else oracle.taylor(*args, order, samples_per_step=sps)
+        for got in ([c[b]] if b >= 3 else [c[b], c2[b]]):
+            assert np.linalg.norm(got.cpu().numpy() - ref) < tol * np.linalg.norm(ref), b
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("df32", 1e-10), ("fp64", 1e-10)])
+def test_without_room_for_digits_the_other_path_serves(tdse_lib, prec, tol):
+    lmax, n, B, dt, steps = 2, 200, 12, 0.02, 3
+    E, U = inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8)
+    C = np.stack([inputs.random_state((lmax + 1) * n, b) for b in range(B)])
+    F = np.full((B, steps + 1), 0.1)
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, prec)
+    used = tdse_lib.device_memory_in_use()
+    tdse_lib.set_device_memory_limit(used + 4 * 16 * B * (lmax + 1) * n + 65536)    # the batch's own vectors, no digits
+    try:
+        c = torch.from_numpy(C.copy()).cuda()
+        H.propagate_batch(c, torch.from_numpy(F).cuda(), B, dt, steps)
+        H.sync()
+    finally:
+        tdse_lib.set_device_memory_limit(0)
+    H.close()
+    for b in range(B):
+        ref, _ = oracle.rk4(lmax, n, E, U, C[b], F[b], dt, steps)
+        assert np.linalg.norm(c[b].cpu().numpy() - ref) < tol * np.linalg.norm(ref), b
