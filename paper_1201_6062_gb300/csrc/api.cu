@@ -99,6 +99,25 @@ struct DevBuf {
     template <class T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// Whether memory a call can do without (a second form of the dipole blocks for
+// a faster kernel) may be taken: at most an eighth of what the device and the
+// cap leave, so that allocations that are needed rarely meet it; one that does
+// gets it back (with_room).
+static bool optional_room(size_t nbytes)
+{
+    size_t free_b = 0, total = 0;
+    if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    const long long cap = g_dev_limit.load();
+    if (cap > 0) {
+        const long long left = cap - g_dev_bytes.load();
+        free_b = left < 0 ? 0 : std::min(free_b, (size_t)left);
+    }
+    return nbytes <= free_b / 8;
+}
+
 // Launch plan of the block mat-vec for one or several systems.
 struct MvPlan {
     tdse::MvCfg cfg{};
@@ -112,6 +131,8 @@ struct tdse_ctx {
     int lmax = 0, n = 0, N = 0, ld = 0, prec = 0;
     long long bstride = 0;
     DevBuf U, E, R, P, x, acc, xq, sb, sys, umax;
+    DevBuf Uf, ue;                     // FP64: fixed-point copy of U and its exponents (create_fixed)
+    bool in_group = false;             // a group's descriptors may point at them
     DevBuf part;                       // populations scratch
     DevBuf errw;                       // device status word (kErrTimeout, ...)
     DevBuf hc, hfield;                 // device copies for the host-buffer entry point
@@ -177,7 +198,8 @@ static int sm_count()
 
 // Build the mat-vec plan for the given systems and upload it.
 static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std::vector<int> &n, MvPlan &mp,
-                              tdse::Plan &plan, const std::vector<int> *global_id = nullptr, int layout = -1)
+                              tdse::Plan &plan, const std::vector<int> *global_id = nullptr, int layout = -1,
+                              bool fixed = false)
 {
     int nmax = 1;
     long long rows = 0, amps = 0;
@@ -196,8 +218,10 @@ static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std:
         // more CTAs only add column-partial slots and per-CTA overhead.
         long long ubytes = 0;
         for (size_t q = 0; q < n.size(); ++q) ubytes += (long long)lmax[q] * n[q] * n[q] * elem_bytes(prec);
+        const bool streamed = ubytes >= (64LL << 20);
         mp.cfg.per_sm = 1;
-        if (ubytes >= (64LL << 20)) {
+        if (fixed) (void)tdse::mvt_use_fixed(prec, nmax, streamed, &mp.cfg);
+        if (streamed) {
             // Rows per stage and resident CTAs trade against each other (a
             // deeper stage needs more registers, which can leave room for
             // fewer CTAs): take the depth with the most rows in flight per SM,
@@ -448,12 +472,63 @@ static tdse_status propagate_batch_tc(tdse_ctx *ctx, double *c, const double *fi
 // 3645 us float-float, 388 against 945 us FP32) but short rows with many
 // pulses, where most of a 128-row tile is padding (n=40, 200 pulses: 50
 // against 36 us; n=60: 45 against 48).  FP64 batches otherwise run pulse by
-// pulse: one stage of lmax=7, n=301 takes 29 us a pulse, 67 us for 2 and 70 us
-// for 4 pulses here.
+// pulse: a stage of lmax=7, n=301 takes 24 us a pulse and 70 us for 4 pulses
+// here, of lmax=15, n=1000 65 and 209 us; blocks streamed from HBM (32 bytes of
+// digits an element against 8) 335 and 1690 us at lmax=31, n=2000.  Without the
+// fixed-point copy a pulse takes 29, 152 and 1043 us.
 static bool dig_wanted(const tdse_ctx *ctx, int B)
 {
     if (ctx->lmax < 1) return false;
-    return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
+    if (ctx->prec != TDSE_FP64) return ctx->n >= 56 || B <= 32;
+    if (!ctx->Uf.p) return B >= 3;
+    return B >= ((long long)ctx->lmax * ctx->n * ctx->n * 8 >= (64LL << 20) ? 6 : 4);
+}
+
+// Fixed-point copy of an FP64 context's dipole blocks for the integer products
+// of the ring kernel (PolI64, 335 us a stage of lmax=31, n=2000 against the FP64
+// kernel's 1043).  Not made, and the FP64 kernel kept, for short rows (mv.cu), rows beyond the fixed-point layouts, blocks with a
+// non-finite element or a nonzero row or column whose largest element is below
+// 2^-6 of the block's (58 bits of the block's scale would leave it fewer than
+// 53 of its own), or when the memory for it cannot be had.
+static tdse_status create_fixed(tdse_ctx *c)
+{
+    const int n = c->n, lmax = c->lmax;
+    tdse::MvCfg cfg{};
+    if (!tdse::mvt_config(TDSE_FP64, n, c->ld, &cfg) || !tdse::mvt_use_fixed(TDSE_FP64, n, false, &cfg)) return TDSE_OK;
+    const size_t count = 2 * (size_t)lmax * n;
+    const size_t ubytes = (size_t)lmax * (size_t)c->bstride * 8;
+    if (!optional_room(ubytes)) return TDSE_OK;
+    if (c->ue.ensure(sizeof(int) * count) != cudaSuccess || c->Uf.ensure(ubytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        c->ue.release();
+        c->Uf.release();
+        return TDSE_OK;
+    }
+    CUDA_TRY(tdse::launch_fix_maxima(c->U.as<double>(), c->bstride, c->ld, n, lmax, c->ue.as<int>(), 0));
+    std::vector<int> h(count), e((size_t)lmax);
+    CUDA_TRY(cudaMemcpy(h.data(), c->ue.p, sizeof(int) * count, cudaMemcpyDeviceToHost));
+    bool ok = true;
+    for (int l = 0; l < lmax && ok; ++l) {
+        int m = 0;
+        for (int i = 0; i < n; ++i) m = std::max(m, h[(size_t)l * n + i]);
+        ok = m < 0x7ff00000;
+        for (int i = 0; i < n && ok; ++i)
+            for (int q = 0; q < 2; ++q) {
+                const int v = h[((size_t)q * lmax + l) * n + i];
+                ok = ok && (v == 0 || (v >> 20) >= (m >> 20) - 6);
+            }
+        e[(size_t)l] = std::max(m >> 20, 1) - 1022;
+    }
+    if (!ok) {
+        c->ue.release();
+        c->Uf.release();
+        return TDSE_OK;
+    }
+    CUDA_TRY(cudaMemcpy(c->ue.p, e.data(), sizeof(int) * e.size(), cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemset(c->Uf.p, 0, ubytes));
+    CUDA_TRY(tdse::launch_fix(c->U.as<double>(), c->bstride, (long long)n * c->ld, lmax, c->ue.as<int>(), c->Uf.p, 0));
+    CUDA_TRY(cudaDeviceSynchronize());
+    return TDSE_OK;
 }
 
 // Device storage, dipole digits and tensor maps of a digit-sliced batch; false
@@ -477,7 +552,7 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
               ctx->dgmax.ensure(sizeof(int) * 2 * 2 * (size_t)B * L) == cudaSuccess &&
               ctx->dgF.ensure(sizeof(double) * 3 * (size_t)B * nsteps) == cudaSuccess;
     if (ok && !ctx->dg_ready) {
-        ok = ctx->dgE.ensure(sizeof(int) * 2 * (size_t)ctx->lmax * n) == cudaSuccess &&
+        ok = optional_room(ub) && ctx->dgE.ensure(sizeof(int) * 2 * (size_t)ctx->lmax * n) == cudaSuccess &&
              ctx->dgU.ensure(ub) == cudaSuccess &&
              tdse::launch_dig_u(ctx->prec, ctx->U.p, ctx->bstride, ctx->ld, n, ctx->lmax, ldb, ctx->dgE.as<int>(),
                                 ctx->dgU.as<__nv_bfloat16>(), s) == cudaSuccess;
@@ -504,8 +579,64 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
         if (!ctx->dg_ready) { ctx->dgU.release(); ctx->dgE.release(); }
         ctx->dgX.release();
         ctx->dg_B = 0;
+        if (ctx->prec == TDSE_FP64) { ctx->bx.release(); ctx->bacc.release(); }      // (the pulse-by-pulse path has no use for them)
     }
     return ok;
+}
+
+// Work split, column-partial slots and slot starts of a context's own products.
+static tdse_status plan_context(tdse_ctx *c)
+{
+    tdse::Plan plan;
+    tdse_status st = build_plan(c->prec, std::vector<int>{c->lmax}, std::vector<int>{c->n}, c->plan, plan, nullptr, -1,
+                                c->Uf.p != nullptr);
+    if (st != TDSE_OK) return st;
+    c->nslots = plan.nslots[0];
+    CUDA_TRY(c->P.ensure(sizeof(double2) * (size_t)(c->nslots > 0 ? c->nslots : 1) * c->n));
+    CUDA_TRY(c->sb.ensure(sizeof(int) * (c->lmax + 1)));
+    CUDA_TRY(cudaMemcpy(c->sb.p, plan.sb[0].data(), sizeof(int) * (c->lmax + 1), cudaMemcpyHostToDevice));
+    c->step_ok = -1;
+    SysDesc &d = c->desc;
+    d.P = c->P.as<double2>();
+    d.sb = c->sb.as<int>();
+    d.Uf = c->Uf.p;
+    d.ue = c->ue.as<int>();
+    return TDSE_OK;
+}
+
+// Gives back the memory a context could do without (the fixed-point copy and
+// the digits of its dipole blocks, which the slower kernels do not need);
+// false if it holds none.
+static bool shed(tdse_ctx *c)
+{
+    const bool digits = c->dgU.p != nullptr, copy = c->Uf.p != nullptr && !c->in_group;
+    if (!digits && !copy) return false;
+    if (cudaDeviceSynchronize() != cudaSuccess) return false;
+    if (digits) {
+        c->dgU.release();
+        c->dgE.release();
+        c->dgX.release();
+        c->dg_ready = false;
+        c->dg_B = 0;
+    }
+    if (copy) {
+        c->Uf.release();
+        c->ue.release();
+        return plan_context(c) == TDSE_OK;
+    }
+    return true;
+}
+
+// A call that may allocate: once more without the optional memory when there
+// was not enough (allocations precede every write to the caller's data).
+template <class F> static tdse_status with_room(tdse_ctx *ctx, F call)
+{
+    tdse_status st = call();
+    if (st == TDSE_ENOMEM && ctx && shed(ctx)) {
+        (void)cudaGetLastError();
+        st = call();
+    }
+    return st;
 }
 
 static tdse_status propagate_batch_dig(tdse_ctx *ctx, double *c, const double *field, int B, int sps, double dt,
@@ -637,18 +768,29 @@ tdse_status tdse_create(const double *energies, const double *dipole_blocks, int
         CTRY(c->umax.ensure(sizeof(float) * um.size()));
         CTRY(cudaMemcpy(c->umax.p, um.data(), sizeof(float) * um.size(), cudaMemcpyHostToDevice));
     }
-    tdse::Plan plan;
-    st = build_plan(prec, std::vector<int>{lmax}, std::vector<int>{n}, c->plan, plan);
+    if (prec == TDSE_FP64 && lmax > 0) {
+        st = create_fixed(c);
+        if (st != TDSE_OK) return bail(st);
+    }
+    st = plan_context(c);
+    if (st == TDSE_ENOMEM && c->Uf.p) {
+        (void)cudaGetLastError();
+        c->Uf.release();
+        c->ue.release();
+        st = plan_context(c);
+    }
     if (st != TDSE_OK) return bail(st);
-    c->nslots = plan.nslots[0];
-    CTRY(c->R.ensure(sizeof(double2) * c->N));
+    const auto vectors = [c]() -> cudaError_t {
+        cudaError_t e = c->R.ensure(sizeof(double2) * c->N);
+        if (e == cudaSuccess) e = c->x.ensure(sizeof(double2) * c->N);
+        if (e == cudaSuccess) e = c->acc.ensure(sizeof(double2) * c->N);
+        if (e == cudaSuccess) e = c->xq.ensure((size_t)16 * c->N);
+        if (e == cudaSuccess) e = c->errw.ensure(sizeof(int));
+        return e == cudaSuccess ? c->sys.ensure(2 * sizeof(SysDesc)) : e;
+    };
+    if (vectors() == cudaErrorMemoryAllocation && c->Uf.p && !shed(c)) return bail(TDSE_ENOMEM);
+    CTRY(vectors());
     CTRY(cudaMemset(c->R.p, 0, sizeof(double2) * c->N));
-    CTRY(c->P.ensure(sizeof(double2) * (size_t)(c->nslots > 0 ? c->nslots : 1) * n));
-    CTRY(c->x.ensure(sizeof(double2) * c->N));
-    CTRY(c->acc.ensure(sizeof(double2) * c->N));
-    CTRY(c->xq.ensure((size_t)16 * c->N));
-    CTRY(c->sb.ensure(sizeof(int) * (lmax + 1)));
-    CTRY(cudaMemcpy(c->sb.p, plan.sb[0].data(), sizeof(int) * (lmax + 1), cudaMemcpyHostToDevice));
     CTRY(c->sys.ensure(2 * sizeof(SysDesc)));
     CTRY(c->errw.ensure(sizeof(int)));
     CTRY(cudaMemset(c->errw.p, 0, sizeof(int)));
@@ -657,7 +799,7 @@ tdse_status tdse_create(const double *energies, const double *dipole_blocks, int
 #undef CTRY
     SysDesc &d = c->desc;
     d.U = c->U.p; d.bstride = c->bstride; d.ld = c->ld; d.n = n; d.lmax = lmax; d.N = c->N;
-    d.E = c->E.as<double>(); d.R = c->R.as<double2>(); d.P = c->P.as<double2>(); d.sb = c->sb.as<int>();
+    d.E = c->E.as<double>(); d.R = c->R.as<double2>();
     d.umax = c->umax.as<float>();
     d.c = nullptr; d.x = c->x.as<double2>(); d.acc = c->acc.as<double2>(); d.xq = c->xq.p; d.field = nullptr;
     *out = c;
@@ -933,7 +1075,7 @@ static tdse_status propagate_impl(tdse_ctx *ctx, double *c, const double *field,
     return TDSE_OK;
 }
 
-tdse_status tdse_propagate(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt,
+static tdse_status propagate_once(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt,
                            long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
 {
     g_err.clear();
@@ -947,7 +1089,12 @@ tdse_status tdse_propagate(tdse_ctx *ctx, double *c, const double *field, int sa
                           (cudaStream_t)stream);
 }
 
-tdse_status tdse_propagate_rkf45(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1,
+tdse_status tdse_propagate(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+{
+    return with_room(ctx, [&] { return propagate_once(ctx, c, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
+}
+
+static tdse_status propagate_rkf45_once(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1,
                                  double dt0, double tol, double dt_min, double dt_max, long max_attempts,
                                  tdse_rkf_stats *stats, void *stream)
 {
@@ -1041,7 +1188,12 @@ tdse_status tdse_propagate_rkf45(tdse_ctx *ctx, double *c, const tdse_field_fn *
     return TDSE_OK;
 }
 
-tdse_status tdse_propagate_host(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step,
+tdse_status tdse_propagate_rkf45(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1, double dt0, double tol, double dt_min, double dt_max, long max_attempts, tdse_rkf_stats *stats, void *stream)
+{
+    return with_room(ctx, [&] { return propagate_rkf45_once(ctx, c, field, t0, t1, dt0, tol, dt_min, dt_max, max_attempts, stats, stream); });
+}
+
+static tdse_status propagate_host_once(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step,
                                 double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
                                 void *stream)
 {
@@ -1067,6 +1219,11 @@ tdse_status tdse_propagate_host(tdse_ctx *ctx, double *c_host, const double *fie
     if (st != TDSE_OK) return st;
     CUDA_TRY(cudaMemcpyAsync(c_host, ctx->hc.p, cb, cudaMemcpyDeviceToHost, s));
     return tdse_sync(ctx, stream);
+}
+
+tdse_status tdse_propagate_host(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+{
+    return with_room(ctx, [&] { return propagate_host_once(ctx, c_host, field_host, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
 }
 
 tdse_status tdse_set_gauge(tdse_ctx *ctx, tdse_gauge gauge)
@@ -1276,7 +1433,7 @@ static tdse_status propagate_batch_df(tdse_ctx *ctx, double *c, const double *fi
     return TDSE_OK;
 }
 
-tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step,
+static tdse_status propagate_batch_once(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step,
                                  double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
                                  void *stream)
 {
@@ -1355,6 +1512,11 @@ tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, 
     return TDSE_OK;
 }
 
+tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+{
+    return with_room(ctx, [&] { return propagate_batch_once(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
+}
+
 // Field samples that a stage's field value depends on, with weights
 // (reading of the field samples: linear mean at half steps on the step grid).
 static void field_deps(int sps, long k, int h, long long *i0, long long *i1, double *w0, double *w1)
@@ -1368,7 +1530,7 @@ static void field_deps(int sps, long k, int h, long long *i0, long long *i1, dou
     *i0 = k; *i1 = k + 1; *w0 = 0.5; *w1 = 0.5;
 }
 
-tdse_status tdse_adjoint(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt,
+static tdse_status adjoint_once(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt,
                          long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, const double *weights,
                          int checkpoint_every, double *grad_field, double *c_final, double *loss, void *stream)
 {
@@ -1555,6 +1717,11 @@ tdse_status tdse_adjoint(tdse_ctx *ctx, const double *c0, const double *field, i
     return TDSE_OK;
 }
 
+tdse_status tdse_adjoint(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, const double *weights, int checkpoint_every, double *grad_field, double *c_final, double *loss, void *stream)
+{
+    return with_room(ctx, [&] { return adjoint_once(ctx, c0, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, weights, checkpoint_every, grad_field, c_final, loss, stream); });
+}
+
 // Systems whose rows take the same thread layout share one product launch.
 struct GroupBucket {
     std::vector<int> members;           // system indices in the group
@@ -1610,7 +1777,9 @@ static tdse_status bucket_plan(tdse_group *g, GroupBucket &bk)
     std::vector<int> blm, bnn;
     for (int i : bk.members) { blm.push_back(g->sys[i]->lmax); bnn.push_back(g->sys[i]->n); }
     tdse::Plan plan;
-    tdse_status st = build_plan(g->prec, blm, bnn, bk.plan, plan, &bk.members, bk.layout);
+    bool fixed = true;
+    for (int i : bk.members) fixed = fixed && g->sys[i]->Uf.p != nullptr;
+    tdse_status st = build_plan(g->prec, blm, bnn, bk.plan, plan, &bk.members, bk.layout, fixed);
     if (st != TDSE_OK) return st;
     for (size_t k = 0; k < bk.members.size(); ++k) {
         const int i = bk.members[k];
@@ -1640,7 +1809,9 @@ static tdse_status group_persistent_plan(tdse_group *g)
     std::vector<int> lm(count), nn(count), ids(count);
     for (int i = 0; i < count; ++i) { lm[i] = g->sys[i]->lmax; nn[i] = g->sys[i]->n; ids[i] = i; }
     tdse::Plan plan;
-    tdse_status st = build_plan(g->prec, lm, nn, g->pplan, plan, &ids, g->playout);
+    bool fixed = true;
+    for (int i = 0; i < count; ++i) fixed = fixed && g->sys[i]->Uf.p != nullptr;
+    tdse_status st = build_plan(g->prec, lm, nn, g->pplan, plan, &ids, g->playout, fixed);
     if (st != TDSE_OK) return st;
     if (!g->pplan.cfg.tma || g->pplan.grid <= 0)
         return fail(TDSE_ENOTSUP, "one launch for the group needs rows long enough for the bulk-copy ring");
@@ -1694,6 +1865,7 @@ tdse_status tdse_group_create(tdse_ctx *const *systems, int count, tdse_group **
     auto bail = [&](tdse_status st) { delete g; return st; };
     g->sys.assign(systems, systems + count);
     g->prec = systems[0]->prec;
+    for (int i = 0; i < count; ++i) systems[i]->in_group = true;
     std::vector<int> lm(count), nn(count);
     for (int i = 0; i < count; ++i) { lm[i] = systems[i]->lmax; nn[i] = systems[i]->n; }
     // The epilogue and prep block map over all systems (its product plan is not used).
