@@ -247,9 +247,9 @@ static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std:
     // (its x_{l+1} columns, the |x| bounds of the offset sums, one more
     // partial slot to write): measured at about 8 rows of a float-float
     // product with 500-element rows (FP32 products, with the same offset
-    // sums, are charged alike) and 1 row of an FP64 one.  Charged only when
-    // CTAs get enough rows for it to matter.
-    const int seg_rows = rows >= 16LL * G ? (prec == TDSE_FP64 ? 1 : 8) : 0;
+    // sums, are charged alike), 1 row of an FP64 one and 6 rows of a
+    // fixed-point one.  Charged only when CTAs get enough rows for it to matter.
+    const int seg_rows = mp.cfg.fix ? (rows >= 8LL * G ? 6 : 0) : rows >= 16LL * G ? (prec == TDSE_FP64 ? 1 : 8) : 0;
     tdse::make_plan(G, lmax, n, 32, plan, seg_rows);
     mp.grid = rows > 0 ? G : 0;
     std::vector<Seg> segs(plan.segs.size());
@@ -485,9 +485,9 @@ static bool dig_wanted(const tdse_ctx *ctx, int B)
 }
 
 // Fixed-point copy of an FP64 context's dipole blocks for the integer products
-// of the ring kernel (PolI64, 335 us a stage of lmax=31, n=2000 against the FP64
-// kernel's 1043).  Not made, and the FP64 kernel kept, for short rows (mv.cu), rows beyond the fixed-point layouts, blocks with a
-// non-finite element or a nonzero row or column whose largest element is below
+// of the ring kernel (PolI64, 305 us a stage of lmax=31, n=2000 against the FP64
+// kernel's 1043).  Not made, and the FP64 kernel kept, for short rows (mv.cu),
+// rows beyond the fixed-point layouts, blocks with a non-finite element or a nonzero row or column whose largest element is below
 // 2^-6 of the block's (58 bits of the block's scale would leave it fewer than
 // 53 of its own), or when the memory for it cannot be had.
 static tdse_status create_fixed(tdse_ctx *c)

@@ -175,6 +175,11 @@ struct PolF64 {
     {
         reinterpret_cast<double2 *>(xq)[a] = v;
     }
+    // one component (0 real, 1 imaginary)
+    static __device__ __forceinline__ void store_xq1(void *xq, long long a, int comp, double v)
+    {
+        reinterpret_cast<double *>(xq)[2 * a + comp] = v;
+    }
 };
 
 // FP32 products: U stored as float, 4 columns per 16-byte load.
@@ -246,6 +251,11 @@ struct PolF32 {
     static __device__ __forceinline__ void store_xq(void *xq, long long a, double2 v)
     {
         reinterpret_cast<float4 *>(xq)[a] = make_float4(__double2float_rn(v.x), __double2float_rn(v.y), 0.f, 0.f);
+    }
+    static __device__ __forceinline__ void store_xq1(void *xq, long long a, int comp, double v)
+    {
+        reinterpret_cast<float *>(xq)[4 * a + comp] = __double2float_rn(v);
+        reinterpret_cast<float *>(xq)[4 * a + 2 + comp] = 0.f;
     }
 };
 
@@ -369,6 +379,11 @@ struct PolDF32 {
         df r = df_from_double(v.x), i = df_from_double(v.y);
         reinterpret_cast<float4 *>(xq)[a] = make_float4(r.h, r.l, i.h, i.l);
     }
+    static __device__ __forceinline__ void store_xq1(void *xq, long long a, int comp, double v)
+    {
+        const df r = df_from_double(v);
+        reinterpret_cast<float2 *>(xq)[2 * a + comp] = make_float2(r.h, r.l);
+    }
 };
 
 // FP64-accurate products in integer arithmetic, for the ring kernel.
@@ -388,8 +403,8 @@ struct PolDF32 {
 // Taken for blocks whose rows and columns all reach 2^-6 of the block's
 // largest element (create_fixed in api.cu), so that each output keeps this
 // relative to its own row or column.
-// Measured, one product and its update: lmax=31, n=2000 1043 -> 335 us, lmax=15,
-// n=500 47.6 -> 30.8 us a stage; error of a product against extended precision
+// Measured, one product and its update: lmax=31, n=2000 1043 -> 305 us, lmax=15,
+// n=500 47.6 -> 23.4 us a stage; error of a product against extended precision
 // 3.0e-16 (FP64 kernel 3.35e-16, n=2000).  Bound by the multiply pipe (60%
 // active: 12 wide multiply-adds an element) and the issue slots of the sums.
 struct PolI64 {
@@ -410,10 +425,10 @@ struct PolI64 {
         const int E = (int)((bits >> 52) & 0x7ff);
         unsigned long long m = (unsigned long long)bits & 0xfffffffffffffULL;
         if (E) m |= 1ULL << 52;
-        const int sh = max(E, 1) - 1075 + BITS - e;          // at most 5
-        if (sh >= 0) m <<= (sh & 7);
-        else if (sh > -63) m = (m + (1ULL << (-sh - 1))) >> -sh;
-        else m = 0;
+        // |v| = m 2^(max(E,1) - 1075) < 2^e: one bit more than the result holds, then round
+        const int d = e - (max(E, 1) - 1022);                // >= 0
+        m = (m << 6) >> min(d, 63);
+        m = (m + 1) >> 1;
         const long long q = bits < 0 ? -(long long)m : (long long)m;
         const int hi = (int)((q + (1LL << (LOW - 1))) >> LOW);
         return make_int2((int)(q - ((long long)hi << LOW)), hi);
@@ -489,26 +504,54 @@ struct PolI64 {
     {
         return ex >= kNonfinite ? kNonfinite : ue + ex - 2 * BITS + LOW + 5;
     }
-    static __device__ __forceinline__ double scaled(double v, Sigma s)
+    // (w2 w1 w0) 2^s rounded to nearest, from the bits: a conversion or an
+    // addition in FP64 holds the FP64 pipe for 19 cycles a warp instruction, and
+    // a segment's end took 5200 cycles of them (n = 500).
+    static __device__ __forceinline__ double to_f64(CRun a, Sigma s)
     {
         if (s >= kNonfinite) return __longlong_as_double(0x7ff8000000000000LL);
-        if (s > -900 && s < 900) return v * __hiloint2double((s + 1023) << 20, 0);
-        return scalbn(v, s);
+        const unsigned neg = (unsigned)(a.w2 >> 31);                     // all ones if negative
+        unsigned h = (unsigned)a.w2, m = a.w1, l = a.w0;
+        if (neg) {
+            l = ~l + 1u;
+            m = ~m + (l == 0u);
+            h = ~h + (l == 0u && m == 0u);
+        }
+        if ((h | m | l) == 0u) return 0.0;
+        int e = 95;
+        if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
+        if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
+        const int z = __clz((int)h);
+        h = __funnelshift_l(m, h, z);
+        m = __funnelshift_l(l, m, z);
+        l <<= z;
+        e -= z;                                                          // value = 1.x 2^e, leading bit at the top of h
+        // 53 bits, round to nearest (ties up: below half a unit of the sum's own truncation)
+        unsigned long long r = ((unsigned long long)h << 32) | m;
+        r = (r >> 11) + ((r >> 10) & 1u);
+        e += s;
+        if (e > -1000 && e < 1000)
+            // (the leading bit of r adds 1 to the exponent field)
+            return __longlong_as_double((long long)((r + ((unsigned long long)(e + 1022) << 52)) |
+                                                    ((unsigned long long)(neg & 0x80000000u) << 32)));
+        const double v = scalbn((double)r, e - 52);
+        return neg ? -v : v;
     }
-    static __device__ __forceinline__ double cto_double(CRun a, Sigma s)
-    {
-        const long long top = ((long long)a.w2 << 32) | a.w1;
-        return scaled((double)top * 0x1p32 + (double)a.w0, s);
-    }
+    static __device__ __forceinline__ double cto_double(CRun a, Sigma s) { return to_f64(a, s); }
     // sums of up to 16 warps' parts
     static __device__ __forceinline__ double parts_to_double(const long long p[4], Sigma s)
     {
-        const long long lo = p[0] + (p[1] << 24), hi = p[2] + (p[3] << 24);
-        return scaled((double)hi * 0x1p48 + (double)lo, s);
+        const long long lo = p[0] + (p[1] << 24), hi = p[2] + (p[3] << 24);          // lo + hi 2^48
+        CRun r{(unsigned)lo, (unsigned)(lo >> 32), (int)(lo >> 63)};
+        return to_f64(cadd(r, CRun{0u, (unsigned)hi << 16, (int)(hi >> 16)}), s);
     }
     static __device__ __forceinline__ void store_xq(void *xq, long long a, double2 v)      // as PolF64
     {
         reinterpret_cast<double2 *>(xq)[a] = v;
+    }
+    static __device__ __forceinline__ void store_xq1(void *xq, long long a, int comp, double v)
+    {
+        reinterpret_cast<double *>(xq)[2 * a + comp] = v;
     }
 };
 

@@ -1,7 +1,7 @@
-// Per-amplitude epilogue of one stage (paper Sec. 4: H x = E x + f D x with
-// D x assembled from the row sums R and the column-partial slots P; App. B:
-// the RK4 stage and Taylor term combinations), all in FP64.  Used by the
-// epilogue kernel that follows each block product.
+// Update of one stage (paper Sec. 4: H x = E x + f D x with D x assembled from
+// the row sums R and the column-partial slots P; App. B: the RK4 stage and
+// Taylor term combinations), all in FP64.  Used by the update kernel that
+// follows each block product and by the persistent stepping kernel.
 #pragma once
 #include "kernels.h"
 
@@ -18,107 +18,156 @@ struct EpiPre {
 __device__ __forceinline__ EpiPre epi_pre(const SysDesc &S, long long a)
 {
     EpiPre p;
-    p.m = (int)(a / S.n);
-    p.i = (int)(a - (long long)p.m * S.n);
+    p.m = (int)((unsigned)a / (unsigned)S.n);                // (a < 2^31)
+    p.i = (int)a - p.m * S.n;
     p.e = S.E[a];
     p.b0 = p.m >= 1 ? S.sb[p.m - 1] : 0;
     p.b1 = p.m >= 1 ? S.sb[p.m] : 0;
     return p;
 }
 
-// D x at amplitude a: the row sum (blocks below lmax) plus the column
-// partials of block m-1 in slot order; velocity gauge D x = i (R - sum P).
-// kCG: read through L2 only (in a persistent launch other CTAs wrote R and P
-// moments ago); a separate update launch reads them plainly, which lets the
-// compiler batch the loads (3% of an FP32 step).
-template <bool kCG = false>
-__device__ __forceinline__ double2 epi_dx(const SysDesc &S, long long a, const EpiPre &p)
+// The update in halves: a thread assembles one component (own) of D x, and
+// with it h = E x + f D x, whose k = -i h is the other component's derivative,
+// so it updates that one (tgt) and no values are exchanged.  Twice the threads,
+// half the dependent FP64 instructions of each; KIND is a template parameter
+// because the compiler evaluates short alternatives of a uniform branch side by
+// side and every FP64 instruction takes 64 cycles of its scheduler.  Bound by the
+// latency of those instructions and of the loads: a stage of the persistent
+// kernel 21.0 -> 18.7 us float-float and 30.9 -> 23.5 us FP64 at lmax=15, n=500,
+// 24.2 -> 16.9 us FP64 at lmax=7, n=301 (from one thread an amplitude).
+enum EpiKind { EK_RK4_FIRST, EK_RK4_MID, EK_RK4_LAST, EK_TAYLOR, EK_HX, EK_MIHX };
+
+struct EpiHalf {
+    double f, s;           // field value; RK4: a_{s+1} dt (last stage dt/6), Taylor: dt/m
+    bool first, last;      // Taylor: first and last term
+    double2 *st_x, *st_c;  // as EpiArgs
+};
+
+// One component of D x at (m, i): row sum plus column partials in slot order,
+// read eight at a time (velocity gauge D x = i (R - sum P)).  kCG: through L2
+// only (in a persistent launch other CTAs wrote R and P moments ago).
+template <bool kCG>
+__device__ __forceinline__ double dx_comp(const SysDesc &S, long long a, const EpiPre &pre, int own)
 {
-    double rr = 0.0, ri = 0.0, pr = 0.0, pi = 0.0;
-    if (p.m < S.lmax) {
-        const double2 r = kCG ? __ldcg(S.R + a) : S.R[a];
-        rr = r.x; ri = r.y;
+    const int src = S.gauge ? own ^ 1 : own;
+    const double *R = reinterpret_cast<const double *>(S.R) + 2 * a + src;
+    const double *Pp = reinterpret_cast<const double *>(S.P) + 2 * ((long long)pre.b0 * S.n + pre.i) + src;
+    const long long step = 2LL * S.n;
+    auto ld = [](const double *p) { return kCG ? __ldcg(p) : *p; };
+    const double r = pre.m < S.lmax ? ld(R) : 0.0;
+    double p = 0.0;
+    for (int s = pre.b0; s < pre.b1; s += 8, Pp += 8 * step) {
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = s + j < pre.b1 ? ld(Pp + j * step) : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (s + j < pre.b1) p += v[j];
     }
-    for (int s = p.b0; s < p.b1; ++s) {
-        const double2 q = kCG ? __ldcg(S.P + (long long)s * S.n + p.i) : S.P[(long long)s * S.n + p.i];
-        pr += q.x; pi += q.y;
-    }
-    if (S.gauge == 0) return make_double2(rr + pr, ri + pi);
-    return make_double2(-(ri - pi), rr - pr);
+    if (S.gauge == 0) return r + p;
+    return own == 0 ? -(r - p) : r - p;
 }
 
-template <class P, bool kCG = false>
-__device__ __forceinline__ void epi_amp(const SysDesc &S, long long a, const EpiArgs &A, const EpiPre &pre)
+// What an update reads besides D x (nothing that other threads' updates of
+// the same stage write, but for the other component's lane).
+struct EpiIn {
+    EpiPre pre;
+    double xo, ct, at;     // own component of the stage input; the other one's state and accumulator
+};
+
+template <int KIND>
+__device__ __forceinline__ EpiIn epi_load(const SysDesc &S, long long a, int own, bool live, const EpiHalf &A)
 {
-    const double2 dx = epi_dx<kCG>(S, a, pre);
-    const double dr = dx.x, di = dx.y;
-    const double e = pre.e;
-    double f;
-    double2 xin;
-    if (A.mode == EPI_RK4) {
-        const int h = (A.stage == 0) ? 0 : (A.stage == 3 ? 2 : 1);
-        f = field_at(S.field, A.sps, A.k, h);
-        xin = (A.stage == 0) ? S.c[a] : S.x[a];
-    } else if (A.mode == EPI_TAYLOR) {
-        f = field_at(S.field, A.sps, A.k, A.hold ? 1 : 0);
-        xin = (A.stage == 1) ? S.c[a] : S.x[a];
-    } else {
-        f = A.fval;
-        xin = S.x[a];
+    const int tgt = own ^ 1;
+    const double *c = reinterpret_cast<const double *>(S.c) + 2 * a, *x = reinterpret_cast<const double *>(S.x) + 2 * a;
+    constexpr bool kRk = KIND == EK_RK4_FIRST || KIND == EK_RK4_MID || KIND == EK_RK4_LAST;
+    const bool from_c = KIND == EK_RK4_FIRST || (KIND == EK_TAYLOR && A.first);
+    EpiIn in{};
+    if (live) {
+        in.pre = epi_pre(S, a);
+        in.xo = from_c ? c[own] : x[own];
+        if (kRk || from_c) in.ct = c[tgt];
+        if (KIND == EK_RK4_MID || KIND == EK_RK4_LAST || (KIND == EK_TAYLOR && !A.first))
+            in.at = reinterpret_cast<const double *>(S.acc)[2 * a + tgt];
     }
-    const double hr = e * xin.x + f * dr;
-    const double hi = e * xin.y + f * di;
-    // k = -i (hr + i hi)
-    const double kr = hi, ki = -hr;
-    if (A.mode == EPI_HX) { S.acc[a] = make_double2(hr, hi); return; }
-    if (A.mode == EPI_MIHX) { S.acc[a] = make_double2(kr, ki); return; }
-    if (A.mode == EPI_RK4) {
-        const double2 c = S.c[a];
-        const double dt = A.dt;
-        if (A.stage == 0) {
-            S.acc[a] = make_double2(kr, ki);
-            const double2 xn = make_double2(c.x + 0.5 * dt * kr, c.y + 0.5 * dt * ki);
-            S.x[a] = xn;
-            P::store_xq(S.xq, a, xn);
-            if (A.st_x) A.st_x[a] = xn;
-        } else if (A.stage < 3) {
-            const double2 ac = S.acc[a];
-            S.acc[a] = make_double2(ac.x + 2.0 * kr, ac.y + 2.0 * ki);
-            const double s = (A.stage == 1) ? 0.5 * dt : dt;
-            const double2 xn = make_double2(c.x + s * kr, c.y + s * ki);
-            S.x[a] = xn;
-            P::store_xq(S.xq, a, xn);
-            if (A.st_x) A.st_x[a] = xn;
-        } else {
-            const double2 ac = S.acc[a];
-            const double w = dt / 6.0;
-            const double2 cn = make_double2(c.x + w * (ac.x + kr), c.y + w * (ac.y + ki));
-            S.c[a] = cn;
-            P::store_xq(S.xq, a, cn);
-            if (A.st_c) A.st_c[a] = cn;
-        }
+    return in;
+}
+
+// Called by whole warps, the two components of an amplitude on adjacent lanes;
+// live: whether this lane has one.
+template <class P, int KIND, bool kCG>
+__device__ __forceinline__ void epi_half(const SysDesc &S, long long a, int own, bool live, const EpiIn &in, const EpiHalf &A)
+{
+    const int tgt = own ^ 1;
+    double *c = reinterpret_cast<double *>(S.c) + 2 * a, *x = reinterpret_cast<double *>(S.x) + 2 * a;
+    double *acc = reinterpret_cast<double *>(S.acc) + 2 * a;
+    const double h = live ? in.pre.e * in.xo + A.f * dx_comp<kCG>(S, a, in.pre, own) : 0.0;
+    __syncwarp();                          // both components are read before either is written
+    if (!live) return;
+    if constexpr (KIND == EK_HX) {
+        acc[own] = h;
         return;
     }
-    // Taylor term m = A.stage: T_m = (dt/m) k; sum += T_m.
-    const double s = A.dt / (double)A.stage;
-    const double2 T = make_double2(s * kr, s * ki);
-    double2 sum;
-    if (A.stage == 1) {
-        sum = make_double2(xin.x + T.x, xin.y + T.y);
+    const double k = own ? h : -h;         // (k_re, k_im) = (h_im, -h_re)
+    if constexpr (KIND == EK_MIHX) {
+        acc[tgt] = k;
+    } else if constexpr (KIND == EK_RK4_FIRST || KIND == EK_RK4_MID) {
+        acc[tgt] = KIND == EK_RK4_FIRST ? k : in.at + 2.0 * k;
+        const double xn = in.ct + A.s * k;
+        x[tgt] = xn;
+        P::store_xq1(S.xq, a, tgt, xn);
+        if (A.st_x) reinterpret_cast<double *>(A.st_x)[2 * a + tgt] = xn;
+    } else if constexpr (KIND == EK_RK4_LAST) {
+        const double cn = in.ct + A.s * (in.at + k);
+        c[tgt] = cn;
+        P::store_xq1(S.xq, a, tgt, cn);
+        if (A.st_c) reinterpret_cast<double *>(A.st_c)[2 * a + tgt] = cn;
     } else {
-        const double2 ac = S.acc[a];
-        sum = make_double2(ac.x + T.x, ac.y + T.y);
+        const double T = A.s * k;
+        const double sum = (A.first ? in.ct : in.at) + T;
+        const double xn = A.last ? sum : T;
+        if (A.last) {
+            c[tgt] = sum;
+        } else {
+            acc[tgt] = sum;
+            x[tgt] = T;
+        }
+        P::store_xq1(S.xq, a, tgt, xn);
+        double2 *st = A.last ? A.st_c : A.st_x;
+        if (st) reinterpret_cast<double *>(st)[2 * a + tgt] = xn;
     }
-    if (A.stage < A.order) {
-        S.acc[a] = sum;
-        S.x[a] = T;
-        P::store_xq(S.xq, a, T);
-        if (A.st_x) A.st_x[a] = T;
-    } else {
-        S.c[a] = sum;
-        P::store_xq(S.xq, a, sum);
-        if (A.st_c) A.st_c[a] = sum;
+}
+
+// The amplitudes [a0, a1) of S by the nthr threads of whole warps (tid: this
+// thread's number), two threads each.  ready() is called once the first
+// amplitudes' own data are requested, before any of D x is read (false: give
+// up); later ones' are requested an iteration ahead.
+template <class P, int KIND, bool kCG, class Ready>
+__device__ __forceinline__ bool epi_span_kind(const SysDesc &S, long long a0, long long a1, int tid, int nthr, const EpiHalf &A, Ready ready)
+{
+    const int own = tid & 1;
+    long long a = a0 + tid / 2;
+    EpiIn in = epi_load<KIND>(S, a, own, a < a1, A);
+    if (!ready()) return false;
+#pragma unroll 1
+    for (long long b = a0; b < a1; b += nthr / 2, a += nthr / 2) {
+        const long long an = a + nthr / 2;
+        const EpiIn nx = epi_load<KIND>(S, an, own, an < a1, A);
+        epi_half<P, KIND, kCG>(S, a, own, a < a1, in, A);
+        in = nx;
     }
+    return true;
+}
+
+template <class P, bool kCG, class Ready>
+__device__ __forceinline__ bool epi_span(const SysDesc &S, long long a0, long long a1, int tid, int nthr, int kind, const EpiHalf &A, Ready ready)
+{
+    switch (kind) {
+    case EK_RK4_FIRST: return epi_span_kind<P, EK_RK4_FIRST, kCG>(S, a0, a1, tid, nthr, A, ready);
+    case EK_RK4_MID: return epi_span_kind<P, EK_RK4_MID, kCG>(S, a0, a1, tid, nthr, A, ready);
+    case EK_RK4_LAST: return epi_span_kind<P, EK_RK4_LAST, kCG>(S, a0, a1, tid, nthr, A, ready);
+    }
+    return epi_span_kind<P, EK_TAYLOR, kCG>(S, a0, a1, tid, nthr, A, ready);
 }
 
 }  // namespace tdse

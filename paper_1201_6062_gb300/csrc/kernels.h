@@ -70,6 +70,7 @@ struct StepArgs {
     int mode;              // EPI_RK4 or EPI_TAYLOR
     int order, hold, sps;  // Taylor order and hold, samples per step
     double dt;
+    double coef[65];       // dt / m (m >= 1), set by launch_mvt_step
     long long k0;          // step index of the first pass (a pass is one stage)
     unsigned *gbar;        // grid-barrier arrival counter, zero at launch
     // Adjoint forward pass: after step k, if (k+1) % ckpt_every == 0 and
@@ -124,6 +125,7 @@ struct EpiArgs {
     long long k;    // step index
     double dt;
     double fval;    // field for EPI_HX / EPI_MIHX
+    double s;       // set by launch_epi: RK4 a_{s+1} dt (last stage dt/6), Taylor dt/m
     double2 *st_x;  // if set: also store this stage's new x (next stage input / Taylor term)
     double2 *st_c;  // if set: also store the new c (last RK4 stage / last Taylor term)
     const long long *kdev;   // if set: the step index is *kdev (captured step graphs)

@@ -264,7 +264,7 @@ cudaError_t launch_mv(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, 
 // partial slots of block m-1 (m >= 1), in slot order;  then H x = E x + f D x
 // and the stage / term update of the chosen scheme, all in FP64.
 template <class P>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(512)
 epi_kernel(const SysDesc *__restrict__ sys, const int2 *__restrict__ blk, EpiArgs A)
 {
     pdl_launch_dependents();
@@ -272,13 +272,39 @@ epi_kernel(const SysDesc *__restrict__ sys, const int2 *__restrict__ blk, EpiArg
     // for every launch of a call: read them before waiting for the product.
     const int2 bm = blk[blockIdx.x];
     const SysDesc S = sys[bm.x];
-    const long long a = (long long)bm.y + threadIdx.x;
+    const long long a = (long long)bm.y + (threadIdx.x >> 1);
+    const int own = threadIdx.x & 1;
     const bool live = a < S.N;
     const EpiPre pre = live ? epi_pre(S, a) : EpiPre{};
     pdl_wait();
-    if (!live) return;
-    if (A.kdev) A.k = *A.kdev;
-    epi_amp<P>(S, a, A, pre);
+    EpiHalf h{};
+    h.s = A.s;
+    h.st_x = A.st_x;
+    h.st_c = A.st_c;
+    h.first = A.stage == 1;
+    h.last = A.stage == A.order;
+    auto run = [&](auto kc) {
+        constexpr int KIND = decltype(kc)::value;
+        EpiIn in = epi_load<KIND>(S, a, own, live, h);
+        in.pre = pre;
+        epi_half<P, KIND, false>(S, a, own, live, in, h);
+    };
+    if (A.mode == EPI_HX || A.mode == EPI_MIHX) {
+        h.f = A.fval;
+        if (A.mode == EPI_HX) run(std::integral_constant<int, EK_HX>{});
+        else run(std::integral_constant<int, EK_MIHX>{});
+        return;
+    }
+    const long long k = A.kdev ? *A.kdev : A.k;
+    if (A.mode == EPI_TAYLOR) {
+        h.f = field_at(S.field, A.sps, k, A.hold ? 1 : 0);
+        run(std::integral_constant<int, EK_TAYLOR>{});
+        return;
+    }
+    h.f = field_at(S.field, A.sps, k, A.stage == 0 ? 0 : (A.stage == 3 ? 2 : 1));
+    if (A.stage == 0) run(std::integral_constant<int, EK_RK4_FIRST>{});
+    else if (A.stage < 3) run(std::integral_constant<int, EK_RK4_MID>{});
+    else run(std::integral_constant<int, EK_RK4_LAST>{});
 }
 
 template <class P>
@@ -334,8 +360,10 @@ cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, 
     case 2: fn = (const void *)epi_kernel<PolDF32>; break;
     default: return cudaErrorInvalidValue;
     }
+    if (a.mode == EPI_RK4) a.s = a.stage == 3 ? a.dt / 6.0 : (a.stage == 2 ? a.dt : 0.5 * a.dt);
+    else if (a.mode == EPI_TAYLOR) a.s = a.dt / (double)a.stage;
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&a};
-    return launch_pdl(fn, dim3(nblk), dim3(256), 0, stream, args);
+    return launch_pdl(fn, dim3(nblk), dim3(512), 0, stream, args);       // two threads per amplitude, 256 per block
 }
 
 __global__ void bump_kernel(long long *kdev) { *kdev += 1; }

@@ -159,6 +159,7 @@ cudaError_t launch_mvt_step(int prec, const MvCfg &cfg, int grid, const SysDesc 
     const cudaError_t z = cudaMemsetAsync(a.gbar, 0, sizeof(unsigned), stream);
     if (z != cudaSuccess) return z;
     StepArgs sa = a;
+    for (int m = 1; m < 65; ++m) sa.coef[m] = a.dt / (double)m;
     void *args[] = {(void *)&sys, (void *)&segs, (void *)&cta_off, (void *)&err, (void *)&stage, (void *)&sa};
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(grid);

@@ -82,6 +82,155 @@ __device__ __forceinline__ bool grid_sync(unsigned *ctr, unsigned target, volati
     return *go != 0;
 }
 
+// A grid barrier to pass on to the stage update.
+struct GridBar {
+    unsigned *ctr;
+    unsigned target;
+    volatile int *abort;
+    int *err;
+    volatile int *go;
+    int tid, nthreads;
+    __device__ __forceinline__ bool operator()() const { return grid_sync(ctr, target, abort, err, go, tid, nthreads); }
+};
+struct NoBar {
+    __device__ __forceinline__ bool operator()() const { return true; }
+};
+
+// What follows a pass's block products in a stepping launch: a grid barrier
+// (every row sum and column partial is written), the stage update of this
+// CTA's slice [u0, u1) of amplitudes, whose own data are requested before the barrier,
+// and a second barrier (every input of the next pass is written); false: this
+// CTA or another one has given up.
+template <class P, int CTT>
+__device__ __forceinline__ bool step_update_inline(const SysDesc *sys, const StepArgs &A, int pass, volatile int *abort, int *err,
+                                         volatile int *go_flag, double *dot_sh, long long u0, long long u1)
+{
+    constexpr int NWT = CTT / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const GridBar written{A.gbar, (unsigned)(2 * pass + 1) * gridDim.x, abort, err, go_flag, tid, CTT};
+    const GridBar updated{A.gbar, (unsigned)(2 * pass + 2) * gridDim.x, abort, err, go_flag, tid, CTT};
+    const SysDesc &S0 = sys[0];
+    const int per = A.mode == EPI_RK4 ? 4 : A.order;
+    if (A.reverse) {
+        // reverse stage q of step k0+i (the segment's last step first)
+        const int i = A.ns - 1 - pass / per;
+        const int q = A.mode == EPI_RK4 ? 3 - pass % per : A.order - pass % per;
+        const int fq = A.mode == EPI_RK4 ? q : q - 1;
+        const SysDesc &Sa = sys[0];
+        const long long Na = Sa.N;
+        const int h = A.mode == EPI_RK4 ? (q == 0 ? 0 : (q == 3 ? 2 : 1)) : (A.hold ? 1 : 0);
+        AdjHalf aa{};
+        aa.f = field_at(Sa.field, A.sps, A.k0 + i, h);
+        aa.fwd = (fq == 0 && i == 0) ? A.ckpt0 : A.store + (size_t)((long long)i * A.nst + fq) * Na;
+        aa.G = A.G;
+        double dot = 0.0;
+        bool go;
+        if (A.mode != EPI_RK4) {
+            // term m: (dt/(m-1)) Gamma_{m-1}, or at m = 1 the previous step's (dt/K) G
+            aa.to_G = q == 1;
+            aa.cg = A.coef[q > 1 ? q - 1 : A.order];
+            go = adj_span<P, AK_TAYLOR, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+        } else if (q == 3) {
+            aa.cG = A.coef[3];
+            aa.cg = A.dt;
+            go = adj_span<P, AK_RK4_LAST, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+        } else if (q > 0) {
+            aa.cG = A.coef[q == 2 ? 3 : 6];
+            aa.cg = A.coef[2];
+            go = adj_span<P, AK_RK4_MID, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+        } else {
+            aa.cG = A.coef[6];
+            go = adj_span<P, AK_RK4_FIRST, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+        }
+        if (!go) return false;
+        // fixed-order sum over the CTA: lanes, then warps
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, off);
+        if (lane == 0) dot_sh[warp] = dot;
+        named_sync(1, CTT);
+        if (tid == 0) {
+            double t = 0.0;
+#pragma unroll
+            for (int w = 0; w < NWT; ++w) t += dot_sh[w];
+            A.dots[blockIdx.x] = t;
+        }
+        if (!updated()) return false;
+        if (blockIdx.x == 0 && warp == 0) {
+            // this stage's dL/df term onto the field samples it reads: the
+            // CTA partials summed by one warp in a fixed order (lane-strided
+            // sums, then a fixed shuffle tree)
+            double t = 0.0;
+            for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(A.dots + b);
+#pragma unroll
+            for (int off = 16; off >= 1; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+            if (lane == 0) {
+                const long long k = A.k0 + i;
+                if (A.sps == 2) {
+                    A.grad[2 * k + h] += t;
+                } else if (h == 0) {
+                    A.grad[k] += t;
+                } else if (h == 2) {
+                    A.grad[k + 1] += t;
+                } else {
+                    A.grad[k] += 0.5 * t;
+                    A.grad[k + 1] += 0.5 * t;
+                }
+            }
+        }
+        return true;
+    }
+    const int est = A.mode == EPI_RK4 ? pass % per : pass % per + 1;
+    const long long ek = A.k0 + pass / per;
+    const int qlast = A.mode == EPI_RK4 ? 3 : A.order;
+    const int eh = A.mode == EPI_RK4 ? (est == 0 ? 0 : (est == 3 ? 2 : 1)) : (A.hold ? 1 : 0);
+    const int kind = A.mode != EPI_RK4 ? EK_TAYLOR : est == 0 ? EK_RK4_FIRST : est < 3 ? EK_RK4_MID : EK_RK4_LAST;
+    const long long N = S0.N;
+    EpiHalf e{};
+    e.s = A.mode == EPI_RK4 ? (est == 3 ? A.coef[6] : est == 2 ? A.dt : A.coef[2]) : A.coef[est];
+    e.first = est == 1;
+    e.last = est == qlast;
+    if (A.ckpt && est == qlast && (ek + 1) % A.ckpt_every == 0 && ek + 1 < A.k_end)
+        e.st_c = A.ckpt + (size_t)((ek + 1) / A.ckpt_every) * N;
+    if (A.store) {
+        const long long i = pass / per;
+        if (est < qlast)
+            e.st_x = A.store + (size_t)(i * A.nst + (A.mode == EPI_RK4 ? est + 1 : est)) * N;
+        else
+            e.st_c = A.store + (size_t)((i + 1) * A.nst) * N;
+    }
+    if (A.nsys > 1) {
+        if (!written()) return false;
+        // this CTA's slice of all systems' amplitudes, system by system
+        const long long T = A.amp_off[A.nsys];
+        const long long g0 = T * blockIdx.x / gridDim.x, g1 = T * (blockIdx.x + 1) / gridDim.x;
+        int si = 0;
+        while (si + 1 < A.nsys && A.amp_off[si + 1] <= g0) ++si;
+#pragma unroll 1
+        for (; si < A.nsys && A.amp_off[si] < g1; ++si) {
+            const SysDesc &Sx = sys[si];
+            const long long o = A.amp_off[si];
+            e.f = field_at(Sx.field, A.sps, ek, eh);
+            epi_span<P, true>(Sx, max(g0, o) - o, min(g1, A.amp_off[si + 1]) - o, tid, CTT, kind, e, NoBar{});
+        }
+    } else {
+        e.f = field_at(S0.field, A.sps, ek, eh);
+        if (!epi_span<P, true>(S0, u0, u1, tid, CTT, kind, e, written)) return false;
+    }
+    return updated();
+}
+
+// Out of line, so that the product's loop, whose accumulators are dead here, is
+// compiled by itself (float-float, lmax=31, n=2000: 180.0 us a stage inlined,
+// 176.5 not).  Inlined where the kernel moves registers between its warps: a
+// function is compiled for the launch's count, and the arguments it would take
+// from before the loop spill (fixed point: 353 us out of line, 331 inlined).
+template <class P, int CTT>
+__device__ __noinline__ bool step_update(const SysDesc *sys, const StepArgs &A, int pass, volatile int *abort, int *err,
+                                         volatile int *go_flag, double *dot_sh, long long u0, long long u1)
+{
+    return step_update_inline<P, CTT>(sys, A, pass, abort, err, go_flag, dot_sh, u0, u1);
+}
+
 // Threads of a launch: the consumers and the producer warp.  Nine warps are
 // left 168 registers each, and fixed-point columns take 18 (two 64-bit sums,
 // the running one, x): with six or eight columns a thread the producer gets a
@@ -96,7 +245,7 @@ template <class P, int CT, int MAXG, int NGRP> __host__ __device__ constexpr int
 // consumers with column sums of their own take the stages in turn.  For blocks
 // that stay in L2, where a plan has one CTA per SM and one warp per scheduler
 // would wait out the latency of every multiply (lmax=15, n=500: 34.3 -> 30.9 us
-// a stage).  Not for single products: 288 threads of 168 registers do not fit
+// a stage, both with the update by whole amplitudes; 23.4 by components).  Not for single products: 288 threads of 168 registers do not fit
 // beside the previous kernel's blocks, so the ring no longer fills while that
 // one finishes (lmax=7, n=301: a product and its update 34 -> 46 us).
 template <class P, int CT, int MAXG, int RS, bool STEP, int NGRP = 1>
@@ -130,6 +279,7 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
     __shared__ typename std::conditional<(NGRP > 1), CRun, char>::type comb[NGRP > 1 ? 2 * MAXG * CW : 1][NGRP > 1 ? CT : 1];   // the second group's column sums
     __shared__ float xmax_sh[NWT], xrow_sh[NWT];
     __shared__ __align__(16) typename std::conditional<P::kFixed, int2, char>::type xfix[P::kFixed ? NWT : 1][2 * RS];   // the stage's x_l in fixed point, per warp
+    __shared__ typename std::conditional<STEP, StepArgs, char>::type step_args;       // STEP: the launch's arguments, for step_update
     __shared__ int xready, go_flag;       // STEP: passes whose stage inputs are written; barrier verdict
     __shared__ double dot_sh[NWT];         // STEP, adjoint: per-warp field-gradient partials
 
@@ -146,6 +296,9 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
         xready = 0;
         go_flag = 0;
         fence_mbar_init();
+    }
+    if constexpr (STEP) {
+        if (tid == 0) step_args = A;
     }
     __syncthreads();
     const int s0 = cta_off[blockIdx.x], s1 = cta_off[blockIdx.x + 1];
@@ -268,6 +421,11 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
         // ------------------------------------------------- consumer warps
         if constexpr (kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
         const int grp = NGRP > 1 ? warp / NW : 0, lw = NGRP > 1 ? warp % NW : warp, ctid = NGRP > 1 ? tid % CT : tid;
+        long long u0 = 0, u1 = 0;          // STEP: this CTA's slice of sys[0]'s amplitudes
+        if constexpr (STEP && !kSplit) {
+            u0 = (long long)sys[0].N * blockIdx.x / gridDim.x;
+            u1 = (long long)sys[0].N * (blockIdx.x + 1) / gridDim.x;
+        }
         int q = 0;
         int parity = 0;
         for (int pass = 0; pass < npass; ++pass) {
@@ -387,8 +545,11 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                         if (live && lane < 2 * nr) xfix[warp][lane] = P::fix(reinterpret_cast<const double *>(&xs_raw[s][0])[lane], xexp);
                         __syncwarp();
                     }
+                    // Narrow fixed-point layouts stop at the segment's last row (half-empty stages are
+                    // a sixth of n = 500's); wide ones run the constant count: their stages are
+                    // nearly all full and the bound's register spills (306 against 324 us at 31:2000).
 #pragma unroll 1
-                    for (int sub = 0; sub < RS; sub += CR) {
+                    for (int sub = 0; sub < (P::kFixed && !kSplit ? nr : RS); sub += CR) {
                     typename P::RowAcc rre[CR], rim[CR];
 #pragma unroll
                     for (int rr = 0; rr < CR; ++rr) { rre[rr] = P::rzero(sig); rim[rr] = P::rzero(sig); }
@@ -428,7 +589,7 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                                     P::rfmax(cpr[g][c], cpi[g][c], u[rr][g][c], xi[rr], csig);
                                 }
                     }
-                    if (sub + CR >= RS) {
+                    if (!P::kFixed) {
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&empty[s]);
                         ++q;
@@ -468,6 +629,11 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                     }
                     if ((lane & (DUPS - 1)) == 0) red[parity][lw][2 * (st * RS + sub) + idx] = v[0];
                     }
+                    }
+                    if constexpr (P::kFixed) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&empty[s]);
+                        ++q;
                     }
                 }
                 if constexpr (P::kOffsetSums || P::kFixed) {
@@ -543,116 +709,13 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
             }
         }
         if constexpr (STEP) {
-            // every row sum and column partial of this pass is written
-            if (!grid_sync(A.gbar, (unsigned)(2 * pass + 1) * gridDim.x, abort, err, &go_flag, tid, CTT)) break;
-            // the stage update of this CTA's slice of amplitudes
-            const SysDesc &S0 = sys[0];
-            const int per = A.mode == EPI_RK4 ? 4 : A.order;
-            if (A.reverse) {
-                // reverse stage q of step k0+i (the segment's last step first)
-                const int i = A.ns - 1 - pass / per;
-                const int q = A.mode == EPI_RK4 ? 3 - pass % per : A.order - pass % per;
-                const int fq = A.mode == EPI_RK4 ? q : q - 1;
-                const SysDesc &Sa = sys[0];
-                const long long Na = Sa.N;
-                AdjArgs aa{};
-                aa.scheme = A.mode == EPI_RK4 ? 0 : 1;
-                aa.stage = q;
-                aa.order = A.order;
-                aa.hold = A.hold;
-                aa.sps = A.sps;
-                aa.k = A.k0 + i;
-                aa.dt = A.dt;
-                aa.fwd = (fq == 0 && i == 0) ? A.ckpt0 : A.store + (size_t)((long long)i * A.nst + fq) * Na;
-                aa.G = A.G;
-                double dot = 0.0;
-                const long long a1 = Na * (blockIdx.x + 1) / gridDim.x;
-#pragma unroll 1
-                for (long long a = Na * blockIdx.x / gridDim.x + tid; a < a1; a += CTT) dot += adj_amp<P, true>(Sa, a, aa);
-                // fixed-order sum over the CTA: lanes, then warps
-#pragma unroll
-                for (int off = 16; off >= 1; off >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, off);
-                if (lane == 0) dot_sh[warp] = dot;
-                named_sync(1, CTT);
-                if (tid == 0) {
-                    double t = 0.0;
-#pragma unroll
-                    for (int w = 0; w < NWT; ++w) t += dot_sh[w];
-                    A.dots[blockIdx.x] = t;
-                }
-                if (!grid_sync(A.gbar, (unsigned)(2 * pass + 2) * gridDim.x, abort, err, &go_flag, tid, CTT)) break;
-                if (blockIdx.x == 0 && warp == 0) {
-                    // this stage's dL/df term onto the field samples it reads: the
-                    // CTA partials summed by one warp in a fixed order (lane-strided
-                    // sums, then a fixed shuffle tree)
-                    double t = 0.0;
-                    for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(A.dots + b);
-#pragma unroll
-                    for (int off = 16; off >= 1; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-                    if (lane == 0) {
-                        const int h = A.mode == EPI_RK4 ? (q == 0 ? 0 : (q == 3 ? 2 : 1)) : (A.hold ? 1 : 0);
-                        const long long k = A.k0 + i;
-                        if (A.sps == 2) {
-                            A.grad[2 * k + h] += t;
-                        } else if (h == 0) {
-                            A.grad[k] += t;
-                        } else if (h == 2) {
-                            A.grad[k + 1] += t;
-                        } else {
-                            A.grad[k] += 0.5 * t;
-                            A.grad[k + 1] += 0.5 * t;
-                        }
-                    }
-                }
-                if (tid == 0) {
-                    __threadfence_block();
-                    *(volatile int *)&xready = pass + 1;
-                }
-                continue;
-            }
-            EpiArgs e{};
-            e.mode = A.mode;
-            e.stage = A.mode == EPI_RK4 ? pass % per : pass % per + 1;
-            e.order = A.order;
-            e.hold = A.hold;
-            e.sps = A.sps;
-            e.dt = A.dt;
-            e.k = A.k0 + pass / per;
-            const long long N = S0.N;
-            const int qlast = A.mode == EPI_RK4 ? 3 : A.order;
-            if (A.ckpt && e.stage == qlast && (e.k + 1) % A.ckpt_every == 0 && e.k + 1 < A.k_end)
-                e.st_c = A.ckpt + (size_t)((e.k + 1) / A.ckpt_every) * N;
-            if (A.store) {
-                const long long i = pass / per;
-                if (e.stage < qlast)
-                    e.st_x = A.store + (size_t)(i * A.nst + (A.mode == EPI_RK4 ? e.stage + 1 : e.stage)) * N;
-                else
-                    e.st_c = A.store + (size_t)((i + 1) * A.nst) * N;
-            }
-            if (A.nsys > 1) {
-                // this CTA's slice of all systems' amplitudes, system by system
-                const long long T = A.amp_off[A.nsys];
-                const long long g0 = T * blockIdx.x / gridDim.x, g1 = T * (blockIdx.x + 1) / gridDim.x;
-                int si = 0;
-                while (si + 1 < A.nsys && A.amp_off[si + 1] <= g0) ++si;
-#pragma unroll 1
-                for (; si < A.nsys && A.amp_off[si] < g1; ++si) {
-                    const SysDesc &Sx = sys[si];
-                    const long long o = A.amp_off[si];
-                    const long long hi = min(g1, A.amp_off[si + 1]) - o;
-#pragma unroll 1
-                    for (long long a = max(g0, o) - o + tid; a < hi; a += CTT) epi_amp<P, true>(Sx, a, e, epi_pre(Sx, a));
-                }
-            } else {
-                const long long a1 = N * (blockIdx.x + 1) / gridDim.x;
-#pragma unroll 1
-                for (long long a = N * blockIdx.x / gridDim.x + tid; a < a1; a += CTT) {
-                    const EpiPre pre = epi_pre(S0, a);
-                    epi_amp<P, true>(S0, a, e, pre);
-                }
-            }
-            // every input of the next pass is written
-            if (!grid_sync(A.gbar, (unsigned)(2 * pass + 2) * gridDim.x, abort, err, &go_flag, tid, CTT)) break;
+            bool go;
+            if constexpr (kSplit)
+                go = step_update_inline<P, CTT>(sys, A, pass, abort, err, &go_flag, dot_sh,
+                                                (long long)sys[0].N * blockIdx.x / gridDim.x,
+                                                (long long)sys[0].N * (blockIdx.x + 1) / gridDim.x);
+            else go = step_update<P, CTT>(sys, step_args, pass, abort, err, &go_flag, dot_sh, u0, u1);
+            if (!go) break;
             if (tid == 0) {
                 __threadfence_block();
                 *(volatile int *)&xready = pass + 1;
