@@ -538,7 +538,7 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
 {
     const int S = tdse::dig_slices(ctx->prec), L = ctx->lmax + 1, n = ctx->n;
     const int ldb = (n + 7) & ~7, nb = (n + 63) & ~63;
-    const tdse::DigTile tile = tdse::dig_tile(S, n, B);
+    const tdse::DigTile tile = tdse::dig_tile(S, n, ctx->lmax, B);
     const long long plane = (long long)L * nb;
     const size_t ub = sizeof(__nv_bfloat16) * 2 * S * (size_t)ctx->lmax * n * ldb;
     const size_t xb = sizeof(__nv_bfloat16) * S * 2 * (size_t)B * plane;

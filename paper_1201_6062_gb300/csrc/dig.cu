@@ -244,12 +244,34 @@ static int dig_sms()
     return sms < 2 ? 2 : sms & ~1;
 }
 
-DigTile dig_tile(int slices, int n, int B)
+// The tile whose longest CTA (pair) is estimated to finish first.  CTA 0 has the
+// longest share of the walk (dig_tile_of).  Cycles of a step (one digit pair of
+// tiles, 64 columns): measured 500-530 at 32 planes, 510-600 at 64 and 620-840 at
+// 128, 620 and 690 for single CTAs: the issue of the products and their loads
+// more than the products themselves, except at 128.  The update of the last tile
+// follows its products, some 1000 cycles a pulse.  Measured, us a stage at 32 /
+// 64 / 128 planes: FP32, lmax=9, n=487, 100 pulses 71 / 77 / 80, lmax=20, n=200,
+// 300 pulses 104 / 95 / 119, lmax=15, n=1000, 64 pulses 195 / 141 / 128;
+// float-float, lmax=15, n=1000, 256 pulses - / 706 / 499; FP64, lmax=7, n=301, 24
+// pulses 68 / 85 (one size for all shapes gave 80, 119, 128, 499 and 85).
+DigTile dig_tile(int slices, int n, int lmax, int B)
 {
-    const int want = 2 * B;
-    if (want <= 32) return DigTile{1, 32};
-    if (want <= 64) return DigTile{n > 128 ? 2 : 1, 64};
-    return DigTile{n > 128 ? 2 : 1, n > 128 && slices < 8 ? 128 : 64};
+    const int cg = n > DBM ? 2 : 1, units = dig_sms() / cg, mt = (n + DBM * cg - 1) / (DBM * cg);
+    const long long steps = (long long)((n + DBK - 1) / DBK) * (slices / 2) * (slices / 2 + 1);
+    DigTile best{cg, 32};
+    long long low = 0;
+    for (int bn = 32; bn <= (cg == 2 && slices < 8 ? 128 : 64); bn *= 2) {
+        const long long per = (long long)mt * ((2LL * B + bn - 1) / bn), tiles = per * (lmax + 1);
+        long long parts = 0;                             // products of CTA 0
+        for (long long t = 0; t < tiles; t += units) parts += lmax > 1 && t < per * (lmax - 1) ? 2 : 1;
+        const int step = cg == 1 ? (bn == 32 ? 620 : 690) : (bn == 32 ? 510 : (bn == 64 ? 570 : 700));
+        const long long est = parts * steps * step + 500LL * bn;
+        if (bn == 32 || est < low) {
+            low = est;
+            best.bn = bn;
+        }
+    }
+    return best;
 }
 
 size_t dig_scratch_bytes(DigTile t) { return (size_t)dig_sms() * (t.bn / 2) * DBM * sizeof(float4); }

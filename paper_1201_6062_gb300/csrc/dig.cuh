@@ -53,14 +53,18 @@ namespace tdse {
 
 constexpr int DBM = 128, DBK = 64;
 constexpr int DA_BYTES = DBM * DBK * 2;                 // 16 KB
-constexpr int DIG_DRAIN_WARPS = 8, DIG_UPD_WARPS = 4;
-constexpr int DIG_THREADS = 128 + 32 * (DIG_DRAIN_WARPS + DIG_UPD_WARPS);   // warps 0..2: operand loads, MMA issue, state loads
-// Registers: launched with 128 per thread; the first warpgroup keeps 40, the
-// draining ones take 176 each for the running sums, the updating one 120:
-// 128 * (40 + 2 * 176 + 120) = 512 * 128.
-constexpr int DIG_REGS_LAUNCH = 128, DIG_REGS_LOW = 40, DIG_REGS_DRAIN = 176, DIG_REGS_UPD = 120;
-static_assert(128 * DIG_REGS_LOW + 32 * DIG_DRAIN_WARPS * DIG_REGS_DRAIN + 32 * DIG_UPD_WARPS * DIG_REGS_UPD <=
-              DIG_THREADS * DIG_REGS_LAUNCH, "register split");
+constexpr int DIG_DRAIN_WARPS = 8, DIG_UPD_WARPS = 8;
+constexpr int DIG_THREADS = 128 + 32 * (DIG_DRAIN_WARPS + DIG_UPD_WARPS);   // warps 0..3: loads of A, MMA issue, state loads, loads of B
+// Registers: launched with 96 per thread.  Tiles of 128 planes: the first
+// warpgroup keeps 32, the draining ones take 160 each for the running sums, the
+// updating ones keep 64: 128 * (32 + 2 * 160 + 2 * 64) = 640 * 96; smaller
+// tiles: 40, 144, 72.
+constexpr int DIG_REGS_LAUNCH = 96;
+__host__ __device__ constexpr int dig_regs_low(int bn) { return bn == 128 ? 32 : 40; }
+__host__ __device__ constexpr int dig_regs_drain(int bn) { return bn == 128 ? 160 : 144; }
+__host__ __device__ constexpr int dig_regs_upd(int bn) { return bn == 128 ? 64 : 72; }
+__host__ __device__ constexpr int dig_regs(int bn) { return 128 * dig_regs_low(bn) + 32 * DIG_DRAIN_WARPS * dig_regs_drain(bn) + 32 * DIG_UPD_WARPS * dig_regs_upd(bn); }
+static_assert(dig_regs(128) <= DIG_THREADS * DIG_REGS_LAUNCH && dig_regs(64) <= DIG_THREADS * DIG_REGS_LAUNCH, "register split");
 constexpr uint64_t DIG_WAIT_NS = 2000000000ull;
 constexpr int DIG_SUPER = 8;                            // K tiles (of 64) per round over the groups
 constexpr int DIG_NONFINITE = 0x7ff00000;               // xmax / eu mark of a non-finite maximum
@@ -134,7 +138,14 @@ template <int NC> struct DigAcc<8, NC> {
             a[j] += (long long)__float2int_rn(even) << 32;
         }
     }
-    __device__ __forceinline__ double value(int j) const { return ((double)a[j] + (double)l[j]) * 0x1p-32; }
+    // the sum times 2^e, from the bits (96: units of 2^-24 of the fourth weight's, 2^-9 of what the left-out
+    // pairs may add); in FP64, conversions, sum and scale held the pipe 20000 cycles a product
+    __device__ __forceinline__ double value(int j, int e) const
+    {
+        const long long f = __float2ll_rn(__fmul_rn(l[j], 0x1p24f));
+        PolI64::CRun r{(unsigned)(a[j] << 24), (unsigned)(a[j] >> 8), (int)(a[j] >> 40)};
+        return PolI64::to_f64(PolI64::cadd(r, PolI64::CRun{(unsigned)f, (unsigned)(f >> 32), (int)(f >> 63)}), e - 56);
+    }
 };
 
 // Exponent of the power of two above a maximum with high word h (S = 8 keeps one bit of headroom).
@@ -146,12 +157,6 @@ template <int S> __device__ __forceinline__ int dig_exp(int h)
 __device__ __forceinline__ float dig_pow2f(int e)       // 2^e for e <= 127, 0 below 2^-126
 {
     return e < -126 ? 0.f : __int_as_float((e + 127) << 23);
-}
-
-__device__ __forceinline__ double dig_scale(double v, int e)
-{
-    if (e > -1000 && e < 1000) return v * __hiloint2double((e + 1023) << 20, 0);
-    return scalbn(v, e);
 }
 
 // f 2^e for a float f that is zero or normal (a subnormal f counts as zero) and |e| < 800, from the bits of f.
@@ -166,6 +171,14 @@ __device__ __forceinline__ double dig_join(float h, float l, int e)     // (h + 
 {
     if (e > -800 && e < 800) return dig_widen(h, e) + dig_widen(l, e);
     return scalbn((double)h + (double)l, e);
+}
+
+// Biased exponents (+ 2048) of a pulse's two columns in 16-bit halves, bit 15 of a half: not finite.
+template <int S> __device__ __forceinline__ int dig_pack(const int *m)
+{
+    const int2 h = *reinterpret_cast<const int2 *>(m);
+    return (dig_exp<S>(h.x) + 2048 + (h.x >= DIG_NONFINITE ? 0x8000 : 0)) |
+           (int)((unsigned)(dig_exp<S>(h.y) + 2048 + (h.y >= DIG_NONFINITE ? 0x8000 : 0)) << 16);
 }
 
 // The shift applied to the first product's sum, in exponents of the two products' units.
@@ -244,8 +257,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
     __shared__ __align__(8) uint64_t mma_drain;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
-    __shared__ int issued, consumed;
-    __shared__ int st_issued, st_used;
+    __shared__ int issued[2], consumed;
+    __shared__ int st_issued, st_used[2];
     unsigned char *slots = smem + (size_t)NST * STAGE;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform)
@@ -270,13 +283,13 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         mbar_init(&d_empty, DIG_UPD_WARPS);
         for (int q = 0; q < DIG_NSU; ++q) {
             mbar_init(&st_full[q], 1);
-            mbar_init(&st_empty[q], DIG_UPD_WARPS);
+            mbar_init(&st_empty[q], DIG_UPD_WARPS / 2);
         }
         mbar_init(&mma_drain, 1);
         st_issued = 0;
-        st_used = 0;
+        st_used[0] = st_used[1] = 0;
         abort_flag = 0;
-        issued = 0;
+        issued[0] = issued[1] = 0;
         consumed = 0;
         fence_mbar_init();
     }
@@ -291,43 +304,49 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
     pdl_wait();                                          // state digits and maxima come from the previous kernel
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(DIG_REGS_LOW));
-        if (warp == 0) {
-            // --------------------------------------------------- TMA producer
-            if (lane == 0) {
-                int s = 0, it = 0;
-                uint32_t ph = 1;                         // parity of the slot's previous release
-                for (int t = first; t < ntiles && !*abort; t += stride) {
-                    int l, rem;
-                    dig_tile_of(t, mt * nt, L, l, rem);
-                    const int i0 = ((rem / nt) * CG + rank) * DBM, c0 = (rem % nt) * BN + rank * (BN / CG);
-                    for (int part = 0; part < 2 && !*abort; ++part) {
-                        if ((part == 0 && l >= A.lmax) || (part == 1 && l < 1)) continue;
-                        const int za = part * S * A.lmax + (part == 0 ? l : l - 1);       // + s * lmax
-                        const int xcol = (part == 0 ? l + 1 : l - 1) * A.nb;
-                        for (int k0 = 0; k0 < nk && !*abort; k0 += DIG_SUPER)
-                            for (int g = NG - 1; g >= 0 && !*abort; --g) {
-                                const int k1 = min(k0 + DIG_SUPER, nk);
-                                for (int kb = k0; kb < k1 && !*abort; ++kb)
-                                    for (int st = 0; st < 2 * g + 2; ++st) {
-                                        if (it >= NST && !mbar_wait_bounded(&empty[s], ph, abort, DIG_WAIT_NS)) break;
-                                        unsigned char *p = smem + (size_t)s * STAGE;
-                                        if (rank == 0) mbar_arrive_expect_tx(&full[s], CG * STAGE);
-                                        if constexpr (CG == 2) {
-                                            const uint32_t bar = cluster_addr(&full[s], 0);
-                                            tma_load_3d_pair(p, &M.U, kb * DBK, i0, za + st * A.lmax, bar);
-                                            tma_load_3d_pair(p + DA_BYTES, &M.X, xcol + kb * DBK, c0, 2 * g + 1 - st, bar);
-                                        } else {
-                                            tma_load_3d(p, &M.U, kb * DBK, i0, za + st * A.lmax, &full[s]);
-                                            tma_load_3d(p + DA_BYTES, &M.X, xcol + kb * DBK, c0, 2 * g + 1 - st, &full[s]);
-                                        }
-                                        issued = ++it;
-                                        if (++s == NST) { s = 0; ph ^= 1; }
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_low(BN)));
+        if (warp == 0 || warp == 3) {
+            // ------- operand loads: warp 0 those of A (rows of U), warp 3 those of B (pulse planes)
+            // Whole-warp loops with an elected issuer, as the products below: one
+            // diverged lane loading both took 400 cycles a step.
+            const bool isb = warp == 3;
+            const CUtensorMap *tm = isb ? &M.X : &M.U;
+            int s = 0, it = 0;
+            uint32_t ph = 1;                             // parity of the slot's previous release
+            bool ok = true;
+            for (int t = first; t < ntiles && ok; t += stride) {
+                int l, rem;
+                dig_tile_of(t, mt * nt, L, l, rem);
+                const int y = isb ? (rem % nt) * BN + rank * (BN / CG) : ((rem / nt) * CG + rank) * DBM;
+                for (int part = 0; part < 2 && ok; ++part) {
+                    if ((part == 0 && l >= A.lmax) || (part == 1 && l < 1)) continue;
+                    const int za = part * S * A.lmax + (part == 0 ? l : l - 1), dz = isb ? -1 : A.lmax;
+                    const int xcol = isb ? (part == 0 ? l + 1 : l - 1) * A.nb : 0;
+                    for (int k0 = 0; k0 < nk && ok; k0 += DIG_SUPER)
+                        for (int g = NG - 1; g >= 0 && ok; --g) {
+                            const int k1 = min(k0 + DIG_SUPER, nk);
+                            for (int kb = k0; kb < k1 && ok; ++kb) {
+                                int z = isb ? 2 * g + 1 : za;                // digit plane of step 0
+                                for (int st = 0; st < 2 * g + 2; ++st, z += dz) {
+                                    if (it >= NST) {
+                                        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph, abort, DIG_WAIT_NS)) != 0;
+                                        if (!ok) break;
                                     }
+                                    if (elect_one()) {
+                                        unsigned char *p = smem + (size_t)s * STAGE + (isb ? DA_BYTES : 0);
+                                        if (!isb && rank == 0) mbar_arrive_expect_tx(&full[s], CG * STAGE);
+                                        if constexpr (CG == 2) tma_load_3d_pair(p, tm, xcol + kb * DBK, y, z, cluster_addr(&full[s], 0));
+                                        else tma_load_3d(p, tm, xcol + kb * DBK, y, z, &full[s]);
+                                    }
+                                    __syncwarp();
+                                    ++it;
+                                    if (++s == NST) { s = 0; ph ^= 1; }
+                                }
                             }
-                    }
+                        }
                 }
             }
+            if (lane == 0) issued[isb] = it;
         } else if (warp == 1 && rank == 0) {
             // ----------------------------------- MMA issuer (of the pair's even CTA)
             constexpr uint32_t idesc = idesc_bf16(DBM * CG, BN);
@@ -426,7 +445,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         }
     } else if (warp < 4 + DIG_DRAIN_WARPS) {
         // ------------------------------------------- draining warps 4..11
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(DIG_REGS_DRAIN));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(dig_regs_drain(BN)));
         const int quarter = warp & 3;                    // TMEM lanes this warp may read
         const int half = (warp - 4) >> 2;                // which half of the tile's columns
         const int ncol = 2 * A.B;
@@ -495,8 +514,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                             const int col = c0 + 2 * p;
                             double2 v = make_double2(0.0, 0.0);
                             if (both && col < ncol)
-                                v = make_double2(dig_scale(R.value(2 * p), eu0 + dig_exp<S>(m0[col]) - 14),
-                                                 dig_scale(R.value(2 * p + 1), eu0 + dig_exp<S>(m0[col + 1]) - 14));
+                                v = make_double2(R.value(2 * p, eu0 + dig_exp<S>(m0[col]) - 14),
+                                                 R.value(2 * p + 1, eu0 + dig_exp<S>(m0[col + 1]) - 14));
                             scr[p * DBM].d = v;
                         }
                         R.clear();
@@ -525,8 +544,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                     if (row < n && col < ncol) {
                         const int *m = A.xmax + (long long)(l >= 1 ? l - 1 : l + 1) * ncol + col;
                         const int e = (l >= 1 ? A.eu[(long long)(A.lmax + l - 1) * n + row] : A.eu[(long long)l * n + row]) - 14;
-                        v = make_double2(dig_scale(R.value(2 * p), e + dig_exp<S>(m[0])),
-                                         dig_scale(R.value(2 * p + 1), e + dig_exp<S>(m[1])));
+                        v = make_double2(R.value(2 * p, e + dig_exp<S>(m[0])), R.value(2 * p + 1, e + dig_exp<S>(m[1])));
                         if (l >= 1 && A.gauge) v = make_double2(-v.x, -v.y);
                         if (both) {
                             const double2 w = scr[p * DBM].d;
@@ -542,18 +560,20 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             if (lane == 0) mbar_arrive(&d_full);
         }
     } else {
-        // ------------------------------------------- updating warps 12..15
-        // The states of a pulse are staged in shared memory by warp 2 (a load
-        // takes some 3500 cycles behind the operand tiles), D x is read UD
-        // pulses ahead.
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(DIG_REGS_UPD));
-        constexpr int UD = 4;
-        const int r0 = (warp - 4 - DIG_DRAIN_WARPS) * 32 + lane;
+        // ------------------------------------------- updating warps 12..19
+        // Two groups of four warps (128 rows) take the pulses in turn: a pulse is
+        // a chain of some 1200 cycles besides the 640 its FP64 instructions hold
+        // a scheduler's pipe, so one group alone leaves that pipe idle.  The states
+        // of a pulse are staged in shared memory by warp 2 (a load takes some 3500
+        // cycles behind the operand tiles), D x is read one pulse ahead.
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_upd(BN)));
+        const int grp = (warp - 4 - DIG_DRAIN_WARPS) >> 2;
+        const int r0 = (warp & 3) * 32 + lane;
         const int ncol = 2 * A.B;
         const bool first_stage = dig_first(A);
         const bool last_stage = A.stage == (A.mode == EPI_RK4 ? 3 : A.order);
         const DigOut *scr = reinterpret_cast<const DigOut *>(A.scratch) + (size_t)blockIdx.x * (BN / 2) * DBM + r0;
-        int jt = 0, it = 0;
+        int jt = 0, it0 = 0;                             // tiles, state slots before this tile
         bool ok = true;
         for (int t = first; t < ntiles && ok; t += stride, ++jt) {
             int l, rem;
@@ -562,90 +582,79 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             const int b0 = (rem % nt) * (BN / 2);        // first pulse
             const int np = i0 < n ? min(BN / 2, A.B - b0) : 0;
             const bool valid = row < n;
-            const long long a = (long long)l * n + row;
             const bool up = l < A.lmax, dn = l >= 1;
-            const int eu0 = valid && up ? A.eu[(long long)l * n + row] : 0;
-            const int eu1 = valid && dn ? A.eu[(long long)(A.lmax + l - 1) * n + row] : 0;
-            const double e = valid ? A.E[a] : 0.0;
-            const int *m0 = A.xmax + (long long)(l + 1) * ncol, *m1 = A.xmax + (long long)(l - 1) * ncol;
+            int eu0 = valid && up ? A.eu[(long long)l * n + row] : 0;
+            int eu1 = valid && dn ? A.eu[(long long)(A.lmax + l - 1) * n + row] : 0;
+            const int ubad = max(eu0, eu1) >= DIG_NONFINITE ? 0x80008000 : 0;
+            const long long a = (long long)b0 * A.N + (long long)l * n + row;
+            const double e = valid ? A.E[(long long)l * n + row] : 0.0;
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(&d_full, (uint32_t)(jt & 1), abort, DIG_WAIT_NS)) != 0;
             if (!ok) break;
-            DigOut o[UD], nx[UD];
-#pragma unroll
-            for (int u = 0; u < UD; ++u) nx[u].f = scr[u * DBM].f;
-            int h0 = 0, h1 = 0, mine = 0;                // of column 2 (b0 + 16 block) + lane
-            double fv = 0.0;                             // of pulse b0 + 16 block + lane % 16
+            DigOut nx;
+            nx.f = scr[grp * DBM].f;
             auto pulses = [&](auto kc) {
                 constexpr int KIND = decltype(kc)::value;
 #pragma unroll 1
-            for (int p4 = 0; p4 < np && ok; p4 += UD) {
-                if ((p4 & 15) == 0) {
-                    const int col = 2 * (b0 + p4) + lane, pb = b0 + p4 + (lane & 15);
-                    h0 = up && col < ncol ? __ldg(m0 + col) : 0;
-                    h1 = dn && col < ncol ? __ldg(m1 + col) : 0;
-                    fv = pb < A.B ? __ldg(A.fval + pb) : 0.0;
-                    mine = 0;
-                }
+                for (int p32 = 0; p32 < np && ok; p32 += 32) {
+                    // pulse b0 + p32 + lane: field value, exponents of the columns of the two products (two 16-bit
+                    // halves, bias 2048, bit 15: not finite); the maxima of column lane % 2 of the group's pulse lane / 2
+                    const int pb = b0 + p32 + lane;
+                    const double fv = pb < A.B ? __ldg(A.fval + pb) : 0.0;
+                    const int x0 = up && pb < A.B ? dig_pack<S>(A.xmax + (long long)(l + 1) * ncol + 2 * pb) : 0;
+                    const int x1 = dn && pb < A.B ? dig_pack<S>(A.xmax + (long long)(l - 1) * ncol + 2 * pb) : 0;
+                    int mine = 0;
+                    const int pe = min(p32 + 32, np);
+#pragma unroll 1
+                    for (int p = p32 + grp; p < pe; p += 2) {
+                        DigOut o;
+                        o.f = nx.f;
+                        nx.f = scr[min(p + 2, BN / 2 - 1) * DBM].f;
+                        const int it = it0 + p, s = it % DIG_NSU;
+                        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&st_full[s], (uint32_t)((it / DIG_NSU) & 1), abort, DIG_WAIT_NS)) != 0;
+                        if (!ok) return;
+                        const double2 *sl = reinterpret_cast<const double2 *>(slots + s * DIG_SLOT) + r0;
+                        DigIn in;
+                        in.c = sl[0];
+                        in.x = first_stage ? in.c : sl[DBM];
+                        in.acc = sl[2 * DBM];
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&st_empty[s]);
+                        const int q = p & 31;
+                        const double f = __shfl_sync(0xffffffffu, fv, q);
+                        const int s0 = __shfl_sync(0xffffffffu, x0, q), s1 = __shfl_sync(0xffffffffu, x1, q);
+                        const int bad = s0 | s1 | ubad;
+                        double d[2];
 #pragma unroll
-                for (int u = 0; u < UD; ++u) {
-                    o[u].f = nx[u].f;
-                    nx[u].f = scr[min(p4 + UD + u, BN / 2 - 1) * DBM].f;
-                }
-#pragma unroll
-                for (int u = 0; u < UD; ++u) {
-                    const int p = p4 + u;
-                    if (p >= np || !ok) continue;
-                    const int s = it % DIG_NSU;
-                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&st_full[s], (uint32_t)((it / DIG_NSU) & 1), abort, DIG_WAIT_NS)) != 0;
-                    const double2 *sl = reinterpret_cast<const double2 *>(slots + s * DIG_SLOT) + r0;
-                    DigIn in;
-                    in.c = sl[0];
-                    in.x = first_stage ? in.c : sl[DBM];
-                    in.acc = sl[2 * DBM];
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&st_empty[s]);
-                    ++it;
-                    const int q0 = 2 * (p & 15);
-                    const double f = __shfl_sync(0xffffffffu, fv, q0 >> 1);
-                    double d[2];
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        const int g0 = __shfl_sync(0xffffffffu, h0, q0 + w), g1 = __shfl_sync(0xffffffffu, h1, q0 + w);
-                        const bool bad = max(max(eu0, eu1), max(g0, g1)) >= DIG_NONFINITE;
-                        if constexpr (S == 8) {
-                            d[w] = w ? o[u].d.y : o[u].d.x;
-                        } else {
-                            const int e0 = eu0 + dig_exp<S>(g0), e1 = eu1 + dig_exp<S>(g1);
-                            int ee = e0;
-                            if (dn) ee = up ? e1 + max(e0 - e1 - 100, 0) : e1;
-                            const float4 v = o[u].f;
-                            d[w] = dig_join(w ? v.z : v.x, w ? v.w : v.y, ee - 14);
-                            if (dn && A.gauge) d[w] = -d[w];
+                        for (int w = 0; w < 2; ++w) {
+                            if constexpr (S == 8) {
+                                d[w] = w ? o.d.y : o.d.x;
+                            } else {
+                                const int e0 = eu0 + ((s0 >> (16 * w)) & 0x7fff), e1 = eu1 + ((s1 >> (16 * w)) & 0x7fff);
+                                int ee = e0;
+                                if (dn) ee = up ? e1 + max(e0 - e1 - 100, 0) : e1;
+                                const float4 v = o.f;
+                                d[w] = dig_join(w ? v.z : v.x, w ? v.w : v.y, ee - (2048 + 14));
+                                if (dn && A.gauge) d[w] = -d[w];
+                            }
+                            if (bad & (0x8000 << (16 * w))) d[w] = __longlong_as_double(0x7ff8000000000000LL);
                         }
-                        if (bad) d[w] = __longlong_as_double(0x7ff8000000000000LL);
-                    }
-                    const DigNext nw = dig_update<KIND>(A, e, f, d[0], d[1], in);
-                    if (valid) {
-                        const long long q = (long long)(b0 + p) * A.N + a;
-                        if (last_stage) {
-                            A.c[q] = nw.out;
-                        } else {
-                            A.x[q] = nw.out;
-                            A.acc[q] = nw.acc;
+                        const DigNext nw = dig_update<KIND>(A, e, f, d[0], d[1], in);
+                        if (valid) {
+                            const long long at = a + (long long)p * A.N;
+                            if (last_stage) {
+                                A.c[at] = nw.out;
+                            } else {
+                                A.x[at] = nw.out;
+                                A.acc[at] = nw.acc;
+                            }
                         }
+                        const int mr = (int)__reduce_max_sync(0xffffffffu, valid ? (unsigned)__double2hiint(nw.out.x) & 0x7fffffffu : 0u);
+                        const int mi = (int)__reduce_max_sync(0xffffffffu, valid ? (unsigned)__double2hiint(nw.out.y) & 0x7fffffffu : 0u);
+                        if ((lane >> 1) == (q >> 1)) mine = lane & 1 ? mi : mr;
                     }
-                    // the maxima of the pulse's two columns over the warp's rows, kept by lanes q0 and q0 + 1
-                    const int mr = (int)__reduce_max_sync(0xffffffffu, valid ? (unsigned)__double2hiint(nw.out.x) & 0x7fffffffu : 0u);
-                    const int mi = (int)__reduce_max_sync(0xffffffffu, valid ? (unsigned)__double2hiint(nw.out.y) & 0x7fffffffu : 0u);
-                    if (lane == q0) mine = mr;
-                    if (lane == q0 + 1) mine = mi;
+                    const int pl = p32 + 2 * (lane >> 1) + grp;
+                    if (pl < pe && mine > 0) atomicMax(A.xmax_next + (long long)l * ncol + 2 * (b0 + pl) + (lane & 1), mine);
                 }
-                if (!ok) return;
-                if ((p4 & 15) == 16 - UD || p4 + UD >= np) {
-                    const int col = 2 * (b0 + (p4 & ~15)) + lane;
-                    if (col < ncol && mine > 0) atomicMax(A.xmax_next + (long long)l * ncol + col, mine);
-                }
-            }
             };
             switch (A.mode != EPI_RK4 ? DIG_TAYLOR : A.stage == 0 ? DIG_RK4_FIRST : A.stage < 3 ? DIG_RK4_MID : DIG_RK4_LAST) {
             case DIG_RK4_FIRST: pulses(std::integral_constant<int, DIG_RK4_FIRST>{}); break;
@@ -654,19 +663,20 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             default: pulses(std::integral_constant<int, DIG_TAYLOR>{});
             }
             if (!ok) break;
+            it0 += np;
             __syncwarp();
             if (lane == 0) mbar_arrive(&d_empty);
         }
-        if (threadIdx.x == 128 + 32 * DIG_DRAIN_WARPS) st_used = it;
+        if ((warp & 3) == 0 && lane == 0) st_used[grp] = it0;
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) {
         // Let copies still in flight land before the CTA's shared memory goes
         // away (a pair's copies complete on the even CTA's barriers).
         volatile int never = 0;
-        for (int q = consumed; rank == 0 && q < issued; ++q)
+        for (int q = consumed; rank == 0 && q < max(issued[0], issued[1]); ++q)
             mbar_wait_bounded(&full[q % NST], (uint32_t)((q / NST) & 1), &never, DIG_WAIT_NS);
-        for (int q = st_used; q < st_issued; ++q)
+        for (int q = min(st_used[0], st_used[1]); q < st_issued; ++q)
             mbar_wait_bounded(&st_full[q % DIG_NSU], (uint32_t)((q / DIG_NSU) & 1), &never, DIG_WAIT_NS);
         atomicOr(A.err, kErrTimeout);
     }

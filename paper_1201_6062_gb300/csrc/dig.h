@@ -36,7 +36,7 @@ struct DigArgs {
 
 // Tile of the batched product: cg CTAs share 128 cg rows, bn pulse planes.
 struct DigTile { int cg, bn; };
-DigTile dig_tile(int slices, int n, int B);
+DigTile dig_tile(int slices, int n, int lmax, int B);
 size_t dig_scratch_bytes(DigTile t);
 cudaError_t launch_dig(int slices, DigTile t, const DigMaps &m, const DigArgs &A, cudaStream_t stream);
 const void *dig_fn4(int cg, int bn);

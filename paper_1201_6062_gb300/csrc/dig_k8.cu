@@ -7,6 +7,7 @@ const void *dig_fn8(int cg, int bn)
 {
     if (cg == 1 && bn == 32) return (const void *)dig_kernel<8, 32, 1>;
     if (cg == 1 && bn == 64) return (const void *)dig_kernel<8, 64, 1>;
+    if (cg == 2 && bn == 32) return (const void *)dig_kernel<8, 32, 2>;
     if (cg == 2 && bn == 64) return (const void *)dig_kernel<8, 64, 2>;
     return nullptr;
 }
