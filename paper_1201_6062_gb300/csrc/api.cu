@@ -468,14 +468,14 @@ static tdse_status propagate_batch_tc(tdse_ctx *ctx, double *c, const double *fi
 // ------------------------------------------- digit-sliced batches (dig.cuh) --
 // Whether a batch of B pulses runs as digit-sliced products on the tensor
 // cores.  Against the FMA-pipe GEMMs (FP32, float-float) they win at every
-// measured shape (1.1x-6.7x a stage: lmax=15, n=1000, 256 pulses 546 against
-// 3645 us float-float, 388 against 945 us FP32) but short rows with many
-// pulses, where most of a 128-row tile is padding (n=40, 200 pulses: 50
-// against 36 us; n=60: 45 against 48).  FP64 batches otherwise run pulse by
-// pulse: a stage of lmax=7, n=301 takes 24 us a pulse and 70 us for 4 pulses
-// here, of lmax=15, n=1000 65 and 209 us; blocks streamed from HBM (32 bytes of
-// digits an element against 8) 335 and 1690 us at lmax=31, n=2000.  Without the
-// fixed-point copy a pulse takes 29, 152 and 1043 us.
+// measured shape (lmax=15, n=1000, 256 pulses 502 against 3645 us a stage
+// float-float, 317 against 945 us FP32) but short rows with many pulses, where
+// most of a 128-row tile is padding (FP32, n=40, 200 pulses: 40 against 36 us;
+// n=56, 300: 38).  FP64 batches otherwise run pulse by pulse: a stage of lmax=7,
+// n=301 takes 17 us a pulse and 62 us for 6 pulses here, of lmax=15, n=1000 51
+// and 202 us; blocks streamed from HBM (32 bytes of digits an element against 8)
+// 305 and 1595 us at lmax=31, n=2000.  Without the fixed-point copy a pulse takes
+// 29, 152 and 1043 us.
 static bool dig_wanted(const tdse_ctx *ctx, int B)
 {
     if (ctx->lmax < 1) return false;
@@ -839,7 +839,7 @@ static tdse_status prof_pair(tdse_ctx *c, cudaEvent_t *e0, cudaEvent_t *e1)
 
 // The block mat-vec of descriptor slot `slot` (0 forward state, 1 adjoint
 // cotangents), traced when profiling is on.
-static tdse_status launch_product(tdse_ctx *c, int slot, cudaStream_t s)
+static tdse_status launch_product(tdse_ctx *c, int slot, cudaStream_t s, bool early = true)
 {
     if (c->plan.grid <= 0) return TDSE_OK;
     const SysDesc *sys = c->sys.as<SysDesc>() + slot;
@@ -852,10 +852,10 @@ static tdse_status launch_product(tdse_ctx *c, int slot, cudaStream_t s)
     }
     if (c->plan.cfg.tma)
         CUDA_TRY(tdse::launch_mvt(c->prec, c->plan.cfg, c->plan.grid, sys, c->plan.segs.as<Seg>(),
-                                  c->plan.cta_off.as<int>(), c->errw.as<int>(), s));
+                                  c->plan.cta_off.as<int>(), c->errw.as<int>(), s, early));
     else
         CUDA_TRY(tdse::launch_mv(c->prec, c->plan.cfg, c->plan.grid, sys, c->plan.segs.as<Seg>(),
-                                 c->plan.cta_off.as<int>(), s));
+                                 c->plan.cta_off.as<int>(), s, early));
     if (traced) {
         CUDA_TRY(cudaEventRecord(e1, s));
         c->prof_products += 1;
@@ -864,11 +864,12 @@ static tdse_status launch_product(tdse_ctx *c, int slot, cudaStream_t s)
     return TDSE_OK;
 }
 
-static tdse_status mv_and_epi(tdse_ctx *c, tdse::EpiArgs a, cudaStream_t s)
+static tdse_status mv_and_epi(tdse_ctx *c, tdse::EpiArgs a, cudaStream_t s, bool early = true)
 {
-    tdse_status st = launch_product(c, 0, s);
+    tdse_status st = launch_product(c, 0, s, early);
     if (st != TDSE_OK) return st;
-    CUDA_TRY(tdse::launch_epi(c->prec, c->plan.nblk, c->plan.blk.as<int2>(), c->sys.as<SysDesc>(), a, s));
+    CUDA_TRY(tdse::launch_epi(c->prec, c->plan.nblk, c->plan.blk.as<int2>(), c->sys.as<SysDesc>(), a, s,
+                              early || c->plan.grid > 0));
     c->launches += (c->plan.nblk > 0 ? 1 : 0);
     return TDSE_OK;
 }
@@ -885,14 +886,17 @@ tdse_status tdse_hmatvec(tdse_ctx *ctx, double f, const double *x, double *y, in
     SysDesc d = ctx->desc;
     d.x = (double2 *)const_cast<double *>(x);
     d.acc = (double2 *)y;
-    tdse_status st = stage_desc(ctx, d, s);
-    if (st != TDSE_OK) return st;
-    CUDA_TRY(tdse::launch_prep(ctx->prec, ctx->plan.nblk, ctx->plan.blk.as<int2>(), ctx->sys.as<SysDesc>(), 1, s));
-    ctx->launches += 1;
+    // FP64 products read x itself; other precisions convert it first.
+    const bool direct = ctx->prec == TDSE_FP64;
+    if (direct) d.xq = d.x;
+    CUDA_TRY(tdse::launch_desc(ctx->sys.as<SysDesc>(), d, s));
+    if (!direct)
+        CUDA_TRY(tdse::launch_prep(ctx->prec, ctx->plan.nblk, ctx->plan.blk.as<int2>(), ctx->sys.as<SysDesc>(), 1, s, false));
+    ctx->launches += direct ? 1 : 2;
     tdse::EpiArgs a{};
     a.mode = scale_by_minus_i ? tdse::EPI_MIHX : tdse::EPI_HX;
     a.fval = f;
-    return mv_and_epi(ctx, a, s);
+    return mv_and_epi(ctx, a, s, !direct);
 }
 
 static tdse_status check_prop_args(tdse_ctx *ctx, const double *c, const double *field, int sps, double dt,
@@ -1015,11 +1019,8 @@ static tdse_status propagate_impl(tdse_ctx *ctx, double *c, const double *field,
     SysDesc d = ctx->desc;
     d.c = (double2 *)c;
     d.field = field;
-    tdse_status st = stage_desc(ctx, d, s);
-    if (st != TDSE_OK) return st;
     if (nsteps == 0) return TDSE_OK;
-    if (scheme == TDSE_LANCZOS) return propagate_lanczos(ctx, c, sps, dt, nsteps, order, hold, s);
-    if (tdse::small_fits(ctx->prec, ctx->lmax, ctx->n, ctx->ld, ctx->N)) {
+    if (scheme != TDSE_LANCZOS && tdse::small_fits(ctx->prec, ctx->lmax, ctx->n, ctx->ld, ctx->N)) {
         // the whole system fits in one CTA's shared memory: one launch for all steps
         tdse::SmallArgs A{};
         A.U = ctx->U.p;
@@ -1046,6 +1047,9 @@ static tdse_status propagate_impl(tdse_ctx *ctx, double *c, const double *field,
         // a cluster this size could not be placed: take the per-stage launches below
         (void)cudaGetLastError();
     }
+    tdse_status st = stage_desc(ctx, d, s);
+    if (st != TDSE_OK) return st;
+    if (scheme == TDSE_LANCZOS) return propagate_lanczos(ctx, c, sps, dt, nsteps, order, hold, s);
     CUDA_TRY(tdse::launch_prep(ctx->prec, ctx->plan.nblk, ctx->plan.blk.as<int2>(), ctx->sys.as<SysDesc>(), 0, s));
     ctx->launches += 1;
     if (step_capable(ctx)) return propagate_persistent(ctx, sps, dt, nsteps, scheme, order, hold, s);
@@ -1995,7 +1999,7 @@ static tdse_status group_step(tdse_group *g, int sps, double dt, cudaStream_t s,
                 a.stage = q;
                 tdse_status st = bucket_product(g, bk, bucket_cfg(bk), sb);
                 if (st != TDSE_OK) return st;
-                CUDA_TRY(tdse::launch_epi(g->prec, bk.nblk, bk.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, sb));
+                CUDA_TRY(tdse::launch_epi(g->prec, bk.nblk, bk.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, sb, false));
             }
             CUDA_TRY(cudaEventRecord(fork->done[b], sb));
             CUDA_TRY(cudaStreamWaitEvent(s, fork->done[b], 0));
@@ -2005,7 +2009,7 @@ static tdse_status group_step(tdse_group *g, int sps, double dt, cudaStream_t s,
             a.stage = q;
             tdse_status st = group_product(g, s);
             if (st != TDSE_OK) return st;
-            CUDA_TRY(tdse::launch_epi(g->prec, g->plan.nblk, g->plan.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, s));
+            CUDA_TRY(tdse::launch_epi(g->prec, g->plan.nblk, g->plan.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, s, false));
         }
     }
     CUDA_TRY(tdse::launch_bump(g->kdev.as<long long>(), s));

@@ -26,20 +26,22 @@
 // CTAs (one TPC) shares a 256-row tile, each loading its own rows of A and half
 // of B, which takes the operand traffic of an SM from 73 to 55 bytes per tensor
 // cycle (L2) and from 128 to 96 (shared memory reads; 128 is what it delivers).
-// CG = 1 serves blocks of at most 128 rows and small batches.
+// CG = 1 serves blocks of at most 128 rows.
 //
-// Warp 0 streams digit tiles with TMA, one thread of warp 1 issues the MMAs,
-// two warpgroups drain the accumulators into per-thread running sums, and a
-// fourth applies the FP64 stage update while they are at the next tile: the
+// Warps 0 and 3 stream the digit tiles with TMA, one thread of warp 1 issues the
+// MMAs, two warpgroups drain the accumulators into per-thread running sums, and
+// two more apply the FP64 stage update while they are at the next tile: the
 // update is bound by the FP64 pipe (2 operations per cycle and SM; 8-10 per
 // amplitude here), and run by the draining warps it stalled the products.
 // Measured on GB300, one stage of 256 pulses, lmax=15, n=1000 (31 GFLOP of real
-// products): float-float 3645 (FMA pipe, bgemm_df.cu) -> 546 us, FP32 945
-// (batch.cu) -> 388 us; FP64, 24 pulses, lmax=7, n=301: 692 (pulse by pulse) ->
-// 89 us.  21 products at the bf16 rate of 1927 TFLOP/s would take 334 us.  Of the
-// way there: 128-row tiles of single CTAs updated by the draining warps 1305 us,
-// pairs with updating warps 898, the whole-warp issue loop (elect_one) 603,
-// states by bulk copies 560.
+// products): float-float 3645 (FMA pipe, bgemm_df.cu) -> 502 us, FP32 945
+// (batch.cu) -> 317 us; FP64, 24 pulses, lmax=7, n=301: 692 (pulse by pulse) ->
+// 68 us.  21 products at the bf16 rate of 1927 TFLOP/s would take 334 us.  Of the
+// way there (float-float): 128-row tiles of single CTAs updated by the draining
+// warps 1305 us, pairs with updating warps 898, the whole-warp issue loop
+// (elect_one) 603, states by bulk copies 560, eight updating warps 509.  What is
+// left: a step (24 KB of operands a CTA) takes 620 cycles against 448 of products,
+// 40 bytes a cycle and SM out of L2.
 // All waits are bounded (sync.cuh).
 #pragma once
 #include <type_traits>

@@ -26,7 +26,8 @@ cudaError_t ensure_dyn_smem(const void *fn, int bytes);
 
 // Launch with programmatic stream serialization (the kernel calls pdl_wait()
 // before reading what earlier kernels wrote).
-cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, void **args);
+cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, void **args,
+                       bool early = true);
 
 // prec: 0 FP64, 1 FP32, 2 DF32 (tdse_precision values).
 bool mv_config(int prec, int n, MvCfg *out);
@@ -58,7 +59,7 @@ bool mvt_use_fixed(int prec, int n, bool streamed, MvCfg *cfg);
 // Whether `rs` rows per stage fit the ring for rows of `ld` elements.
 bool mvt_rs_valid(int prec, const MvCfg &cfg, int rs, int ld);
 cudaError_t launch_mvt(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,
-                       const int *cta_off, int *err, cudaStream_t stream);
+                       const int *cta_off, int *err, cudaStream_t stream, bool early = true);
 
 // Persistent stepping of one system (mvt.cuh, STEP instances): `passes` block
 // products in one cooperative launch, each followed by a grid barrier, the
@@ -107,7 +108,7 @@ cudaError_t launch_mvt_step(int prec, const MvCfg &cfg, int grid, const SysDesc 
 
 // Block mat-vec over a segment list: R = U_l x_{l+1} rows, P = column partials.
 cudaError_t launch_mv(int prec, const MvCfg &cfg, int grid, const SysDesc *sys,
-                      const Seg *segs, const int *cta_off, cudaStream_t stream);
+                      const Seg *segs, const int *cta_off, cudaStream_t stream, bool early = true);
 
 // Epilogue modes.
 enum EpiMode { EPI_HX = 0, EPI_MIHX = 1, EPI_RK4 = 2, EPI_TAYLOR = 3 };
@@ -132,8 +133,8 @@ struct EpiArgs {
 };
 // *kdev += 1 (one thread): advances the step index of a captured step graph.
 cudaError_t launch_bump(long long *kdev, cudaStream_t stream);
-cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys,
-                       EpiArgs a, cudaStream_t stream);
+cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream,
+                       bool early = true);
 
 // --- adjoint (adj.cu) ---
 // A pending scalar: the sum of parts[0..n) (fixed order) is added, times w0 and
@@ -171,7 +172,8 @@ cudaError_t launch_flush(Flush f, cudaStream_t stream);
 
 // xq = compute-format copy of c (the first product's input).
 cudaError_t launch_prep(int prec, int nblk, const int2 *blk, const SysDesc *sys,
-                        int from_x, cudaStream_t stream);
+                        int from_x, cudaStream_t stream, bool early = true);
+cudaError_t launch_desc(SysDesc *out, const SysDesc &d, cudaStream_t stream);
 
 // Populations: per (b, l): sum |c|^2, bound part, ionised part.
 //   part [B][L][3] scratch; then totals.

@@ -250,29 +250,34 @@ int mv_ctas_per_sm(int prec, const MvCfg &cfg)
 }
 
 cudaError_t launch_mv(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,
-                      const int *cta_off, cudaStream_t stream)
+                      const int *cta_off, cudaStream_t stream, bool early)
 {
     const void *fn = mv_fn_prec(prec, cfg.idx);
     if (!fn) return cudaErrorInvalidValue;
     if (grid <= 0) return cudaSuccess;
     void *args[] = {(void *)&sys, (void *)&segs, (void *)&cta_off};
-    return launch_pdl(fn, dim3(grid), dim3(cfg.BT), 0, stream, args);
+    return launch_pdl(fn, dim3(grid), dim3(cfg.BT), 0, stream, args, early);
 }
 
 // ----------------------------------------------------------- epilogue --
 // Per amplitude a = (m, i):  D x = R[a] (m < lmax) + sum of the column
 // partial slots of block m-1 (m >= 1), in slot order;  then H x = E x + f D x
 // and the stage / term update of the chosen scheme, all in FP64.
+// Four blocks of 64 amplitudes, two threads each, per entry of blk: bound by the
+// latency of the FP64 instructions, of which an SM completes one a warp in 16
+// cycles, so few amplitudes an SM.  FP32, lmax=28, n=108, us a stage with its
+// product: 12.7 with a thread an amplitude and 256 a block, 11.3 so; lmax=6,
+// n=300 12.0 and 10.2 (two threads each but 256 amplitudes a block: 11.6).
 template <class P>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(128, 8)                // (without the 8, 40 registers: the slots read one by one)
 epi_kernel(const SysDesc *__restrict__ sys, const int2 *__restrict__ blk, EpiArgs A)
 {
     pdl_launch_dependents();
     // The plan, the descriptor, the energies and the slot ranges are the same
     // for every launch of a call: read them before waiting for the product.
-    const int2 bm = blk[blockIdx.x];
+    const int2 bm = blk[blockIdx.x >> 2];
     const SysDesc S = sys[bm.x];
-    const long long a = (long long)bm.y + (threadIdx.x >> 1);
+    const long long a = (long long)bm.y + (((blockIdx.x & 3) * 128 + threadIdx.x) >> 1);
     const int own = threadIdx.x & 1;
     const bool live = a < S.N;
     const EpiPre pre = live ? epi_pre(S, a) : EpiPre{};
@@ -335,7 +340,7 @@ cudaError_t ensure_dyn_smem(const void *fn, int bytes)
     return e;
 }
 
-cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, void **args)
+cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, void **args, bool early)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -346,11 +351,15 @@ cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaS
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream)
+// early: start while the product still runs.  Not for groups of systems, whose
+// products (of several streams, or several CTAs an SM) lack the room that the
+// waiting blocks take (FP32, us for 4 steps: 12 systems 1087 early, 1019 not; 6
+// systems 460 and 420).
+cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream, bool early)
 {
     if (nblk <= 0) return cudaSuccess;
     const void *fn = nullptr;
@@ -363,7 +372,7 @@ cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, 
     if (a.mode == EPI_RK4) a.s = a.stage == 3 ? a.dt / 6.0 : (a.stage == 2 ? a.dt : 0.5 * a.dt);
     else if (a.mode == EPI_TAYLOR) a.s = a.dt / (double)a.stage;
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&a};
-    return launch_pdl(fn, dim3(nblk), dim3(512), 0, stream, args);       // two threads per amplitude, 256 per block
+    return launch_pdl(fn, dim3(4 * nblk), dim3(128), 0, stream, args, early);
 }
 
 __global__ void bump_kernel(long long *kdev) { *kdev += 1; }
@@ -374,7 +383,7 @@ cudaError_t launch_bump(long long *kdev, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-cudaError_t launch_prep(int prec, int nblk, const int2 *blk, const SysDesc *sys, int from_x, cudaStream_t stream)
+cudaError_t launch_prep(int prec, int nblk, const int2 *blk, const SysDesc *sys, int from_x, cudaStream_t stream, bool early)
 {
     if (nblk <= 0) return cudaSuccess;
     const void *fn = nullptr;
@@ -385,7 +394,19 @@ cudaError_t launch_prep(int prec, int nblk, const int2 *blk, const SysDesc *sys,
     default: return cudaErrorInvalidValue;
     }
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&from_x};
-    return launch_pdl(fn, dim3(nblk), dim3(256), 0, stream, args);
+    return launch_pdl(fn, dim3(nblk), dim3(256), 0, stream, args, early);
+}
+
+// A call's descriptor, by value: a copy from pinned memory and the event that
+// guards it take 2-3 us before a product, and a captured copy would read what
+// a later call left there.  Whatever reads it starts after this kernel has
+// ended (early = false), as products read it before they wait.
+__global__ void desc_kernel(SysDesc *out, const __grid_constant__ SysDesc d) { *out = d; }
+
+cudaError_t launch_desc(SysDesc *out, const SysDesc &d, cudaStream_t stream)
+{
+    desc_kernel<<<1, 1, 0, stream>>>(out, d);
+    return cudaGetLastError();
 }
 
 }  // namespace tdse

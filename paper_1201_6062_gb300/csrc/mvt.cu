@@ -103,7 +103,7 @@ int mvt_ctas_per_sm(int prec, const MvCfg &cfg)
 }
 
 cudaError_t launch_mvt(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,
-                       const int *cta_off, int *err, cudaStream_t stream)
+                       const int *cta_off, int *err, cudaStream_t stream, bool early)
 {
     const void *fn = mvt_fn_prec(prec, cfg, cfg.RS);
     if (!fn || cfg.ld <= 0) return cudaErrorInvalidValue;
@@ -118,7 +118,7 @@ cudaError_t launch_mvt(int prec, const MvCfg &cfg, int grid, const SysDesc *sys,
     StepArgs none{};
     none.passes = 1;
     void *args[] = {(void *)&sys, (void *)&segs, (void *)&cta_off, (void *)&err, (void *)&stage, (void *)&none};
-    return launch_pdl(fn, dim3(grid), dim3(cfg.BT), (size_t)smem, stream, args);
+    return launch_pdl(fn, dim3(grid), dim3(cfg.BT), (size_t)smem, stream, args, early);
 }
 
 // Dynamic shared memory of a launch: one CTA per SM requests the whole ring

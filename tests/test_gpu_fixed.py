@@ -147,3 +147,31 @@ def test_without_room_for_the_copy_the_fp64_kernel_serves(tdse_lib):
             assert np.linalg.norm(c.cpu().numpy() - ref) < 1e-12
     H.close()
     H2.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-14), ("df32", 1e-11), ("fp32", 2e-6)])
+@pytest.mark.parametrize("lmax,n", [(0, 70), (3, 40), (4, 301)])
+def test_products_queued_without_a_wait(tdse_lib, lmax, n, prec, tol):
+    """Products of different vectors queued one behind the other, and one
+    recorded in a graph and replayed after another call: each reads the
+    vectors it was called with.  Tolerances: the products' (fp64: 2^-53 times
+    the square root of the terms of a sum)."""
+    rng = np.random.default_rng(3)
+    E, U = inputs.energies(lmax, n), rng.standard_normal((lmax, n, n)) / n ** 0.5
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, prec)
+    X = rng.standard_normal((4, (lmax + 1) * n, 2)).view(np.complex128)[..., 0]
+    x = torch.from_numpy(X.copy()).cuda()
+    y = torch.zeros_like(x)
+    for i in range(3):
+        H.hmatvec(x[i], 0.3, y=y[i])
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        H.hmatvec(x[3], 0.3, y=y[3])
+    H.hmatvec(x[0], 0.3, y=y[0])
+    g.replay()
+    torch.cuda.synchronize()
+    for i in range(4):
+        ref = oracle.hmatvec(lmax, n, E, U, 0.3, X[i])
+        assert np.linalg.norm(y[i].cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
+    H.close()
