@@ -81,6 +81,14 @@ __global__ void __launch_bounds__(256) lz_init(const SysDesc *__restrict__ sys, 
     P::store_xq(S.xq, a, v);
 }
 
+// The vector kernels are bound by the latency of loads and block sums and by the
+// FP64 pipe, which takes 16 cycles a warp instruction and SM.  So one thread takes
+// the root and the reciprocal (some 40 FP64 instructions, formerly in every warp),
+// and lz_orth requests its vectors before it sums the partials.  Product and both
+// kernels, us a Krylov vector: FP32, lmax=31, n=2000 116.4 -> 109.0; float-float,
+// lmax=15, n=500 46.4 -> 43.0 (with D x's slots eight at a time and its loads ahead
+// of the sum in lz_apply too: 113.1 and 50.1).
+//
 // j = 0: x = v_0.  j > 0: b_j = |w| from the partials of lz_orth, x = v_j =
 // w / b_j (stored; zero after a breakdown), and the block products, taken of
 // the unnormalised w, are scaled by 1 / b_j.  Then w = H(f) x and the
@@ -89,16 +97,21 @@ __global__ void __launch_bounds__(256) lz_apply(const SysDesc *__restrict__ sys,
                                                 double2 *__restrict__ w, LzArgs A, const double *__restrict__ parts_b,
                                                 int nparts, double *__restrict__ scal, double *__restrict__ parts_a)
 {
-    __shared__ double sh[9];
+    __shared__ double sh[10];
     pdl_launch_dependents();
     pdl_wait();
     const SysDesc &S = sys[0];
     double inv = 1.0;
     if (j > 0) {
-        const double b = sqrt(lz_sum_parts(parts_b, nparts, sh));
-        const bool brk = !(b > 1e-300);
-        if (blockIdx.x == 0 && threadIdx.x == 0) scal[1 + 64 + j] = brk ? 0.0 : b;
-        inv = brk ? 0.0 : 1.0 / b;
+        const double ss = lz_sum_parts(parts_b, nparts, sh);
+        if (threadIdx.x == 0) {
+            const double b = sqrt(ss);
+            const bool brk = !(b > 1e-300);
+            if (blockIdx.x == 0) scal[1 + 64 + j] = brk ? 0.0 : b;
+            sh[9] = brk ? 0.0 : 1.0 / b;
+        }
+        __syncthreads();
+        inv = sh[9];
     }
     const long long a = (long long)blockIdx.x * 256 + threadIdx.x;
     double v = 0.0;
@@ -134,18 +147,22 @@ __global__ void __launch_bounds__(256) lz_orth(const SysDesc *__restrict__ sys, 
     pdl_launch_dependents();
     pdl_wait();
     const SysDesc &S = sys[0];
-    const double alpha = lz_sum_parts(parts_a, nparts, sh);
-    const double beta = j > 0 ? scal[1 + 64 + j] : 0.0;      // b_j
-    if (blockIdx.x == 0 && threadIdx.x == 0) scal[1 + j] = alpha;
     const long long a = (long long)blockIdx.x * 256 + threadIdx.x;
+    const bool live = a < S.N;
+    double2 x = make_double2(0.0, 0.0), ww = x, y = x;
+    if (live) {
+        x = vj[a];
+        ww = w[a];
+        if (j > 0) y = vjm1[a];
+    }
+    const double beta = j > 0 ? scal[1 + 64 + j] : 0.0;      // b_j
+    const double alpha = lz_sum_parts(parts_a, nparts, sh);
+    if (blockIdx.x == 0 && threadIdx.x == 0) scal[1 + j] = alpha;
     double v = 0.0;
-    if (a < S.N) {
-        const double2 x = vj[a];
-        double2 ww = w[a];
+    if (live) {
         ww.x -= alpha * x.x;
         ww.y -= alpha * x.y;
         if (j > 0) {
-            const double2 y = vjm1[a];
             ww.x -= beta * y.x;
             ww.y -= beta * y.y;
         }
