@@ -73,8 +73,13 @@ constexpr int DIG_NONFINITE = 0x7ff00000;               // xmax / eu mark of a n
 
 __host__ __device__ constexpr int dig_stage_bytes(int bn, int cg) { return DA_BYTES + bn / cg * DBK * 2; }
 __host__ __device__ constexpr int dig_stages(int bn, int cg) { return 196608 / dig_stage_bytes(bn, cg); }
-// Behind the operand ring: DIG_NSU slots of the states (c, x, acc) of one pulse and the tile's rows.
-constexpr int DIG_NSU = 5, DIG_SLOT = 3 * DBM * 16;
+// Behind the operand ring: DIG_NSU slots of the states (c, x, acc) of one pulse and the tile's rows, which
+// DIG_UPD_GROUPS groups of updating warps take in turn.  A wait by parity tells a phase from the one before
+// only, so a waiter must have seen every phase of its barrier: with a multiple of the groups a slot stays
+// with one group within a tile, and the next tile starts (d_full) when both have finished (d_empty).
+constexpr int DIG_NSU = 4, DIG_SLOT = 3 * DBM * 16;
+constexpr int DIG_UPD_GROUPS = 2;
+static_assert(DIG_NSU % DIG_UPD_GROUPS == 0 && DIG_UPD_GROUPS == 2, "a state slot must not change hands within a tile");
 __host__ __device__ constexpr int dig_smem(int bn, int cg)
 {
     return dig_stages(bn, cg) * dig_stage_bytes(bn, cg) + DIG_NSU * DIG_SLOT + 1024;
@@ -260,7 +265,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
     __shared__ int issued[2], consumed;
-    __shared__ int st_issued, st_used[2];
+    __shared__ int st_issued, st_used[DIG_UPD_GROUPS];
     unsigned char *slots = smem + (size_t)NST * STAGE;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform)
@@ -285,7 +290,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         mbar_init(&d_empty, DIG_UPD_WARPS);
         for (int q = 0; q < DIG_NSU; ++q) {
             mbar_init(&st_full[q], 1);
-            mbar_init(&st_empty[q], DIG_UPD_WARPS / 2);
+            mbar_init(&st_empty[q], DIG_UPD_WARPS / DIG_UPD_GROUPS);
         }
         mbar_init(&mma_drain, 1);
         st_issued = 0;
@@ -607,10 +612,10 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                     int mine = 0;
                     const int pe = min(p32 + 32, np);
 #pragma unroll 1
-                    for (int p = p32 + grp; p < pe; p += 2) {
+                    for (int p = p32 + grp; p < pe; p += DIG_UPD_GROUPS) {
                         DigOut o;
                         o.f = nx.f;
-                        nx.f = scr[min(p + 2, BN / 2 - 1) * DBM].f;
+                        nx.f = scr[min(p + DIG_UPD_GROUPS, BN / 2 - 1) * DBM].f;
                         const int it = it0 + p, s = it % DIG_NSU;
                         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&st_full[s], (uint32_t)((it / DIG_NSU) & 1), abort, DIG_WAIT_NS)) != 0;
                         if (!ok) return;
