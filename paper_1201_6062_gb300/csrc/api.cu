@@ -99,8 +99,8 @@ struct DevBuf {
     template <class T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
-// Whether memory a call can do without (a second form of the dipole blocks for
-// a faster kernel) may be taken: at most an eighth of what the device and the
+// Whether memory a call can do without (the digits of the dipole blocks for
+// the batched products) may be taken: at most an eighth of what the device and the
 // cap leave, so that allocations that are needed rarely meet it; one that does
 // gets it back (with_room).
 static bool optional_room(size_t nbytes)
@@ -131,8 +131,6 @@ struct tdse_ctx {
     int lmax = 0, n = 0, N = 0, ld = 0, prec = 0;
     long long bstride = 0;
     DevBuf U, E, R, P, x, acc, xq, sb, sys, umax;
-    DevBuf Uf, ue;                     // FP64: fixed-point copy of U and its exponents (create_fixed)
-    bool in_group = false;             // a group's descriptors may point at them
     DevBuf part;                       // populations scratch
     DevBuf errw;                       // device status word (kErrTimeout, ...)
     DevBuf hc, hfield;                 // device copies for the host-buffer entry point
@@ -198,8 +196,7 @@ static int sm_count()
 
 // Build the mat-vec plan for the given systems and upload it.
 static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std::vector<int> &n, MvPlan &mp,
-                              tdse::Plan &plan, const std::vector<int> *global_id = nullptr, int layout = -1,
-                              bool fixed = false)
+                              tdse::Plan &plan, const std::vector<int> *global_id = nullptr, int layout = -1)
 {
     int nmax = 1;
     long long rows = 0, amps = 0;
@@ -218,10 +215,8 @@ static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std:
         // more CTAs only add column-partial slots and per-CTA overhead.
         long long ubytes = 0;
         for (size_t q = 0; q < n.size(); ++q) ubytes += (long long)lmax[q] * n[q] * n[q] * elem_bytes(prec);
-        const bool streamed = ubytes >= (64LL << 20);
         mp.cfg.per_sm = 1;
-        if (fixed) (void)tdse::mvt_use_fixed(prec, nmax, streamed, &mp.cfg);
-        if (streamed) {
+        if (ubytes >= (64LL << 20)) {
             // Rows per stage and resident CTAs trade against each other (a
             // deeper stage needs more registers, which can leave room for
             // fewer CTAs): take the depth with the most rows in flight per SM,
@@ -247,9 +242,9 @@ static tdse_status build_plan(int prec, const std::vector<int> &lmax, const std:
     // (its x_{l+1} columns, the |x| bounds of the offset sums, one more
     // partial slot to write): measured at about 8 rows of a float-float
     // product with 500-element rows (FP32 products, with the same offset
-    // sums, are charged alike), 1 row of an FP64 one and 6 rows of a
-    // fixed-point one.  Charged only when CTAs get enough rows for it to matter.
-    const int seg_rows = mp.cfg.fix ? (rows >= 8LL * G ? 6 : 0) : rows >= 16LL * G ? (prec == TDSE_FP64 ? 1 : 8) : 0;
+    // sums, are charged alike) and 1 row of an FP64 one.  Charged only when
+    // CTAs get enough rows for it to matter.
+    const int seg_rows = rows >= 16LL * G ? (prec == TDSE_FP64 ? 1 : 8) : 0;
     tdse::make_plan(G, lmax, n, 32, plan, seg_rows);
     mp.grid = rows > 0 ? G : 0;
     std::vector<Seg> segs(plan.segs.size());
@@ -472,63 +467,11 @@ static tdse_status propagate_batch_tc(tdse_ctx *ctx, double *c, const double *fi
 // float-float, 317 against 945 us FP32) but short rows with many pulses, where
 // most of a 128-row tile is padding (FP32, n=40, 200 pulses: 40 against 36 us;
 // n=56, 300: 38).  FP64 batches otherwise run pulse by pulse: a stage of lmax=7,
-// n=301 takes 17 us a pulse and 62 us for 6 pulses here, of lmax=15, n=1000 51
-// and 202 us; blocks streamed from HBM (32 bytes of digits an element against 8)
-// 305 and 1595 us at lmax=31, n=2000.  Without the fixed-point copy a pulse takes
-// 29, 152 and 1043 us.
+// n=301 takes 24 us a pulse and 62 us for 6 pulses here.
 static bool dig_wanted(const tdse_ctx *ctx, int B)
 {
     if (ctx->lmax < 1) return false;
-    if (ctx->prec != TDSE_FP64) return ctx->n >= 56 || B <= 32;
-    if (!ctx->Uf.p) return B >= 3;
-    return B >= ((long long)ctx->lmax * ctx->n * ctx->n * 8 >= (64LL << 20) ? 6 : 4);
-}
-
-// Fixed-point copy of an FP64 context's dipole blocks for the integer products
-// of the ring kernel (PolI64, 305 us a stage of lmax=31, n=2000 against the FP64
-// kernel's 1043).  Not made, and the FP64 kernel kept, for short rows (mv.cu),
-// rows beyond the fixed-point layouts, blocks with a non-finite element or a nonzero row or column whose largest element is below
-// 2^-6 of the block's (58 bits of the block's scale would leave it fewer than
-// 53 of its own), or when the memory for it cannot be had.
-static tdse_status create_fixed(tdse_ctx *c)
-{
-    const int n = c->n, lmax = c->lmax;
-    tdse::MvCfg cfg{};
-    if (!tdse::mvt_config(TDSE_FP64, n, c->ld, &cfg) || !tdse::mvt_use_fixed(TDSE_FP64, n, false, &cfg)) return TDSE_OK;
-    const size_t count = 2 * (size_t)lmax * n;
-    const size_t ubytes = (size_t)lmax * (size_t)c->bstride * 8;
-    if (!optional_room(ubytes)) return TDSE_OK;
-    if (c->ue.ensure(sizeof(int) * count) != cudaSuccess || c->Uf.ensure(ubytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        c->ue.release();
-        c->Uf.release();
-        return TDSE_OK;
-    }
-    CUDA_TRY(tdse::launch_fix_maxima(c->U.as<double>(), c->bstride, c->ld, n, lmax, c->ue.as<int>(), 0));
-    std::vector<int> h(count), e((size_t)lmax);
-    CUDA_TRY(cudaMemcpy(h.data(), c->ue.p, sizeof(int) * count, cudaMemcpyDeviceToHost));
-    bool ok = true;
-    for (int l = 0; l < lmax && ok; ++l) {
-        int m = 0;
-        for (int i = 0; i < n; ++i) m = std::max(m, h[(size_t)l * n + i]);
-        ok = m < 0x7ff00000;
-        for (int i = 0; i < n && ok; ++i)
-            for (int q = 0; q < 2; ++q) {
-                const int v = h[((size_t)q * lmax + l) * n + i];
-                ok = ok && (v == 0 || (v >> 20) >= (m >> 20) - 6);
-            }
-        e[(size_t)l] = std::max(m >> 20, 1) - 1022;
-    }
-    if (!ok) {
-        c->ue.release();
-        c->Uf.release();
-        return TDSE_OK;
-    }
-    CUDA_TRY(cudaMemcpy(c->ue.p, e.data(), sizeof(int) * e.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemset(c->Uf.p, 0, ubytes));
-    CUDA_TRY(tdse::launch_fix(c->U.as<double>(), c->bstride, (long long)n * c->ld, lmax, c->ue.as<int>(), c->Uf.p, 0));
-    CUDA_TRY(cudaDeviceSynchronize());
-    return TDSE_OK;
+    return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
 }
 
 // Device storage, dipole digits and tensor maps of a digit-sliced batch; false
@@ -584,46 +527,16 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
     return ok;
 }
 
-// Work split, column-partial slots and slot starts of a context's own products.
-static tdse_status plan_context(tdse_ctx *c)
-{
-    tdse::Plan plan;
-    tdse_status st = build_plan(c->prec, std::vector<int>{c->lmax}, std::vector<int>{c->n}, c->plan, plan, nullptr, -1,
-                                c->Uf.p != nullptr);
-    if (st != TDSE_OK) return st;
-    c->nslots = plan.nslots[0];
-    CUDA_TRY(c->P.ensure(sizeof(double2) * (size_t)(c->nslots > 0 ? c->nslots : 1) * c->n));
-    CUDA_TRY(c->sb.ensure(sizeof(int) * (c->lmax + 1)));
-    CUDA_TRY(cudaMemcpy(c->sb.p, plan.sb[0].data(), sizeof(int) * (c->lmax + 1), cudaMemcpyHostToDevice));
-    c->step_ok = -1;
-    SysDesc &d = c->desc;
-    d.P = c->P.as<double2>();
-    d.sb = c->sb.as<int>();
-    d.Uf = c->Uf.p;
-    d.ue = c->ue.as<int>();
-    return TDSE_OK;
-}
-
-// Gives back the memory a context could do without (the fixed-point copy and
-// the digits of its dipole blocks, which the slower kernels do not need);
-// false if it holds none.
+// Gives back the memory a context could do without (the digits of its dipole
+// blocks, which the slower kernels do not need); false if it holds none.
 static bool shed(tdse_ctx *c)
 {
-    const bool digits = c->dgU.p != nullptr, copy = c->Uf.p != nullptr && !c->in_group;
-    if (!digits && !copy) return false;
-    if (cudaDeviceSynchronize() != cudaSuccess) return false;
-    if (digits) {
-        c->dgU.release();
-        c->dgE.release();
-        c->dgX.release();
-        c->dg_ready = false;
-        c->dg_B = 0;
-    }
-    if (copy) {
-        c->Uf.release();
-        c->ue.release();
-        return plan_context(c) == TDSE_OK;
-    }
+    if (!c->dgU.p || cudaDeviceSynchronize() != cudaSuccess) return false;
+    c->dgU.release();
+    c->dgE.release();
+    c->dgX.release();
+    c->dg_ready = false;
+    c->dg_B = 0;
     return true;
 }
 
@@ -768,29 +681,18 @@ tdse_status tdse_create(const double *energies, const double *dipole_blocks, int
         CTRY(c->umax.ensure(sizeof(float) * um.size()));
         CTRY(cudaMemcpy(c->umax.p, um.data(), sizeof(float) * um.size(), cudaMemcpyHostToDevice));
     }
-    if (prec == TDSE_FP64 && lmax > 0) {
-        st = create_fixed(c);
-        if (st != TDSE_OK) return bail(st);
-    }
-    st = plan_context(c);
-    if (st == TDSE_ENOMEM && c->Uf.p) {
-        (void)cudaGetLastError();
-        c->Uf.release();
-        c->ue.release();
-        st = plan_context(c);
-    }
+    tdse::Plan plan;
+    st = build_plan(prec, std::vector<int>{lmax}, std::vector<int>{n}, c->plan, plan);
     if (st != TDSE_OK) return bail(st);
-    const auto vectors = [c]() -> cudaError_t {
-        cudaError_t e = c->R.ensure(sizeof(double2) * c->N);
-        if (e == cudaSuccess) e = c->x.ensure(sizeof(double2) * c->N);
-        if (e == cudaSuccess) e = c->acc.ensure(sizeof(double2) * c->N);
-        if (e == cudaSuccess) e = c->xq.ensure((size_t)16 * c->N);
-        if (e == cudaSuccess) e = c->errw.ensure(sizeof(int));
-        return e == cudaSuccess ? c->sys.ensure(2 * sizeof(SysDesc)) : e;
-    };
-    if (vectors() == cudaErrorMemoryAllocation && c->Uf.p && !shed(c)) return bail(TDSE_ENOMEM);
-    CTRY(vectors());
+    c->nslots = plan.nslots[0];
+    CTRY(c->R.ensure(sizeof(double2) * c->N));
     CTRY(cudaMemset(c->R.p, 0, sizeof(double2) * c->N));
+    CTRY(c->P.ensure(sizeof(double2) * (size_t)(c->nslots > 0 ? c->nslots : 1) * n));
+    CTRY(c->x.ensure(sizeof(double2) * c->N));
+    CTRY(c->acc.ensure(sizeof(double2) * c->N));
+    CTRY(c->xq.ensure((size_t)16 * c->N));
+    CTRY(c->sb.ensure(sizeof(int) * (lmax + 1)));
+    CTRY(cudaMemcpy(c->sb.p, plan.sb[0].data(), sizeof(int) * (lmax + 1), cudaMemcpyHostToDevice));
     CTRY(c->sys.ensure(2 * sizeof(SysDesc)));
     CTRY(c->errw.ensure(sizeof(int)));
     CTRY(cudaMemset(c->errw.p, 0, sizeof(int)));
@@ -799,7 +701,7 @@ tdse_status tdse_create(const double *energies, const double *dipole_blocks, int
 #undef CTRY
     SysDesc &d = c->desc;
     d.U = c->U.p; d.bstride = c->bstride; d.ld = c->ld; d.n = n; d.lmax = lmax; d.N = c->N;
-    d.E = c->E.as<double>(); d.R = c->R.as<double2>();
+    d.E = c->E.as<double>(); d.R = c->R.as<double2>(); d.P = c->P.as<double2>(); d.sb = c->sb.as<int>();
     d.umax = c->umax.as<float>();
     d.c = nullptr; d.x = c->x.as<double2>(); d.acc = c->acc.as<double2>(); d.xq = c->xq.p; d.field = nullptr;
     *out = c;
@@ -1781,9 +1683,7 @@ static tdse_status bucket_plan(tdse_group *g, GroupBucket &bk)
     std::vector<int> blm, bnn;
     for (int i : bk.members) { blm.push_back(g->sys[i]->lmax); bnn.push_back(g->sys[i]->n); }
     tdse::Plan plan;
-    bool fixed = true;
-    for (int i : bk.members) fixed = fixed && g->sys[i]->Uf.p != nullptr;
-    tdse_status st = build_plan(g->prec, blm, bnn, bk.plan, plan, &bk.members, bk.layout, fixed);
+    tdse_status st = build_plan(g->prec, blm, bnn, bk.plan, plan, &bk.members, bk.layout);
     if (st != TDSE_OK) return st;
     for (size_t k = 0; k < bk.members.size(); ++k) {
         const int i = bk.members[k];
@@ -1813,9 +1713,7 @@ static tdse_status group_persistent_plan(tdse_group *g)
     std::vector<int> lm(count), nn(count), ids(count);
     for (int i = 0; i < count; ++i) { lm[i] = g->sys[i]->lmax; nn[i] = g->sys[i]->n; ids[i] = i; }
     tdse::Plan plan;
-    bool fixed = true;
-    for (int i = 0; i < count; ++i) fixed = fixed && g->sys[i]->Uf.p != nullptr;
-    tdse_status st = build_plan(g->prec, lm, nn, g->pplan, plan, &ids, g->playout, fixed);
+    tdse_status st = build_plan(g->prec, lm, nn, g->pplan, plan, &ids, g->playout);
     if (st != TDSE_OK) return st;
     if (!g->pplan.cfg.tma || g->pplan.grid <= 0)
         return fail(TDSE_ENOTSUP, "one launch for the group needs rows long enough for the bulk-copy ring");
@@ -1869,7 +1767,6 @@ tdse_status tdse_group_create(tdse_ctx *const *systems, int count, tdse_group **
     auto bail = [&](tdse_status st) { delete g; return st; };
     g->sys.assign(systems, systems + count);
     g->prec = systems[0]->prec;
-    for (int i = 0; i < count; ++i) systems[i]->in_group = true;
     std::vector<int> lm(count), nn(count);
     for (int i = 0; i < count; ++i) { lm[i] = systems[i]->lmax; nn[i] = systems[i]->n; }
     // The epilogue and prep block map over all systems (its product plan is not used).

@@ -33,8 +33,6 @@ struct SysDesc {
     double2 *c, *x, *acc;
     void *xq;
     const double *field;
-    const void *Uf;         // FP64 systems: U as 58-bit fixed point (PolI64), same strides; NULL: none
-    const int *ue;          // [lmax]: its exponents, |U_l| < 2^ue
     int gauge;              // 0: length gauge, D = U-blocks (real symmetric);
                             // 1: velocity gauge, D = i K with K antisymmetric (Sec. 5)
 };
@@ -106,7 +104,6 @@ __device__ __forceinline__ double shfl_xor_d(double v, int m)
 // FP64 products: U stored as double, 2 columns per 16-byte load.
 struct PolF64 {
     static constexpr int CW = 2;
-    static constexpr bool kFixed = false;        // (PolI64 only)
     static constexpr bool kOffsetSums = false;   // plain accumulators
     using Elem = double;
     using Uv = double;
@@ -185,7 +182,6 @@ struct PolF64 {
 // FP32 products: U stored as float, 4 columns per 16-byte load.
 struct PolF32 {
     static constexpr int CW = 4;
-    static constexpr bool kFixed = false;        // (PolI64 only)
     static constexpr bool kOffsetSums = false;
     using Elem = float;
     using Uv = float;
@@ -263,7 +259,6 @@ struct PolF32 {
 // 16-byte load; x as (re.hi, re.lo, im.hi, im.lo).
 struct PolDF32 {
     static constexpr int CW = 2;
-    static constexpr bool kFixed = false;        // (PolI64 only)
     static constexpr bool kOffsetSums = true;    // offset accumulators need bounds on |x|
     using Elem = float2;
     using Uv = df;
@@ -383,175 +378,6 @@ struct PolDF32 {
     {
         const df r = df_from_double(v);
         reinterpret_cast<float2 *>(xq)[2 * a + comp] = make_float2(r.h, r.l);
-    }
-};
-
-// FP64-accurate products in integer arithmetic, for the ring kernel.
-//
-// GB300 has 2 FP64 multiply-adds per cycle and SM, and 32 x 32 + 64 bit
-// integer ones at 25 (measured, 16 warps).  A block U_l and the stage input it meets are
-// scaled by powers of two and held as 58-bit integers
-//     u = 2^(ue-58) (uh 2^29 + ul),  |uh| <= 2^29, |ul| <= 2^28
-// (half a unit is 2^-59 of the block's largest element).  A product adds
-// uh xh to one 64-bit sum and uh xl + ul xh to another, three multiply-adds;
-// ul xl, below 2^-60 of max|u| max|x|, is left out.  The sums are exact: 16
-// products stay below 2^62, after which (K = the thread's columns for row
-// sums, RBT rows for column sums) they are joined into a 96-bit integer, in
-// which a row's or segment's sum is exact too (truncated at 2^-82 of a
-// product's largest value).  So the only errors are the two roundings to 58
-// bits and ul xl; FP64 rounds every product and every partial sum at 2^-53.
-// Taken for blocks whose rows and columns all reach 2^-6 of the block's
-// largest element (create_fixed in api.cu), so that each output keeps this
-// relative to its own row or column.
-// Measured, one product and its update: lmax=31, n=2000 1043 -> 305 us, lmax=15,
-// n=500 47.6 -> 23.4 us a stage; error of a product against extended precision
-// 3.0e-16 (FP64 kernel 3.35e-16, n=2000).  Bound by the multiply pipe (60%
-// active: 12 wide multiply-adds an element) and the issue slots of the sums.
-struct PolI64 {
-    static constexpr int CW = 2;
-    static constexpr bool kFixed = true;
-    static constexpr bool kOffsetSums = false;
-    static constexpr int BITS = 58, LOW = 29;
-    static constexpr int kNonfinite = 0x7ff00000;        // mark in maxima, exponents and Sigma
-    using Elem = int2;                                   // (ul, uh)
-    using Uv = int2;
-    struct XV { int rl, rh, il, ih; };
-    // high word of a maximum -> e with max < 2^e
-    static __device__ __forceinline__ int expo(int h) { return h >= kNonfinite ? kNonfinite : max(h >> 20, 1) - 1022; }
-    // v / 2^(e-58) rounded to an integer, as (low, high), for |v| < 2^e
-    static __device__ __forceinline__ int2 fix(double v, int e)
-    {
-        const long long bits = __double_as_longlong(v);
-        const int E = (int)((bits >> 52) & 0x7ff);
-        unsigned long long m = (unsigned long long)bits & 0xfffffffffffffULL;
-        if (E) m |= 1ULL << 52;
-        // |v| = m 2^(max(E,1) - 1075) < 2^e: one bit more than the result holds, then round
-        const int d = e - (max(E, 1) - 1022);                // >= 0
-        m = (m << 6) >> min(d, 63);
-        m = (m + 1) >> 1;
-        const long long q = bits < 0 ? -(long long)m : (long long)m;
-        const int hi = (int)((q + (1LL << (LOW - 1))) >> LOW);
-        return make_int2((int)(q - ((long long)hi << LOW)), hi);
-    }
-    static __device__ __forceinline__ void loads(const Elem *p, Uv u[CW])   // from shared memory
-    {
-        const int4 v = *reinterpret_cast<const int4 *>(p);
-        u[0] = make_int2(v.x, v.y); u[1] = make_int2(v.z, v.w);
-    }
-    static __device__ __forceinline__ XV zerox() { return XV{0, 0, 0, 0}; }
-    static __device__ __forceinline__ XV fixx(double2 v, int e)
-    {
-        const int2 r = fix(v.x, e), i = fix(v.y, e);
-        return XV{r.x, r.y, i.x, i.y};
-    }
-    using Sigma = int;                                   // exponent of a sum's unit (or kNonfinite)
-    struct RowAcc { long long h, c; };
-    static __device__ __forceinline__ RowAcc rzero(Sigma) { return RowAcc{0, 0}; }
-    static __device__ __forceinline__ void racc(RowAcc &a, Uv u, int xl, int xh)
-    {
-        mad_wide(a.h, u.y, xh);
-        mad_wide(a.c, u.y, xl);
-        mad_wide(a.c, u.x, xh);
-    }
-    // s += a b.  In PTX, since the compiler hoists the sign extension of the
-    // loop-invariant x and then multiplies 64 by 64 bits (68 instructions per
-    // dipole element instead of 12).
-    static __device__ __forceinline__ void mad_wide(long long &s, int a, int b)
-    {
-        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
-    }
-    static __device__ __forceinline__ void rfmax(RowAcc &re, RowAcc &im, Uv u, const XV &x, Sigma)
-    {
-        racc(re, u, x.rl, x.rh);
-        racc(im, u, x.il, x.ih);
-    }
-    // (h 2^29 + c) / 2^5 as a 96-bit integer: a column's sum over a segment
-    struct CRun { unsigned w0, w1; int w2; };
-    static __device__ __forceinline__ CRun czero() { return CRun{0u, 0u, 0}; }
-    static __device__ __forceinline__ CRun cadd(CRun a, CRun b)
-    {
-        CRun r;
-        asm("add.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\taddc.u32 %2, %5, %8;"
-            : "=r"(r.w0), "=r"(r.w1), "=r"(r.w2)
-            : "r"(a.w0), "r"(a.w1), "r"(a.w2), "r"(b.w0), "r"(b.w1), "r"(b.w2));
-        return r;
-    }
-    static __device__ __forceinline__ void cfold(CRun &run, RowAcc &a, Sigma s)
-    {
-        const long long c = a.c >> 5;
-        run = cadd(run, CRun{(unsigned)a.h << 24, (unsigned)(a.h >> 8), (int)(a.h >> 40)});
-        run = cadd(run, CRun{(unsigned)c, (unsigned)(c >> 32), (int)(c >> 63)});
-        a = rzero(s);
-    }
-    // The same in four parts of at most 25 bits, parts[j] of weight 2^24j: a
-    // warp's sum of a row, each part by one reduction instruction
-    // (32 parts stay below 2^31).
-    struct RComp { int p[4]; };
-    static __device__ __forceinline__ RComp rwarp(RowAcc a)
-    {
-        const long long c = a.c >> 5;
-        RComp r;
-        r.p[0] = (int)c & 0xffffff;
-        r.p[1] = ((int)(c >> 24) & 0xffffff) + ((int)a.h & 0xffffff);
-        r.p[2] = (int)(c >> 48) + ((int)(a.h >> 24) & 0xffffff);
-        r.p[3] = (int)(a.h >> 48);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) r.p[j] = __reduce_add_sync(0xffffffffu, r.p[j]);
-        return r;
-    }
-    // unit of the 96-bit sums: 2^(ue + ex - 2 BITS + LOW + 5)
-    static __device__ __forceinline__ Sigma sigma(int ue, int ex)
-    {
-        return ex >= kNonfinite ? kNonfinite : ue + ex - 2 * BITS + LOW + 5;
-    }
-    // (w2 w1 w0) 2^s rounded to nearest, from the bits: a conversion or an
-    // addition in FP64 holds the FP64 pipe for 19 cycles a warp instruction, and
-    // a segment's end took 5200 cycles of them (n = 500).
-    static __device__ __forceinline__ double to_f64(CRun a, Sigma s)
-    {
-        if (s >= kNonfinite) return __longlong_as_double(0x7ff8000000000000LL);
-        const unsigned neg = (unsigned)(a.w2 >> 31);                     // all ones if negative
-        unsigned h = (unsigned)a.w2, m = a.w1, l = a.w0;
-        if (neg) {
-            l = ~l + 1u;
-            m = ~m + (l == 0u);
-            h = ~h + (l == 0u && m == 0u);
-        }
-        if ((h | m | l) == 0u) return 0.0;
-        int e = 95;
-        if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
-        if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
-        const int z = __clz((int)h);
-        h = __funnelshift_l(m, h, z);
-        m = __funnelshift_l(l, m, z);
-        l <<= z;
-        e -= z;                                                          // value = 1.x 2^e, leading bit at the top of h
-        // 53 bits, round to nearest (ties up: below half a unit of the sum's own truncation)
-        unsigned long long r = ((unsigned long long)h << 32) | m;
-        r = (r >> 11) + ((r >> 10) & 1u);
-        e += s;
-        if (e > -1000 && e < 1000)
-            // (the leading bit of r adds 1 to the exponent field)
-            return __longlong_as_double((long long)((r + ((unsigned long long)(e + 1022) << 52)) |
-                                                    ((unsigned long long)(neg & 0x80000000u) << 32)));
-        const double v = scalbn((double)r, e - 52);
-        return neg ? -v : v;
-    }
-    static __device__ __forceinline__ double cto_double(CRun a, Sigma s) { return to_f64(a, s); }
-    // sums of up to 16 warps' parts
-    static __device__ __forceinline__ double parts_to_double(const long long p[4], Sigma s)
-    {
-        const long long lo = p[0] + (p[1] << 24), hi = p[2] + (p[3] << 24);          // lo + hi 2^48
-        CRun r{(unsigned)lo, (unsigned)(lo >> 32), (int)(lo >> 63)};
-        return to_f64(cadd(r, CRun{0u, (unsigned)hi << 16, (int)(hi >> 16)}), s);
-    }
-    static __device__ __forceinline__ void store_xq(void *xq, long long a, double2 v)      // as PolF64
-    {
-        reinterpret_cast<double2 *>(xq)[a] = v;
-    }
-    static __device__ __forceinline__ void store_xq1(void *xq, long long a, int comp, double v)
-    {
-        reinterpret_cast<double *>(xq)[2 * a + comp] = v;
     }
 };
 

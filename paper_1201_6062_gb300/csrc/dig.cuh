@@ -119,6 +119,48 @@ template <int S, int NC> struct DigAcc {
     }
 };
 
+// A signed 96-bit integer.
+struct Dig96 { unsigned w0, w1; int w2; };
+
+__device__ __forceinline__ Dig96 dig_add(Dig96 a, Dig96 b)
+{
+    Dig96 r;
+    asm("add.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\taddc.u32 %2, %5, %8;"
+        : "=r"(r.w0), "=r"(r.w1), "=r"(r.w2)
+        : "r"(a.w0), "r"(a.w1), "r"(a.w2), "r"(b.w0), "r"(b.w1), "r"(b.w2));
+    return r;
+}
+
+// a 2^s rounded to nearest, from the bits: a conversion or an addition in FP64
+// holds the FP64 pipe for 19 cycles a warp instruction.
+__device__ __forceinline__ double dig_to_f64(Dig96 a, int s)
+{
+    const unsigned neg = (unsigned)(a.w2 >> 31);                         // all ones if negative
+    unsigned h = (unsigned)a.w2, m = a.w1, l = a.w0;
+    if (neg) {
+        l = ~l + 1u;
+        m = ~m + (l == 0u);
+        h = ~h + (l == 0u && m == 0u);
+    }
+    if ((h | m | l) == 0u) return 0.0;
+    int e = 95;
+    if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
+    if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
+    const int z = __clz((int)h);
+    h = __funnelshift_l(m, h, z);
+    m = __funnelshift_l(l, m, z);
+    e += s - z;                                                          // value = 1.x 2^e, leading bit at the top of h
+    // 53 bits, round to nearest (ties up: below half a unit of the sum's own truncation)
+    unsigned long long r = ((unsigned long long)h << 32) | m;
+    r = (r >> 11) + ((r >> 10) & 1u);
+    if (e > -1000 && e < 1000)
+        // (the leading bit of r adds 1 to the exponent field)
+        return __longlong_as_double((long long)((r + ((unsigned long long)(e + 1022) << 52)) |
+                                                ((unsigned long long)(neg & 0x80000000u) << 32)));
+    const double v = scalbn((double)r, e - 52);
+    return neg ? -v : v;
+}
+
 // FP64 contexts: weights 0..4 as an exact integer in units of the fourth
 // (|sum| < 2^59 for K <= 4096), the rest in FP32 (below 2^-8 of that unit per product).
 template <int NC> struct DigAcc<8, NC> {
@@ -150,8 +192,8 @@ template <int NC> struct DigAcc<8, NC> {
     __device__ __forceinline__ double value(int j, int e) const
     {
         const long long f = __float2ll_rn(__fmul_rn(l[j], 0x1p24f));
-        PolI64::CRun r{(unsigned)(a[j] << 24), (unsigned)(a[j] >> 8), (int)(a[j] >> 40)};
-        return PolI64::to_f64(PolI64::cadd(r, PolI64::CRun{(unsigned)f, (unsigned)(f >> 32), (int)(f >> 63)}), e - 56);
+        const Dig96 r{(unsigned)(a[j] << 24), (unsigned)(a[j] >> 8), (int)(a[j] >> 40)};
+        return dig_to_f64(dig_add(r, Dig96{(unsigned)f, (unsigned)(f >> 32), (int)(f >> 63)}), e - 56);
     }
 };
 

@@ -16,7 +16,6 @@ struct MvCfg {
     int tma = 0;        // 1: bulk-copy ring kernel (mvt.cu), 0: per-thread loads (mv.cu)
     int RS = 0;         // rows per ring stage (tma only)
     int ld = 0;         // largest row stride the configuration serves (tma only): stage = RS rows of it
-    int fix = 0;        // FP64 systems in fixed point (PolI64; ring only): consumer groups of stepping launches, 0: FP64 pipe
     int per_sm = 1;     // ring CTAs the plan places on each SM (tma only); 1: each CTA holds an SM alone
 };
 
@@ -33,12 +32,6 @@ cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaS
 bool mv_config(int prec, int n, MvCfg *out);
 int mv_ctas_per_sm(int prec, const MvCfg &cfg);
 
-// Fixed-point copies of FP64 dipole blocks (fix.cu).  launch_fix_maxima: high
-// words of the row maxima (first lmax*n ints of out) and column maxima (the
-// next lmax*n) of every block; launch_fix: |U_l| < 2^ue[l] as PolI64's integers.
-cudaError_t launch_fix_maxima(const double *U, long long bstride, int ld, int n, int lmax, int *out, cudaStream_t s);
-cudaError_t launch_fix(const double *U, long long bstride, long long count, int lmax, const int *ue, void *out, cudaStream_t s);
-
 // Ring-fed variant for rows of more than 32 column groups; false if n/ld do
 // not qualify.
 bool mvt_config(int prec, int n, int ld, MvCfg *out);
@@ -52,10 +45,6 @@ cudaError_t mvt_prepare(int prec, const MvCfg &cfg);
 // columns they hold.
 bool mvt_config_layout(int prec, int n, int ld, int idx, MvCfg *out);
 int mvt_layouts(void);
-// Turns a ring configuration of FP64 products into the fixed-point kernel's
-// for rows of up to n columns (false, unchanged: not served); streamed: the
-// dipole blocks come from HBM, with several CTAs per SM where rows are short.
-bool mvt_use_fixed(int prec, int n, bool streamed, MvCfg *cfg);
 // Whether `rs` rows per stage fit the ring for rows of `ld` elements.
 bool mvt_rs_valid(int prec, const MvCfg &cfg, int rs, int ld);
 cudaError_t launch_mvt(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,

@@ -4,10 +4,8 @@
 
 namespace tdse {
 
-static const void *mvt_fn_prec(int prec, const MvCfg &cfg, int rs, bool step = false)
+static const void *mvt_fn_prec(int prec, int idx, int rs, bool step = false)
 {
-    const int idx = cfg.idx;
-    if (cfg.fix) return step ? mvt_fn_i64_step(idx, rs, cfg.fix) : mvt_fn_i64_product(idx, rs);
     switch (prec) {
     case 0: return step ? mvt_fn_f64_step(idx, rs) : mvt_fn_f64_product(idx, rs);
     case 1: return step ? mvt_fn_f32_step(idx, rs) : mvt_fn_f32_product(idx, rs);
@@ -51,34 +49,22 @@ bool mvt_config_layout(int prec, int n, int ld, int idx, MvCfg *out)
     out->tma = 1;
     out->RS = c.RS;
     out->ld = ld;
-    if (!mvt_fn_prec(prec, *out, out->RS)) out->RS = 2;      // the widest layout serves at most 2 rows per stage
-    return mvt_fn_prec(prec, *out, out->RS) != nullptr;
+    if (!mvt_fn_prec(prec, idx, out->RS)) out->RS = 2;      // the widest layout serves at most 2 rows per stage
+    return mvt_fn_prec(prec, idx, out->RS) != nullptr;
 }
 
 int mvt_layouts(void) { return kNumTCfg; }
-
-bool mvt_use_fixed(int prec, int n, bool streamed, MvCfg *cfg)
-{
-    if (prec != 0 || !cfg->tma || n > 2048) return false;      // (at most 256 threads of eight columns)
-    if (cfg->idx >= 6) {
-        cfg->CT = 256;
-        cfg->MAXG = 4;
-    }
-    cfg->fix = cfg->CT == 128 && !streamed ? 2 : 1;
-    cfg->BT = cfg->CT == 256 && cfg->MAXG >= 3 ? mvt_threads<PolI64, 256, 4, 1>() : cfg->CT + 32;
-    return true;
-}
 
 bool mvt_rs_valid(int prec, const MvCfg &cfg, int rs, int ld)
 {
     if (rs != 1 && rs != 2 && rs != 4 && rs != 8) return false;
     if ((long long)rs * ld * elem_size(prec) > STAGE_MAX) return false;
-    return mvt_fn_prec(prec, cfg, rs) != nullptr;
+    return mvt_fn_prec(prec, cfg.idx, rs) != nullptr;
 }
 
 cudaError_t mvt_prepare(int prec, const MvCfg &cfg)
 {
-    const void *fn = mvt_fn_prec(prec, cfg, cfg.RS);
+    const void *fn = mvt_fn_prec(prec, cfg.idx, cfg.RS);
     if (!fn) return cudaErrorInvalidValue;
     return ensure_dyn_smem(fn, NS * STAGE_MAX);
 }
@@ -92,7 +78,7 @@ static int stage_bytes(int prec, const MvCfg &cfg)
 
 int mvt_ctas_per_sm(int prec, const MvCfg &cfg)
 {
-    const void *fn = mvt_fn_prec(prec, cfg, cfg.RS);
+    const void *fn = mvt_fn_prec(prec, cfg.idx, cfg.RS);
     if (!fn || cfg.ld <= 0) return 1;
     if (ensure_dyn_smem(fn, NS * STAGE_MAX) != cudaSuccess) return 1;
     int nb = 0;
@@ -105,7 +91,7 @@ int mvt_ctas_per_sm(int prec, const MvCfg &cfg)
 cudaError_t launch_mvt(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,
                        const int *cta_off, int *err, cudaStream_t stream, bool early)
 {
-    const void *fn = mvt_fn_prec(prec, cfg, cfg.RS);
+    const void *fn = mvt_fn_prec(prec, cfg.idx, cfg.RS);
     if (!fn || cfg.ld <= 0) return cudaErrorInvalidValue;
     if (grid <= 0) return cudaSuccess;
     int stage = stage_bytes(prec, cfg);
@@ -128,19 +114,16 @@ static int launch_smem(int prec, const MvCfg &cfg)
     return cfg.per_sm > 1 ? NS * stage_bytes(prec, cfg) : NS * STAGE_MAX;
 }
 
-// Threads of a stepping launch.
-static int step_threads(const MvCfg &cfg) { return cfg.fix == 2 ? cfg.CT * 2 + 32 : cfg.BT; }
-
 bool mvt_step_fits(int prec, const MvCfg &cfg, int grid)
 {
-    const void *fn = mvt_fn_prec(prec, cfg, cfg.RS, true);
+    const void *fn = mvt_fn_prec(prec, cfg.idx, cfg.RS, true);
     if (!fn || cfg.ld <= 0 || grid <= 0) return false;
     if (stage_bytes(prec, cfg) > STAGE_MAX) return false;
     if (ensure_dyn_smem(fn, NS * STAGE_MAX) != cudaSuccess) return false;
     int dev = 0, sms = 0, nb = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, step_threads(cfg), (size_t)launch_smem(prec, cfg)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, cfg.BT, (size_t)launch_smem(prec, cfg)) != cudaSuccess)
         return false;
     return (long long)nb * sms >= grid;
 }
@@ -148,7 +131,7 @@ bool mvt_step_fits(int prec, const MvCfg &cfg, int grid)
 cudaError_t launch_mvt_step(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, const Seg *segs,
                             const int *cta_off, int *err, const StepArgs &a, cudaStream_t stream)
 {
-    const void *fn = mvt_fn_prec(prec, cfg, cfg.RS, true);
+    const void *fn = mvt_fn_prec(prec, cfg.idx, cfg.RS, true);
     if (!fn || cfg.ld <= 0 || grid <= 0) return cudaErrorInvalidValue;
     int stage = stage_bytes(prec, cfg);
     if (stage > STAGE_MAX) return cudaErrorInvalidValue;
@@ -163,7 +146,7 @@ cudaError_t launch_mvt_step(int prec, const MvCfg &cfg, int grid, const SysDesc 
     void *args[] = {(void *)&sys, (void *)&segs, (void *)&cta_off, (void *)&err, (void *)&stage, (void *)&sa};
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(step_threads(cfg));
+    lc.blockDim = dim3(cfg.BT);
     lc.dynamicSmemBytes = (size_t)launch_smem(prec, cfg);
     lc.stream = stream;
     cudaLaunchAttribute at[1];

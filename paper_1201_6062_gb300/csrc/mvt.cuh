@@ -101,14 +101,17 @@ struct NoBar {
 // CTA's slice [u0, u1) of amplitudes, whose own data are requested before the barrier,
 // and a second barrier (every input of the next pass is written); false: this
 // CTA or another one has given up.
-template <class P, int CTT>
-__device__ __forceinline__ bool step_update_inline(const SysDesc *sys, const StepArgs &A, int pass, volatile int *abort, int *err,
+// Out of line, so that the product's loop, whose accumulators are dead here, is
+// compiled by itself (float-float, lmax=31, n=2000: 180.0 us a stage inlined,
+// 176.5 not).
+template <class P, int CT>
+__device__ __noinline__ bool step_update(const SysDesc *sys, const StepArgs &A, int pass, volatile int *abort, int *err,
                                          volatile int *go_flag, double *dot_sh, long long u0, long long u1)
 {
-    constexpr int NWT = CTT / 32;
+    constexpr int NW = CT / 32;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const GridBar written{A.gbar, (unsigned)(2 * pass + 1) * gridDim.x, abort, err, go_flag, tid, CTT};
-    const GridBar updated{A.gbar, (unsigned)(2 * pass + 2) * gridDim.x, abort, err, go_flag, tid, CTT};
+    const GridBar written{A.gbar, (unsigned)(2 * pass + 1) * gridDim.x, abort, err, go_flag, tid, CT};
+    const GridBar updated{A.gbar, (unsigned)(2 * pass + 2) * gridDim.x, abort, err, go_flag, tid, CT};
     const SysDesc &S0 = sys[0];
     const int per = A.mode == EPI_RK4 ? 4 : A.order;
     if (A.reverse) {
@@ -129,29 +132,29 @@ __device__ __forceinline__ bool step_update_inline(const SysDesc *sys, const Ste
             // term m: (dt/(m-1)) Gamma_{m-1}, or at m = 1 the previous step's (dt/K) G
             aa.to_G = q == 1;
             aa.cg = A.coef[q > 1 ? q - 1 : A.order];
-            go = adj_span<P, AK_TAYLOR, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+            go = adj_span<P, AK_TAYLOR, true>(Sa, u0, u1, tid, CT, aa, &dot, written);
         } else if (q == 3) {
             aa.cG = A.coef[3];
             aa.cg = A.dt;
-            go = adj_span<P, AK_RK4_LAST, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+            go = adj_span<P, AK_RK4_LAST, true>(Sa, u0, u1, tid, CT, aa, &dot, written);
         } else if (q > 0) {
             aa.cG = A.coef[q == 2 ? 3 : 6];
             aa.cg = A.coef[2];
-            go = adj_span<P, AK_RK4_MID, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+            go = adj_span<P, AK_RK4_MID, true>(Sa, u0, u1, tid, CT, aa, &dot, written);
         } else {
             aa.cG = A.coef[6];
-            go = adj_span<P, AK_RK4_FIRST, true>(Sa, u0, u1, tid, CTT, aa, &dot, written);
+            go = adj_span<P, AK_RK4_FIRST, true>(Sa, u0, u1, tid, CT, aa, &dot, written);
         }
         if (!go) return false;
         // fixed-order sum over the CTA: lanes, then warps
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) dot += __shfl_down_sync(0xffffffffu, dot, off);
         if (lane == 0) dot_sh[warp] = dot;
-        named_sync(1, CTT);
+        named_sync(1, CT);
         if (tid == 0) {
             double t = 0.0;
 #pragma unroll
-            for (int w = 0; w < NWT; ++w) t += dot_sh[w];
+            for (int w = 0; w < NW; ++w) t += dot_sh[w];
             A.dots[blockIdx.x] = t;
         }
         if (!updated()) return false;
@@ -210,59 +213,26 @@ __device__ __forceinline__ bool step_update_inline(const SysDesc *sys, const Ste
             const SysDesc &Sx = sys[si];
             const long long o = A.amp_off[si];
             e.f = field_at(Sx.field, A.sps, ek, eh);
-            epi_span<P, true>(Sx, max(g0, o) - o, min(g1, A.amp_off[si + 1]) - o, tid, CTT, kind, e, NoBar{});
+            epi_span<P, true>(Sx, max(g0, o) - o, min(g1, A.amp_off[si + 1]) - o, tid, CT, kind, e, NoBar{});
         }
     } else {
         e.f = field_at(S0.field, A.sps, ek, eh);
-        if (!epi_span<P, true>(S0, u0, u1, tid, CTT, kind, e, written)) return false;
+        if (!epi_span<P, true>(S0, u0, u1, tid, CT, kind, e, written)) return false;
     }
     return updated();
 }
 
-// Out of line, so that the product's loop, whose accumulators are dead here, is
-// compiled by itself (float-float, lmax=31, n=2000: 180.0 us a stage inlined,
-// 176.5 not).  Inlined where the kernel moves registers between its warps: a
-// function is compiled for the launch's count, and the arguments it would take
-// from before the loop spill (fixed point: 353 us out of line, 331 inlined).
-template <class P, int CTT>
-__device__ __noinline__ bool step_update(const SysDesc *sys, const StepArgs &A, int pass, volatile int *abort, int *err,
-                                         volatile int *go_flag, double *dot_sh, long long u0, long long u1)
-{
-    return step_update_inline<P, CTT>(sys, A, pass, abort, err, go_flag, dot_sh, u0, u1);
-}
-
-// Threads of a launch: the consumers and the producer warp.  Nine warps are
-// left 168 registers each, and fixed-point columns take 18 (two 64-bit sums,
-// the running one, x): with six or eight columns a thread the producer gets a
-// warpgroup to itself, which hands its registers to the consumers
-// (256 * 232 + 128 * 40 = 384 * 168).
-template <class P, int CT, int MAXG, int NGRP> __host__ __device__ constexpr int mvt_threads()
-{
-    return P::kFixed && CT == 256 && MAXG >= 3 ? CT + 128 : CT * NGRP + 32;
-}
-
-// NGRP = 2 (fixed-point stepping kernel, 128-thread layouts): two groups of
-// consumers with column sums of their own take the stages in turn.  For blocks
-// that stay in L2, where a plan has one CTA per SM and one warp per scheduler
-// would wait out the latency of every multiply (lmax=15, n=500: 34.3 -> 30.9 us
-// a stage, both with the update by whole amplitudes; 23.4 by components).  Not for single products: 288 threads of 168 registers do not fit
-// beside the previous kernel's blocks, so the ring no longer fills while that
-// one finishes (lmax=7, n=301: a product and its update 34 -> 46 us).
-template <class P, int CT, int MAXG, int RS, bool STEP, int NGRP = 1>
-__global__ void __launch_bounds__(mvt_threads<P, CT, MAXG, NGRP>(), 1)
+template <class P, int CT, int MAXG, int RS, bool STEP>
+__global__ void __launch_bounds__(CT + 32, 1)
 mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const int *__restrict__ cta_off,
            int *__restrict__ err, int stage, const __grid_constant__ StepArgs A)
 {
     constexpr int CW = P::CW;
     constexpr int NW = CT / 32;
-    constexpr int CTT = CT * NGRP, NWT = NW * NGRP;     // all consumers
     constexpr int V = 2 * RBT;
     constexpr int SPC = RBT / RS;          // ring stages per reduction chunk
-    // rows computed at once: a stage's, or fewer where the accumulators need the registers
-    constexpr int CR = !P::kFixed ? RS : (RS == 1 ? 1 : 2);
-    constexpr int VS = 2 * CR;             // row components at once
-    constexpr int DUPS = 32 / VS;          // lanes holding the same component
-    constexpr bool kSplit = mvt_threads<P, CT, MAXG, NGRP>() > CTT + 32;
+    constexpr int VS = 2 * RS;             // row components per stage
+    constexpr int DUPS = 32 / VS;          // lanes holding the same stage component
     static_assert(RBT % RS == 0, "RS must divide RBT");
     using RComp = typename P::RComp;
     using CRun = typename P::CRun;
@@ -273,15 +243,13 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
     __shared__ __align__(8) uint64_t full[NS];
     __shared__ __align__(8) uint64_t empty[NS];
     __shared__ __align__(16) float4 xs_raw[NS][RBT];       // x_l rows of each stage, 16 bytes each
-    __shared__ __align__(16) RComp red[2][NW][V];
+    __shared__ RComp red[2][NW][V];
     __shared__ int abort_flag;
     __shared__ int issued, consumed;
-    __shared__ typename std::conditional<(NGRP > 1), CRun, char>::type comb[NGRP > 1 ? 2 * MAXG * CW : 1][NGRP > 1 ? CT : 1];   // the second group's column sums
-    __shared__ float xmax_sh[NWT], xrow_sh[NWT];
-    __shared__ __align__(16) typename std::conditional<P::kFixed, int2, char>::type xfix[P::kFixed ? NWT : 1][2 * RS];   // the stage's x_l in fixed point, per warp
+    __shared__ float xmax_sh[NW], xrow_sh[NW];
     __shared__ typename std::conditional<STEP, StepArgs, char>::type step_args;       // STEP: the launch's arguments, for step_update
     __shared__ int xready, go_flag;       // STEP: passes whose stage inputs are written; barrier verdict
-    __shared__ double dot_sh[NWT];         // STEP, adjoint: per-warp field-gradient partials
+    __shared__ double dot_sh[NW];         // STEP, adjoint: per-warp field-gradient partials
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
@@ -310,12 +278,12 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
     // previous kernel (whose output, x, is copied only after the wait), so the
     // ring fills while that kernel finishes.
     int npre = 0;
-    if (warp == NWT) {
+    if (warp == NW) {
         for (int si = s0; si < s1 && npre < NS; ++si) {
             const Seg sg = segs[si];
             const SysDesc &S = sys[sg.sys];
             const long long ld = S.ld;
-            const Elem *Ub = reinterpret_cast<const Elem *>(P::kFixed ? S.Uf : S.U) + (long long)sg.l * S.bstride;
+            const Elem *Ub = reinterpret_cast<const Elem *>(S.U) + (long long)sg.l * S.bstride;
             for (int r = sg.i0; r < sg.i1 && npre < NS; r += RS) {
                 const int nr = min(RS, sg.i1 - r);
                 if (lane == 0) {
@@ -332,10 +300,8 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
     pdl_wait();                            // inputs (x) come from the previous kernel
     volatile int *abort = &abort_flag;
 
-    if (warp >= NWT) {
+    if (warp == NW) {
         // ---------------------------------------------------- producer warp
-        if constexpr (kSplit) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-        if (warp == NWT) {
         int q = 0;
         bool ok = true;
         // STEP: x copies of stages of a pass whose inputs are not written yet
@@ -367,7 +333,7 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                 const Seg sg = segs[si];
                 const SysDesc &S = sys[sg.sys];
                 const long long ld = S.ld;
-                const Elem *Ub = reinterpret_cast<const Elem *>(P::kFixed ? S.Uf : S.U) + (long long)sg.l * S.bstride;
+                const Elem *Ub = reinterpret_cast<const Elem *>(S.U) + (long long)sg.l * S.bstride;
                 const long long base_l = (long long)sg.l * S.n;
                 for (int r = sg.i0; r < sg.i1; r += RS) {
                     const int nr = min(RS, sg.i1 - r);
@@ -416,13 +382,10 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
         }
         if (STEP && !flush()) ok = false;
         if (lane == 0) issued = q;
-        }
     } else {
         // ------------------------------------------------- consumer warps
-        if constexpr (kSplit) asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
-        const int grp = NGRP > 1 ? warp / NW : 0, lw = NGRP > 1 ? warp % NW : warp, ctid = NGRP > 1 ? tid % CT : tid;
         long long u0 = 0, u1 = 0;          // STEP: this CTA's slice of sys[0]'s amplitudes
-        if constexpr (STEP && !kSplit) {
+        if constexpr (STEP) {
             u0 = (long long)sys[0].N * blockIdx.x / gridDim.x;
             u1 = (long long)sys[0].N * (blockIdx.x + 1) / gridDim.x;
         }
@@ -438,56 +401,14 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
             const long long base_u = base_l + n;
             // column groups of this thread that lie inside the row (the last may be ragged)
             const int ngrp = (n + CW - 1) / CW;
-            const int mine = ctid < ngrp ? (ngrp - ctid + CT - 1) / CT : 0;
+            const int mine = tid < ngrp ? (ngrp - tid + CT - 1) / CT : 0;
             XV xc[MAXG][CW];
             CRun car[MAXG][CW], cai[MAXG][CW];
-            typename P::Sigma sig, csig;
-            int xexp = 0;                  // kFixed: exponent of the segment's x_l
-            if constexpr (P::kFixed) {
-                // exponents of |x_l| over the segment's rows (column sums) and of
-                // |x_{l+1}| (row sums), then both in fixed point
-                const double2 *xq = reinterpret_cast<const double2 *>(S.xq);
-                double2 raw[MAXG][CW];
-                int xm = 0, xr = 0;
-#pragma unroll
-                for (int g = 0; g < MAXG; ++g)
-#pragma unroll
-                    for (int c = 0; c < CW; ++c) {
-                        const int col = (ctid + g * CT) * CW + c;
-                        raw[g][c] = col < n ? __ldcg(xq + base_u + col) : make_double2(0.0, 0.0);
-                        car[g][c] = P::czero();
-                        cai[g][c] = P::czero();
-                    }
-                for (int r = sg.i0 + tid; r < sg.i1; r += CTT) {
-                    const double2 v = __ldcg(xq + base_l + r);
-                    xm = max(xm, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-                }
-#pragma unroll
-                for (int g = 0; g < MAXG; ++g)
-#pragma unroll
-                    for (int c = 0; c < CW; ++c)
-                        xr = max(xr, max(__double2hiint(raw[g][c].x) & 0x7fffffff, __double2hiint(raw[g][c].y) & 0x7fffffff));
-                xm = __reduce_max_sync(0xffffffffu, xm);
-                xr = __reduce_max_sync(0xffffffffu, xr);
-                if (lane == 0) { xmax_sh[warp] = __int_as_float(xm); xrow_sh[warp] = __int_as_float(xr); }
-                named_sync(1, CTT);
-#pragma unroll
-                for (int w = 0; w < NWT; ++w) { xm = max(xm, __float_as_int(xmax_sh[w])); xr = max(xr, __float_as_int(xrow_sh[w])); }
-                named_sync(1, CTT);
-                xexp = P::expo(xm);
-                const int ex = P::expo(xr), ue = S.ue[sg.l];
-                sig = P::sigma(ue, ex);
-                csig = P::sigma(ue, xexp);
-#pragma unroll
-                for (int g = 0; g < MAXG; ++g)
-#pragma unroll
-                    for (int c = 0; c < CW; ++c) xc[g][c] = P::fixx(raw[g][c], ex);
-            } else {
 #pragma unroll
             for (int g = 0; g < MAXG; ++g)
 #pragma unroll
                 for (int c = 0; c < CW; ++c) {
-                    const int col = (ctid + g * CT) * CW + c;
+                    const int col = (tid + g * CT) * CW + c;
                     xc[g][c] = (col < n) ? P::loadx_g(S.xq, base_u + col) : P::zerox();
                     car[g][c] = P::czero();
                     cai[g][c] = P::czero();
@@ -497,7 +418,7 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
             // |x_{l+1}| over the row (row sums), each the same for the whole CTA
             float xm = 0.f, xr = 0.f;
             if constexpr (P::kOffsetSums) {
-                for (int r = sg.i0 + tid; r < sg.i1; r += CTT) xm = fmaxf(xm, P::xabs(P::loadx_g(S.xq, base_l + r)));
+                for (int r = sg.i0 + tid; r < sg.i1; r += CT) xm = fmaxf(xm, P::xabs(P::loadx_g(S.xq, base_l + r)));
 #pragma unroll
                 for (int g = 0; g < MAXG; ++g)
 #pragma unroll
@@ -508,19 +429,15 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                     xr = fmaxf(xr, __shfl_xor_sync(0xffffffffu, xr, off));
                 }
                 if (lane == 0) { xmax_sh[warp] = xm; xrow_sh[warp] = xr; }
-                named_sync(1, CTT);
+                named_sync(1, CT);
                 xm = 0.f;
                 xr = 0.f;
 #pragma unroll
-                for (int w = 0; w < NWT; ++w) { xm = fmaxf(xm, xmax_sh[w]); xr = fmaxf(xr, xrow_sh[w]); }
-                named_sync(1, CTT);
+                for (int w = 0; w < NW; ++w) { xm = fmaxf(xm, xmax_sh[w]); xr = fmaxf(xr, xrow_sh[w]); }
+                named_sync(1, CT);
             }
-            sig = P::template rsigma<MAXG * CW>(xr, um);
-            csig = P::template csigma<RBT>(xm, um);
-            }
-            int ucol[MAXG];                // first column of each group, clamped to the row
-#pragma unroll
-            for (int g = 0; g < MAXG; ++g) ucol[g] = min((ctid + g * CT) * CW, (int)ld - CW);
+            const typename P::Sigma sig = P::template rsigma<MAXG * CW>(xr, um);
+            const typename P::Sigma csig = P::template csigma<RBT>(xm, um);
             typename P::RowAcc cpr[MAXG][CW], cpi[MAXG][CW];
 #pragma unroll
             for (int g = 0; g < MAXG; ++g)
@@ -536,43 +453,24 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                 for (int st = 0; st < SPC; ++st) {
                     const int row0 = rb + st * RS;
                     if (row0 >= sg.i1) break;
-                    if (NGRP > 1 && st % NGRP != grp) { ++q; continue; }
                     const int nr = min(RS, sg.i1 - row0);
                     const int s = q % NS;
-                    const bool live = mbar_wait_bounded(&full[s], (uint32_t)((q / NS) & 1), abort, WAIT_NS);
-                    if constexpr (P::kFixed) {
-                        // the stage's x_l in fixed point: one lane converts one component, the warp reads them back
-                        if (live && lane < 2 * nr) xfix[warp][lane] = P::fix(reinterpret_cast<const double *>(&xs_raw[s][0])[lane], xexp);
-                        __syncwarp();
-                    }
-                    // Narrow fixed-point layouts stop at the segment's last row (half-empty stages are
-                    // a sixth of n = 500's); wide ones run the constant count: their stages are
-                    // nearly all full and the bound's register spills (306 against 324 us at 31:2000).
-#pragma unroll 1
-                    for (int sub = 0; sub < (P::kFixed && !kSplit ? nr : RS); sub += CR) {
-                    typename P::RowAcc rre[CR], rim[CR];
+                    typename P::RowAcc rre[RS], rim[RS];
 #pragma unroll
-                    for (int rr = 0; rr < CR; ++rr) { rre[rr] = P::rzero(sig); rim[rr] = P::rzero(sig); }
+                    for (int rr = 0; rr < RS; ++rr) { rre[rr] = P::rzero(sig); rim[rr] = P::rzero(sig); }
+                    const bool live = mbar_wait_bounded(&full[s], (uint32_t)((q / NS) & 1), abort, WAIT_NS);
                     if (live) {
                         const Elem *st_rows = reinterpret_cast<const Elem *>(ring + (size_t)s * stage);
-                        typename P::Uv u[CR][MAXG][CW];
-                        XV xi[CR];
+                        typename P::Uv u[RS][MAXG][CW];
+                        XV xi[RS];
 #pragma unroll
-                        for (int rr = 0; rr < CR; ++rr) {
+                        for (int rr = 0; rr < RS; ++rr) {
                             // rows past the segment end hold stale shared memory: use zeros
-                            if constexpr (P::kFixed) {
-                                const int4 xv = reinterpret_cast<const int4 *>(&xfix[warp][0])[sub + rr];
-                                xi[rr] = sub + rr < nr ? XV{xv.x, xv.y, xv.z, xv.w} : P::zerox();
-                            } else {
-                                xi[rr] = (sub + rr < nr) ? P::loadx(&xs_raw[s][0], sub + rr) : P::zerox();
-                            }
+                            xi[rr] = (rr < nr) ? P::loadx(&xs_raw[s][0], rr) : P::zerox();
 #pragma unroll
                             for (int g = 0; g < MAXG; ++g) {
-                                if constexpr (P::kFixed) {
-                                    // stale rows meet x = 0, threads past the row re-read its last columns and meet x = 0
-                                    P::loads(st_rows + (sub + rr) * ld + ucol[g], u[rr][g]);
-                                } else if (g < mine && sub + rr < nr) {
-                                    P::loads(st_rows + (sub + rr) * ld + (ctid + g * CT) * CW, u[rr][g]);
+                                if (g < mine && rr < nr) {
+                                    P::loads(st_rows + rr * ld + (tid + g * CT) * CW, u[rr][g]);
                                 } else {
 #pragma unroll
                                     for (int c = 0; c < CW; ++c) u[rr][g][c] = typename P::Uv{};
@@ -580,7 +478,7 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                             }
                         }
 #pragma unroll
-                        for (int rr = 0; rr < CR; ++rr)
+                        for (int rr = 0; rr < RS; ++rr)
 #pragma unroll
                             for (int g = 0; g < MAXG; ++g)
 #pragma unroll
@@ -589,25 +487,13 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                                     P::rfmax(cpr[g][c], cpi[g][c], u[rr][g][c], xi[rr], csig);
                                 }
                     }
-                    if (!P::kFixed) {
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&empty[s]);
-                        ++q;
-                    }
-                    if constexpr (P::kFixed) {
-#pragma unroll
-                    for (int rr = 0; rr < CR; ++rr) {
-                        const RComp a = P::rwarp(rre[rr]), b = P::rwarp(rim[rr]);
-                        if (lane == 0) {
-                            red[parity][lw][2 * (st * RS + sub + rr)] = a;
-                            red[parity][lw][2 * (st * RS + sub + rr) + 1] = b;
-                        }
-                    }
-                    } else {
-                    // warp transpose-reduce of the rows' 2*CR components
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty[s]);
+                    ++q;
+                    // warp transpose-reduce of the stage's 2*RS row components
                     RComp v[VS];
 #pragma unroll
-                    for (int rr = 0; rr < CR; ++rr) { v[2 * rr] = P::rdone(rre[rr], sig); v[2 * rr + 1] = P::rdone(rim[rr], sig); }
+                    for (int rr = 0; rr < RS; ++rr) { v[2 * rr] = P::rdone(rre[rr], sig); v[2 * rr + 1] = P::rdone(rim[rr], sig); }
                     int idx = 0;
 #pragma unroll
                     for (int step = 0; step < 5; ++step) {
@@ -627,16 +513,9 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                             v[0] = P::radd(v[0], P::rshfl(v[0], off));
                         }
                     }
-                    if ((lane & (DUPS - 1)) == 0) red[parity][lw][2 * (st * RS + sub) + idx] = v[0];
-                    }
-                    }
-                    if constexpr (P::kFixed) {
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&empty[s]);
-                        ++q;
-                    }
+                    if ((lane & (DUPS - 1)) == 0) red[parity][warp][st * VS + idx] = v[0];
                 }
-                if constexpr (P::kOffsetSums || P::kFixed) {
+                if constexpr (P::kOffsetSums) {
 #pragma unroll
                     for (int g = 0; g < MAXG; ++g)
 #pragma unroll
@@ -645,29 +524,20 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                             P::cfold(cai[g][c], cpi[g][c], csig);
                         }
                 }
-                named_sync(1, CTT);
+                named_sync(1, CT);
                 if (warp == 0 && lane < V) {
                     const int i = rb + (lane >> 1);
                     if (i < sg.i1 && !*abort) {
                         double *dst = reinterpret_cast<double *>(S.R + base_l + i) + (lane & 1);
-                        if constexpr (P::kFixed) {
-                            long long p[4] = {0, 0, 0, 0};
+                        RComp sum = red[parity][0][lane];
 #pragma unroll
-                            for (int w = 0; w < NW; ++w)
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) p[j] += red[parity][w][lane].p[j];
-                            *dst = P::parts_to_double(p, sig);
-                        } else {
-                            RComp sum = red[parity][0][lane];
-#pragma unroll
-                            for (int w = 1; w < NW; ++w) sum = P::radd(sum, red[parity][w][lane]);
-                            *dst = P::rto_double(sum, sig);
-                        }
+                        for (int w = 1; w < NW; ++w) sum = P::radd(sum, red[parity][w][lane]);
+                        *dst = P::rto_double(sum, sig);
                     }
                 }
                 parity ^= 1;
             }
-            if constexpr (!P::kOffsetSums && !P::kFixed) {
+            if constexpr (!P::kOffsetSums) {
 #pragma unroll
                 for (int g = 0; g < MAXG; ++g)
 #pragma unroll
@@ -676,46 +546,20 @@ mvt_kernel(const SysDesc *__restrict__ sys, const Seg *__restrict__ segs, const 
                         P::cfold(cai[g][c], cpi[g][c], csig);
                     }
             }
-            if constexpr (NGRP > 1) {
-                if (grp > 0) {
-#pragma unroll
-                    for (int g = 0; g < MAXG; ++g)
-#pragma unroll
-                        for (int c = 0; c < CW; ++c) {
-                            comb[2 * (g * CW + c)][ctid] = car[g][c];
-                            comb[2 * (g * CW + c) + 1][ctid] = cai[g][c];
-                        }
-                }
-                named_sync(1, CTT);
-                if (grp > 0) continue;
-#pragma unroll
-                for (int g = 0; g < MAXG; ++g)
-#pragma unroll
-                    for (int c = 0; c < CW; ++c) {
-                        car[g][c] = P::cadd(car[g][c], comb[2 * (g * CW + c)][ctid]);
-                        cai[g][c] = P::cadd(cai[g][c], comb[2 * (g * CW + c) + 1][ctid]);
-                    }
-            }
             if (!*abort) {
                 double2 *Pslot = S.P + (long long)sg.slot * n;
 #pragma unroll
                 for (int g = 0; g < MAXG; ++g)
 #pragma unroll
                     for (int c = 0; c < CW; ++c) {
-                        const int col = (ctid + g * CT) * CW + c;
+                        const int col = (tid + g * CT) * CW + c;
                         if (col < n)
                             Pslot[col] = make_double2(P::cto_double(car[g][c], csig), P::cto_double(cai[g][c], csig));
                     }
             }
         }
         if constexpr (STEP) {
-            bool go;
-            if constexpr (kSplit)
-                go = step_update_inline<P, CTT>(sys, A, pass, abort, err, &go_flag, dot_sh,
-                                                (long long)sys[0].N * blockIdx.x / gridDim.x,
-                                                (long long)sys[0].N * (blockIdx.x + 1) / gridDim.x);
-            else go = step_update<P, CTT>(sys, step_args, pass, abort, err, &go_flag, dot_sh, u0, u1);
-            if (!go) break;
+            if (!step_update<P, CT>(sys, step_args, pass, abort, err, &go_flag, dot_sh, u0, u1)) break;
             if (tid == 0) {
                 __threadfence_block();
                 *(volatile int *)&xready = pass + 1;
@@ -740,14 +584,14 @@ struct TCfg { int CT, MAXG; };
 constexpr TCfg kTCfg[] = {{128, 1}, {128, 2}, {192, 2}, {256, 2}, {192, 3}, {256, 3}, {256, 4}, {512, 4}};
 constexpr int kNumTCfg = sizeof(kTCfg) / sizeof(kTCfg[0]);
 
-template <class P, int CT, int MAXG, bool STEP, int NGRP = 1>
+template <class P, int CT, int MAXG, bool STEP>
 inline const void *mvt_fn_rs(int rs)
 {
     switch (rs) {
-    case 1: return (const void *)mvt_kernel<P, CT, MAXG, 1, STEP, NGRP>;
-    case 2: return (const void *)mvt_kernel<P, CT, MAXG, 2, STEP, NGRP>;
-    case 4: return (const void *)mvt_kernel<P, CT, MAXG, 4, STEP, NGRP>;
-    case 8: return (const void *)mvt_kernel<P, CT, MAXG, 8, STEP, NGRP>;
+    case 1: return (const void *)mvt_kernel<P, CT, MAXG, 1, STEP>;
+    case 2: return (const void *)mvt_kernel<P, CT, MAXG, 2, STEP>;
+    case 4: return (const void *)mvt_kernel<P, CT, MAXG, 4, STEP>;
+    case 8: return (const void *)mvt_kernel<P, CT, MAXG, 8, STEP>;
     }
     return nullptr;
 }
@@ -755,7 +599,6 @@ inline const void *mvt_fn_rs(int rs)
 template <class P, bool STEP>
 inline const void *mvt_fn(int idx, int rs)
 {
-    if (P::kFixed && idx == 7) idx = 6;         // (rows of up to 2048 columns only: mvt_use_fixed)
     switch (idx) {
     case 0: return mvt_fn_rs<P, 128, 1, STEP>(rs);
     case 1: return mvt_fn_rs<P, 128, 2, STEP>(rs);
@@ -764,7 +607,7 @@ inline const void *mvt_fn(int idx, int rs)
     case 4: return mvt_fn_rs<P, 192, 3, STEP>(rs);
     case 5: return mvt_fn_rs<P, 256, 3, STEP>(rs);
     case 6: return mvt_fn_rs<P, 256, 4, STEP>(rs);
-    case 7: if constexpr (!P::kFixed) return rs <= 2 ? mvt_fn_rs<P, 512, 4, STEP>(rs) : nullptr;
+    case 7: return rs <= 2 ? mvt_fn_rs<P, 512, 4, STEP>(rs) : nullptr;
     }
     return nullptr;
 }
@@ -774,10 +617,8 @@ inline const void *mvt_fn(int idx, int rs)
 const void *mvt_fn_f64_product(int idx, int rs);
 const void *mvt_fn_f32_product(int idx, int rs);
 const void *mvt_fn_df32_product(int idx, int rs);
-const void *mvt_fn_i64_product(int idx, int rs);
 const void *mvt_fn_f64_step(int idx, int rs);
 const void *mvt_fn_f32_step(int idx, int rs);
 const void *mvt_fn_df32_step(int idx, int rs);
-const void *mvt_fn_i64_step(int idx, int rs, int groups);
 
 }  // namespace tdse
