@@ -212,9 +212,12 @@ tdse_status tdse_populations(tdse_ctx *ctx, const double *c, int B, double *per_
  * each dipole block is read once per stage for all of them (block GEMMs
  * U_l [X_{l+1}] and U_l^T [X_l] with X the n x 2B real matrix of the states'
  * real and imaginary parts).  By precision of the context:
- *   FP32, DF32, FP64   tcgen05 block GEMM of both operands split into 4, 6 or
- *           8 digits of 8 bits, whose products and sums are exact; the digits
- *           of the blocks are made at a context's first batch and kept.  Where
+ *   FP32, DF32, FP64   tcgen05 block GEMM of both operands split into 7
+ *           (FP32, DF32) or 11 digits (FP64) of 8 bits, whose products and sums
+ *           are exact; what is left out is below 2^-53 (FP32, DF32) or 2^-84
+ *           of the largest dipole element of the row times the largest
+ *           amplitude of the block, per product.  The digits of the blocks are
+ *           made at a context's first batch and kept.  Where
  *           their memory cannot be had, or rows are short (n < 56) and pulses
  *           many, or FP64 pulses few: FP32 and DF32 on the FMA pipe (DF32:
  *           float-float), FP64 pulse by pulse on the single-system path (as

@@ -4,30 +4,37 @@
 
 namespace tdse {
 
+// Integers that hold S digits.
+template <int S> using DigInt = typename std::conditional<(S > 7), __int128, long long>::type;
+template <int S> using DigUint = typename std::conditional<(S > 7), unsigned __int128, unsigned long long>::type;
+
 // |v| 2^(8S-1-e) rounded to the nearest integer, with the sign of v, for
-// |v| < 2^e (S = 8: |v| < 2^(e-1)), from the bits of v: the FP64 pipe is
-// 1/64 of the integer one on this GPU.
-template <int S> __device__ __forceinline__ long long dig_fixed(double v, int e)
+// |v| < 2^e, from the bits of v: the FP64 pipe is 1/64 of the integer one on
+// this GPU.
+template <int S> __device__ __forceinline__ DigInt<S> dig_fixed(double v, int e)
 {
     const long long bits = __double_as_longlong(v);
     const int E = (int)((bits >> 52) & 0x7ff);
-    unsigned long long m = (unsigned long long)bits & 0xfffffffffffffULL;
-    if (E) m |= 1ULL << 52;
-    const int sh = max(E, 1) - 1075 + 8 * S - 1 - e;      // |v| = m 2^(max(E,1) - 1075)
-    if (sh >= 0) m <<= (sh < 63 ? sh : 63);               // (sh <= 9 for |v| in range)
-    else if (sh > -63) m = (m + (1ULL << (-sh - 1))) >> -sh;
+    unsigned long long f = (unsigned long long)bits & 0xfffffffffffffULL;
+    if (E) f |= 1ULL << 52;
+    const int sh = max(E, 1) - 1075 + 8 * S - 1 - e;      // |v| = f 2^(max(E,1) - 1075)
+    DigUint<S> m = f;
+    if (sh >= 0) m <<= (sh < 8 * S - 54 ? sh : 8 * S - 54);      // (sh <= 8 S - 54 for |v| in range)
+    else if (sh > -63) m = (f + (1ULL << (-sh - 1))) >> -sh;
     else m = 0;
-    return bits < 0 ? -(long long)m : (long long)m;
+    return bits < 0 ? -(DigInt<S>)m : (DigInt<S>)m;
 }
 
 // Digit s (0 the leading one) of q = sum_s d_s 256^(S-1-s), |d_s| <= 128.
-template <int S> __device__ __forceinline__ void dig_split(long long q, int d[S])
+template <int S> __device__ __forceinline__ void dig_split(DigInt<S> q, int d[S])
 {
-    constexpr unsigned long long half = 0x0080808080808080ULL >> (8 * (8 - S));
-    const unsigned long long u = (unsigned long long)(q + (long long)half);
+    DigUint<S> half = 0;
 #pragma unroll
-    for (int s = 1; s < S; ++s) d[s] = (int)((u >> (8 * (S - 1 - s))) & 0xff) - 128;
-    d[0] = (int)((long long)u >> (8 * (S - 1)));
+    for (int s = 1; s < S; ++s) half = (half << 8) | 0x80;
+    const DigUint<S> u = (DigUint<S>)q + half;
+#pragma unroll
+    for (int s = 1; s < S; ++s) d[s] = (int)((unsigned)(u >> (8 * (S - 1 - s))) & 0xff) - 128;
+    d[0] = (int)((DigInt<S>)u >> (8 * (S - 1)));
 }
 
 __device__ __forceinline__ unsigned dig_bf16x2(int a, int b)
@@ -66,10 +73,10 @@ __global__ void dig_umax_kernel(const void *U, long long bstride, int ld, int n,
 }
 
 // High words of maxima -> exponents (DIG_NONFINITE stays).
-template <int S> __global__ void dig_uexp_kernel(int *eu, long long count)
+__global__ void dig_uexp_kernel(int *eu, long long count)
 {
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < count) eu[q] = eu[q] >= DIG_NONFINITE ? DIG_NONFINITE : dig_exp<S>(eu[q]);
+    if (q < count) eu[q] = eu[q] >= DIG_NONFINITE ? DIG_NONFINITE : dig_exp(eu[q]);
 }
 
 // Digits of U_l (scaled per row) and of U_l^T (scaled per column of U_l), the
@@ -118,7 +125,7 @@ static cudaError_t dig_u_prec(const void *U, long long bstride, int ld, int n, i
     if (z != cudaSuccess) return z;
     dig_umax_kernel<PREC><<<grid, thr, 0, s>>>(U, bstride, ld, n, lmax, eu);
     const long long cnt = 2LL * lmax * n;
-    dig_uexp_kernel<S><<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(eu, cnt);
+    dig_uexp_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(eu, cnt);
     const dim3 g2((ldb + 31) / 32, (ldb + 31) / 32, lmax);
     dig_u_kernel<PREC, S><<<g2, thr, 0, s>>>(U, bstride, ld, n, lmax, ldb, eu, digits);
     return cudaGetLastError();
@@ -195,7 +202,7 @@ dig_x_kernel(const double2 *__restrict__ src, int n, int nb, int lmax, int B, co
 #pragma unroll
                 for (int s = 0; s < S; ++s) d[q][s] = 0;
             } else {
-                dig_split<S>(dig_fixed<S>(v[part][q], dig_exp<S>(h)), d[q]);
+                dig_split<S>(dig_fixed<S>(v[part][q], dig_exp(h)), d[q]);
             }
         }
         __nv_bfloat16 *o = out + (2LL * b + part) * plane + (long long)l * nb + i;   // (nb, i: multiples of 4)
@@ -212,9 +219,7 @@ cudaError_t launch_dig_x(int slices, const double2 *src, int n, int nb, int lmax
 {
     void *args[] = {(void *)&src, (void *)&n, (void *)&nb, (void *)&lmax, (void *)&B, (void *)&xmax, (void *)&xmax_next,
                     (void *)&digits};
-    const void *fn = slices == 4   ? (const void *)dig_x_kernel<4>
-                     : slices == 6 ? (const void *)dig_x_kernel<6>
-                                   : (const void *)dig_x_kernel<8>;
+    const void *fn = slices == 7 ? (const void *)dig_x_kernel<7> : (const void *)dig_x_kernel<11>;
     return launch_pdl(fn, dim3((n + 511) / 512, lmax + 1, B), dim3(128), 0, s, args);
 }
 
@@ -250,17 +255,19 @@ static int dig_sms()
 // 128, 620 and 690 for single CTAs: the issue of the products and their loads
 // more than the products themselves, except at 128.  The update of the last tile
 // follows its products, some 1000 cycles a pulse.  Measured, us a stage at 32 /
-// 64 / 128 planes: FP32, lmax=9, n=487, 100 pulses 71 / 77 / 80, lmax=20, n=200,
-// 300 pulses 104 / 95 / 119, lmax=15, n=1000, 64 pulses 195 / 141 / 128;
-// float-float, lmax=15, n=1000, 256 pulses - / 706 / 499; FP64, lmax=7, n=301, 24
-// pulses 68 / 85 (one size for all shapes gave 80, 119, 128, 499 and 85).
+// 64 / 128 planes: FP32, lmax=9, n=487, 100 pulses 155 / 133 / 124, lmax=20, n=200,
+// 300 pulses 222 / 153 / 151, lmax=7, n=301, 24 pulses 55 / 61 / 68; float-float,
+// lmax=15, n=1000, 256 pulses 1677 / 929 / 632; FP64, lmax=7, n=301, 24 pulses
+// 107 / 137, lmax=15, n=1000, 64 pulses 1050 / 799; single CTAs, FP64, lmax=3, n=100,
+// 200 pulses 65 / 90.
 DigTile dig_tile(int slices, int n, int lmax, int B)
 {
     const int cg = n > DBM ? 2 : 1, units = dig_sms() / cg, mt = (n + DBM * cg - 1) / (DBM * cg);
-    const long long steps = (long long)((n + DBK - 1) / DBK) * (slices / 2) * (slices / 2 + 1);
+    long long steps = 0;                                 // digit pairs of tiles of a product
+    for (int g = 0; g < dig_groups(slices); ++g) steps += (dig_top(slices, g) + 1) * (long long)((n + DBK - 1) / DBK);
     DigTile best{cg, 32};
     long long low = 0;
-    for (int bn = 32; bn <= (cg == 2 && slices < 8 ? 128 : 64); bn *= 2) {
+    for (int bn = 32; bn <= (cg == 2 && !dig_int(slices) ? 128 : 64); bn *= 2) {
         const long long per = (long long)mt * ((2LL * B + bn - 1) / bn), tiles = per * (lmax + 1);
         long long parts = 0;                             // products of CTA 0
         for (long long t = 0; t < tiles; t += units) parts += lmax > 1 && t < per * (lmax - 1) ? 2 : 1;
@@ -278,7 +285,7 @@ size_t dig_scratch_bytes(DigTile t) { return (size_t)dig_sms() * (t.bn / 2) * DB
 
 cudaError_t launch_dig(int slices, DigTile t, const DigMaps &m, const DigArgs &A, cudaStream_t stream)
 {
-    const void *fn = slices == 4 ? dig_fn4(t.cg, t.bn) : (slices == 6 ? dig_fn6(t.cg, t.bn) : dig_fn8(t.cg, t.bn));
+    const void *fn = slices == 7 ? dig_fn7(t.cg, t.bn) : dig_fn11(t.cg, t.bn);
     if (!fn) return cudaErrorInvalidValue;
     const int smem = dig_smem(t.bn, t.cg);
     const cudaError_t e = ensure_dyn_smem(fn, smem);

@@ -10,17 +10,29 @@
 // integer of 8 bits, exact in bf16, and a sum of 1024 products of digits is an
 // integer of at most 2^24, exact in the FP32 accumulators of tcgen05.mma: the
 // products carry no rounding at all.  Digit pairs (s, t) with s + t <= S - 1
-// are multiplied, so what is left out is below 2^-8S of max|u| max|x| per
-// product (S = 4: FP32, 6: float-float, 8: FP64 products).
+// are multiplied, so what is left out is below S 2^-8S of max|u| max|x| per
+// product, the maxima those of the row and of the (block, plane).
+//
+// The digits are fixed point, and a bound state has one amplitude near 1 and
+// others of its block far below, which meet dipole elements that fall off: S is
+// chosen so that the sum of such small terms keeps the digits that FP32 or FP64
+// products would give it.  7 digits (FP32, float-float) carry terms down to
+// 2^-29 of the largest at FP32's accuracy, 11 (FP64) down to 2^-31 at FP64's.
+// Largest error of a component of D x over the sum of its own terms' magnitudes,
+// the products these replace (FMA pipe, FP64 pipe) and these: hydrogen in a
+// sphere of 100 a.u., n=301, 20 a.u. into a pulse, FP32 1.0e-6 and 4.6e-8,
+// float-float 3.7e-7 and 1.2e-8, FP64 1.4e-15 and 1.7e-16; one amplitude of 1
+// whose elements fall to 1e-7 and a tail of 1e-10, 1.7e-6 and 1.1e-7, 4.7e-7
+// and 9.1e-8, 1.2e-15 and 1.7e-16 (with 4, 6 and 8 digits 1.3e-1, 1.0e-5, 1.2e-9).
 //
 // Pairs of one weight w = s + t share an accumulator.  Weights are taken two
-// at a time (2g+1 and 2g, group g): step s = 0 .. 2g+1 loads A_s and B_{2g+1-s}
-// and multiplies A_s B_{2g+1-s} (the odd weight) and A_{s-1} B_{2g+1-s} (the even
-// one), so each digit tile is loaded once per group and two steps are live at
+// at a time (w and w - 1, group by group; S odd: weight 0 alone): step s = 0 .. w
+// loads A_s and B_{w-s} and multiplies A_s B_{w-s} (weight w) and A_{s-1} B_{w-s}
+// (w - 1), so each digit tile is loaded once per group and two steps are live at
 // any time.  A group's accumulators are drained before 1024 products have been
-// added: every 512, 256, 128, 128 columns of K for g = 0 .. 3.  Two pairs of
-// accumulators in tensor memory let the drain of one overlap the products of
-// the next.
+// added: every 512 columns of K for w = 0, 320 for 2, 192, 128, 64, 64 for 4 .. 10.
+// Two pairs of accumulators in tensor memory let the drain of one overlap the
+// products of the next.
 //
 // Bound: the products, S (S + 1) / 2 bf16 MMAs per element.  CG = 2: a pair of
 // CTAs (one TPC) shares a 256-row tile, each loading its own rows of A and half
@@ -34,11 +46,11 @@
 // update is bound by the FP64 pipe (2 operations per cycle and SM; 8-10 per
 // amplitude here), and run by the draining warps it stalled the products.
 // Measured on GB300, one stage of 256 pulses, lmax=15, n=1000 (31 GFLOP of real
-// products): float-float 3645 (FMA pipe, bgemm_df.cu) -> 502 us, FP32 945
-// (batch.cu) -> 317 us; FP64, 24 pulses, lmax=7, n=301: 692 (pulse by pulse) ->
-// 68 us.  21 products at the bf16 rate of 1927 TFLOP/s would take 334 us.  Of the
-// way there (float-float): 128-row tiles of single CTAs updated by the draining
-// warps 1305 us, pairs with updating warps 898, the whole-warp issue loop
+// products): float-float 3637 (FMA pipe, bgemm_df.cu) -> 632 us, FP32 945
+// (batch.cu) -> 628 us; FP64, 24 pulses, lmax=7, n=301: 649 (pulse by pulse) ->
+// 107 us.  28 products at the bf16 rate of 1927 TFLOP/s would take 455 us.  Of the
+// way there (float-float, 6 digits): 128-row tiles of single CTAs updated by the
+// draining warps 1305 us, pairs with updating warps 898, the whole-warp issue loop
 // (elect_one) 603, states by bulk copies 560, eight updating warps 509.  What is
 // left: a step (24 KB of operands a CTA) takes 620 cycles against 448 of products,
 // 40 bytes a cycle and SM out of L2.
@@ -57,16 +69,17 @@ constexpr int DBM = 128, DBK = 64;
 constexpr int DA_BYTES = DBM * DBK * 2;                 // 16 KB
 constexpr int DIG_DRAIN_WARPS = 8, DIG_UPD_WARPS = 8;
 constexpr int DIG_THREADS = 128 + 32 * (DIG_DRAIN_WARPS + DIG_UPD_WARPS);   // warps 0..3: loads of A, MMA issue, state loads, loads of B
-// Registers: launched with 96 per thread.  Tiles of 128 planes: the first
-// warpgroup keeps 32, the draining ones take 160 each for the running sums, the
-// updating ones keep 64: 128 * (32 + 2 * 160 + 2 * 64) = 640 * 96; smaller
-// tiles: 40, 144, 72.
+// Registers: launched with 96 per thread.  Where a draining thread holds 128
+// words of running sums, the first warpgroup keeps 32, the draining ones take
+// 160 each and the updating ones keep 64: 128 * (32 + 2 * 160 + 2 * 64) =
+// 640 * 96; else 40, 144, 72.
 constexpr int DIG_REGS_LAUNCH = 96;
-__host__ __device__ constexpr int dig_regs_low(int bn) { return bn == 128 ? 32 : 40; }
-__host__ __device__ constexpr int dig_regs_drain(int bn) { return bn == 128 ? 160 : 144; }
-__host__ __device__ constexpr int dig_regs_upd(int bn) { return bn == 128 ? 64 : 72; }
-__host__ __device__ constexpr int dig_regs(int bn) { return 128 * dig_regs_low(bn) + 32 * DIG_DRAIN_WARPS * dig_regs_drain(bn) + 32 * DIG_UPD_WARPS * dig_regs_upd(bn); }
-static_assert(dig_regs(128) <= DIG_THREADS * DIG_REGS_LAUNCH && dig_regs(64) <= DIG_THREADS * DIG_REGS_LAUNCH, "register split");
+__host__ __device__ constexpr bool dig_wide(int S, int bn) { return bn * (S > 7 ? 2 : 1) >= 128; }
+__host__ __device__ constexpr int dig_regs_low(bool wide) { return wide ? 32 : 40; }
+__host__ __device__ constexpr int dig_regs_drain(bool wide) { return wide ? 160 : 144; }
+__host__ __device__ constexpr int dig_regs_upd(bool wide) { return wide ? 64 : 72; }
+__host__ __device__ constexpr int dig_regs(bool wide) { return 128 * dig_regs_low(wide) + 32 * DIG_DRAIN_WARPS * dig_regs_drain(wide) + 32 * DIG_UPD_WARPS * dig_regs_upd(wide); }
+static_assert(dig_regs(true) <= DIG_THREADS * DIG_REGS_LAUNCH && dig_regs(false) <= DIG_THREADS * DIG_REGS_LAUNCH, "register split");
 constexpr uint64_t DIG_WAIT_NS = 2000000000ull;
 constexpr int DIG_SUPER = 8;                            // K tiles (of 64) per round over the groups
 constexpr int DIG_NONFINITE = 0x7ff00000;               // xmax / eu mark of a non-finite maximum
@@ -85,12 +98,17 @@ __host__ __device__ constexpr int dig_smem(int bn, int cg)
     return dig_stages(bn, cg) * dig_stage_bytes(bn, cg) + DIG_NSU * DIG_SLOT + 1024;
 }
 
-// K tiles a group's accumulators take before a drain: (2g+2) pairs times 64 per tile <= 1024 products.
-__host__ __device__ constexpr int dig_chunk(int g) { return g == 0 ? 8 : (g == 1 ? 4 : 2); }
+// Weights are taken two at a time: group g has the pairs of weight dig_top(S, g) and of the one below
+// (S odd: group 0 has weight 0 alone).
+__host__ __device__ constexpr int dig_groups(int S) { return (S + 1) / 2; }
+__host__ __device__ constexpr int dig_top(int S, int g) { return 2 * g + 1 - (S & 1); }
+// K tiles the accumulators of top weight w take before a drain: (w+1) pairs times 64 per tile <= 1024 products.
+__host__ __device__ constexpr int dig_chunk(int w) { return w == 0 ? 8 : 16 / (w + 1); }
+__host__ __device__ constexpr bool dig_int(int S) { return S > 7; }      // FP64 contexts: integer sums
 
 // Running sums of NC outputs of one thread, in units of 2^(eu+ex-14).
 // FP32 / float-float contexts: a float-float pair, the three leading weights
-// added exactly (TwoSum), the others (at most 2^-24 of the first) in FP32.
+// added exactly (TwoSum), the others in FP32.
 template <int S, int NC> struct DigAcc {
     float h[NC], l[NC];
     __device__ __forceinline__ void clear()
@@ -104,104 +122,73 @@ template <int S, int NC> struct DigAcc {
         h[j] = s.h;
         l[j] = __fadd_rn(l[j], s.l);
     }
-    template <int G> __device__ __forceinline__ void fold(int j, float odd, float even)
+    // a sum of products of weight W
+    template <int W> __device__ __forceinline__ void fold(int j, float v)
     {
-        if constexpr (G == 2) {
-            l[j] = __fmaf_rn(odd, 0x1p-40f, l[j]);
-            l[j] = __fmaf_rn(even, 0x1p-32f, l[j]);
-        } else if constexpr (G == 1) {
-            l[j] = __fmaf_rn(odd, 0x1p-24f, l[j]);
-            add(j, __fmul_rn(even, 0x1p-16f));
-        } else {
-            add(j, __fmul_rn(odd, 0x1p-8f));
-            add(j, even);
-        }
+        constexpr float unit = 1.0f / (1ULL << (8 * W));
+        if constexpr (W == 0) add(j, v);
+        else if constexpr (W <= 2) add(j, __fmul_rn(v, unit));
+        else l[j] = __fmaf_rn(v, unit, l[j]);
     }
 };
 
-// A signed 96-bit integer.
-struct Dig96 { unsigned w0, w1; int w2; };
-
-__device__ __forceinline__ Dig96 dig_add(Dig96 a, Dig96 b)
-{
-    Dig96 r;
-    asm("add.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\taddc.u32 %2, %5, %8;"
-        : "=r"(r.w0), "=r"(r.w1), "=r"(r.w2)
-        : "r"(a.w0), "r"(a.w1), "r"(a.w2), "r"(b.w0), "r"(b.w1), "r"(b.w2));
-    return r;
-}
-
-// a 2^s rounded to nearest, from the bits: a conversion or an addition in FP64
-// holds the FP64 pipe for 19 cycles a warp instruction.
-__device__ __forceinline__ double dig_to_f64(Dig96 a, int s)
-{
-    const unsigned neg = (unsigned)(a.w2 >> 31);                         // all ones if negative
-    unsigned h = (unsigned)a.w2, m = a.w1, l = a.w0;
-    if (neg) {
-        l = ~l + 1u;
-        m = ~m + (l == 0u);
-        h = ~h + (l == 0u && m == 0u);
-    }
-    if ((h | m | l) == 0u) return 0.0;
-    int e = 95;
-    if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
-    if (h == 0u) { h = m; m = l; l = 0u; e -= 32; }
-    const int z = __clz((int)h);
-    h = __funnelshift_l(m, h, z);
-    m = __funnelshift_l(l, m, z);
-    e += s - z;                                                          // value = 1.x 2^e, leading bit at the top of h
-    // 53 bits, round to nearest (ties up: below half a unit of the sum's own truncation)
-    unsigned long long r = ((unsigned long long)h << 32) | m;
-    r = (r >> 11) + ((r >> 10) & 1u);
-    if (e > -1000 && e < 1000)
-        // (the leading bit of r adds 1 to the exponent field)
-        return __longlong_as_double((long long)((r + ((unsigned long long)(e + 1022) << 52)) |
-                                                ((unsigned long long)(neg & 0x80000000u) << 32)));
-    const double v = scalbn((double)r, e - 52);
-    return neg ? -v : v;
-}
-
-// FP64 contexts: weights 0..4 as an exact integer in units of the fourth
-// (|sum| < 2^59 for K <= 4096), the rest in FP32 (below 2^-8 of that unit per product).
-template <int NC> struct DigAcc<8, NC> {
-    long long a[NC];
-    float l[NC];
+// FP64 contexts: weights 0..4 as an exact integer in units of the fourth, 5..9 as one in units of the ninth
+// (|sum| < 2^59 and 2^61 for K <= 4096), into which the tenth is rounded.
+template <int NC> struct DigAcc<11, NC> {
+    long long a[NC], b[NC];
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
-        for (int j = 0; j < NC; ++j) { a[j] = 0; l[j] = 0.f; }
+        for (int j = 0; j < NC; ++j) { a[j] = 0; b[j] = 0; }
     }
-    template <int G> __device__ __forceinline__ void fold(int j, float odd, float even)
+    template <int W> __device__ __forceinline__ void fold(int j, float v)
     {
-        if constexpr (G == 3) {
-            l[j] = __fmaf_rn(odd, 0x1p-24f, l[j]);
-            l[j] = __fmaf_rn(even, 0x1p-16f, l[j]);
-        } else if constexpr (G == 2) {
-            l[j] = __fmaf_rn(odd, 0x1p-8f, l[j]);
-            a[j] += (long long)__float2int_rn(even);
-        } else if constexpr (G == 1) {
-            a[j] += (long long)__float2int_rn(odd) * (1LL << 8);
-            a[j] += (long long)__float2int_rn(even) * (1LL << 16);
-        } else {
-            a[j] += (long long)__float2int_rn(odd) * (1LL << 24);
-            a[j] += (long long)__float2int_rn(even) << 32;
-        }
+        if constexpr (W == 10) b[j] += (long long)__float2int_rn(__fmul_rn(v, 0x1p-8f));
+        else if constexpr (W > 4) b[j] += (long long)__float2int_rn(v) << (8 * (9 - W));
+        else a[j] += (long long)__float2int_rn(v) << (8 * (4 - W));
     }
-    // the sum times 2^e, from the bits (96: units of 2^-24 of the fourth weight's, 2^-9 of what the left-out
-    // pairs may add); in FP64, conversions, sum and scale held the pipe 20000 cycles a product
+    // The sum times 2^e, rounded to nearest, from the bits: in FP64, conversions, sum and scale held the pipe
+    // 20000 cycles a product (a conversion or an addition takes 19 cycles a warp instruction).
     __device__ __forceinline__ double value(int j, int e) const
     {
-        const long long f = __float2ll_rn(__fmul_rn(l[j], 0x1p24f));
-        const Dig96 r{(unsigned)(a[j] << 24), (unsigned)(a[j] >> 8), (int)(a[j] >> 40)};
-        return dig_to_f64(dig_add(r, Dig96{(unsigned)f, (unsigned)(f >> 32), (int)(f >> 63)}), e - 56);
+        // a 2^40 + b in four words
+        const long long c = b[j] >> 40;                                      // what b carries into a
+        const unsigned long long lo = (unsigned long long)(b[j] - (c << 40)), hi = (unsigned long long)(a[j] + c);
+        unsigned h = (unsigned)((long long)hi >> 56), m = (unsigned)(hi >> 24), l = (unsigned)(hi << 8) | (unsigned)(lo >> 32);
+        unsigned t = (unsigned)lo;
+        const unsigned neg = (unsigned)((int)h >> 31);                       // all ones if negative
+        if (neg) {
+            t = ~t + 1u;
+            l = ~l + (t == 0u);
+            m = ~m + (t == 0u && l == 0u);
+            h = ~h + (t == 0u && l == 0u && m == 0u);
+        }
+        if ((h | m | l | t) == 0u) return 0.0;
+        int x = 127 - 72 + e;                                                // weight of the leading bit of (h m l t)
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (h == 0u) { h = m; m = l; l = t; t = 0u; x -= 32; }
+        const int z = __clz((int)h);
+        h = __funnelshift_l(m, h, z);
+        m = __funnelshift_l(l, m, z);
+        l = __funnelshift_l(t, l, z);
+        t <<= z;
+        x -= z;                                                              // value = 1.x 2^x, leading bit at the top of h
+        unsigned long long r = ((unsigned long long)h << 32) | m;
+        const unsigned low = (unsigned)(r & 0x7ffu);
+        r >>= 11;
+        if (low > 0x400u || (low == 0x400u && ((l | t) != 0u || (r & 1u)))) ++r;
+        if (x > -1000 && x < 1000)
+            // (the leading bit of r adds 1 to the exponent field)
+            return __longlong_as_double((long long)((r + ((unsigned long long)(x + 1022) << 52)) |
+                                                    ((unsigned long long)(neg & 0x80000000u) << 32)));
+        const double v = scalbn((double)r, x - 52);
+        return neg ? -v : v;
     }
 };
 
-// Exponent of the power of two above a maximum with high word h (S = 8 keeps one bit of headroom).
-template <int S> __device__ __forceinline__ int dig_exp(int h)
-{
-    return max(h >> 20, 1) - 1022 + (S == 8 ? 1 : 0);
-}
+// Exponent of the power of two above a maximum with high word h.
+__device__ __forceinline__ int dig_exp(int h) { return max(h >> 20, 1) - 1022; }
 
 __device__ __forceinline__ float dig_pow2f(int e)       // 2^e for e <= 127, 0 below 2^-126
 {
@@ -223,11 +210,11 @@ __device__ __forceinline__ double dig_join(float h, float l, int e)     // (h + 
 }
 
 // Biased exponents (+ 2048) of a pulse's two columns in 16-bit halves, bit 15 of a half: not finite.
-template <int S> __device__ __forceinline__ int dig_pack(const int *m)
+__device__ __forceinline__ int dig_pack(const int *m)
 {
     const int2 h = *reinterpret_cast<const int2 *>(m);
-    return (dig_exp<S>(h.x) + 2048 + (h.x >= DIG_NONFINITE ? 0x8000 : 0)) |
-           (int)((unsigned)(dig_exp<S>(h.y) + 2048 + (h.y >= DIG_NONFINITE ? 0x8000 : 0)) << 16);
+    return (dig_exp(h.x) + 2048 + (h.x >= DIG_NONFINITE ? 0x8000 : 0)) |
+           (int)((unsigned)(dig_exp(h.y) + 2048 + (h.y >= DIG_NONFINITE ? 0x8000 : 0)) << 16);
 }
 
 // The shift applied to the first product's sum, in exponents of the two products' units.
@@ -290,8 +277,9 @@ template <int S, int BN, int CG>
 __global__ void __launch_bounds__(DIG_THREADS, 1)
 dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
 {
-    constexpr int NG = S / 2;
+    constexpr int NG = dig_groups(S);
     constexpr int NC = BN / 2;                          // columns per draining thread
+    static_assert(NG <= 6, "groups");
     constexpr int STAGE = dig_stage_bytes(BN, CG);
     constexpr int NST = dig_stages(BN, CG);
 
@@ -353,7 +341,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
     pdl_wait();                                          // state digits and maxima come from the previous kernel
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_low(BN)));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_low(dig_wide(S, BN))));
         if (warp == 0 || warp == 3) {
             // ------- operand loads: warp 0 those of A (rows of U), warp 3 those of B (pulse planes)
             // Whole-warp loops with an elected issuer, as the products below: one
@@ -375,8 +363,9 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                         for (int g = NG - 1; g >= 0 && ok; --g) {
                             const int k1 = min(k0 + DIG_SUPER, nk);
                             for (int kb = k0; kb < k1 && ok; ++kb) {
-                                int z = isb ? 2 * g + 1 : za;                // digit plane of step 0
-                                for (int st = 0; st < 2 * g + 2; ++st, z += dz) {
+                                const int w = dig_top(S, g);
+                                int z = isb ? w : za;                        // digit plane of step 0
+                                for (int st = 0; st <= w; ++st, z += dz) {
                                     if (it >= NST) {
                                         ok = __all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], ph, abort, DIG_WAIT_NS)) != 0;
                                         if (!ok) break;
@@ -421,17 +410,17 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                 for (int part = 0; part < parts && ok; ++part)
                     for (int k0 = 0; k0 < nk && ok; k0 += DIG_SUPER)
                         for (int g = NG - 1; g >= 0 && ok; --g) {
-                            const int k1 = min(k0 + DIG_SUPER, nk);
-                            for (int kc = k0; kc < k1 && ok; kc += dig_chunk(g), ++j) {
+                            const int k1 = min(k0 + DIG_SUPER, nk), w = dig_top(S, g), chunk = dig_chunk(w);
+                            for (int kc = k0; kc < k1 && ok; kc += chunk, ++j) {
                                 const int ab = j & 1;
                                 if (j >= 2 && !wait(&acc_empty[ab], (uint32_t)(((j >> 1) - 1) & 1))) { ok = false; break; }
                                 tc_fence_after();
                                 const uint32_t dodd = tmem + (uint32_t)(ab * 2 * BN), deven = dodd + BN;
-                                const int ke = min(kc + dig_chunk(g), k1);
+                                const int ke = min(kc + chunk, k1);
                                 for (int kb = kc; kb < ke && ok; ++kb) {
                                     uint64_t aprev = d0;
                                     int sprev = s;
-                                    for (int st = 0; st < 2 * g + 2; ++st) {
+                                    for (int st = 0; st <= w; ++st) {
                                         if (!wait(&full[s], ph)) { ok = false; break; }
                                         tc_fence_after();
                                         const uint64_t da = d0 + (uint64_t)(s * (STAGE >> 4)), db = da + (DA_BYTES >> 4);
@@ -446,7 +435,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                                                     mma(deven, aprev + 2 * kk, db + 2 * kk, kk > 0 || st > 1 ? 1u : fresh);
                                                 commit(&empty[sprev]);       // its A was last read here
                                             }
-                                            if (st == 2 * g + 1) commit(&empty[s]);
+                                            if (st == w) commit(&empty[s]);
                                         }
                                         __syncwarp();
                                         aprev = da;
@@ -494,7 +483,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         }
     } else if (warp < 4 + DIG_DRAIN_WARPS) {
         // ------------------------------------------- draining warps 4..11
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(dig_regs_drain(BN)));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(dig_regs_drain(dig_wide(S, BN))));
         const int quarter = warp & 3;                    // TMEM lanes this warp may read
         const int half = (warp - 4) >> 2;                // which half of the tile's columns
         const int ncol = 2 * A.B;
@@ -512,8 +501,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             R.clear();
             const int eu0 = both ? A.eu[(long long)l * n + row] : 0;
             const int eu1 = both ? A.eu[(long long)(A.lmax + l - 1) * n + row] : 0;
-            auto unit = [&](auto gc) {                   // drain one pair of accumulators of group G
-                constexpr int G = decltype(gc)::value;
+            auto unit = [&](auto wc) {                   // drain one pair of accumulators of top weight W
+                constexpr int W = decltype(wc)::value;
                 const int ab = j & 1;
                 bool have = mbar_wait_bounded(&acc_full[ab], (uint32_t)((j >> 1) & 1), abort, DIG_WAIT_NS);
                 have = __all_sync(0xffffffffu, have);
@@ -525,7 +514,15 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                     float vo[8], ve[8];
                     tmem_ld8x2(ta + (uint32_t)(ch * 8), ta + (uint32_t)(BN + ch * 8), vo, ve);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) R.template fold<G>(ch * 8 + q, vo[q], ve[q]);
+                    for (int q = 0; q < 8; ++q) {
+                        if constexpr (W > 2) {           // the smaller first
+                            R.template fold<W>(ch * 8 + q, vo[q]);
+                            R.template fold<W - 1>(ch * 8 + q, ve[q]);
+                        } else {
+                            R.template fold<W>(ch * 8 + q, vo[q]);
+                            if constexpr (W > 0) R.template fold<W - 1>(ch * 8 + q, ve[q]);
+                        }
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -545,17 +542,24 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                 if ((part == 0 && l >= A.lmax) || (part == 1 && l < 1)) continue;
                 for (int k0 = 0; k0 < nk && ok; k0 += DIG_SUPER) {
                     const int k1 = min(k0 + DIG_SUPER, nk);
-                    if constexpr (NG > 3)
-                        for (int kc = k0; kc < k1 && ok; kc += dig_chunk(3)) unit(std::integral_constant<int, 3>{});
-                    if constexpr (NG > 2)
-                        for (int kc = k0; kc < k1 && ok; kc += dig_chunk(2)) unit(std::integral_constant<int, 2>{});
-                    for (int kc = k0; kc < k1 && ok; kc += dig_chunk(1)) unit(std::integral_constant<int, 1>{});
-                    for (int kc = k0; kc < k1 && ok; kc += dig_chunk(0)) unit(std::integral_constant<int, 0>{});
+                    auto group = [&](auto gc) {
+                        constexpr int G = decltype(gc)::value;
+                        if constexpr (G < NG) {
+                            constexpr int W = dig_top(S, G);
+                            for (int kc = k0; kc < k1 && ok; kc += dig_chunk(W)) unit(std::integral_constant<int, W>{});
+                        }
+                    };
+                    group(std::integral_constant<int, 5>{});
+                    group(std::integral_constant<int, 4>{});
+                    group(std::integral_constant<int, 3>{});
+                    group(std::integral_constant<int, 2>{});
+                    group(std::integral_constant<int, 1>{});
+                    group(std::integral_constant<int, 0>{});
                 }
                 if (part == 0 && l >= 1 && ok) {
                     // the second product has other row and column exponents
                     const int *m0 = A.xmax + (long long)(l + 1) * ncol, *m1 = A.xmax + (long long)(l - 1) * ncol;
-                    if constexpr (S == 8) {
+                    if constexpr (dig_int(S)) {
                         claim();
                         if (!ok) break;
 #pragma unroll
@@ -563,8 +567,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                             const int col = c0 + 2 * p;
                             double2 v = make_double2(0.0, 0.0);
                             if (both && col < ncol)
-                                v = make_double2(R.value(2 * p, eu0 + dig_exp<S>(m0[col]) - 14),
-                                                 R.value(2 * p + 1, eu0 + dig_exp<S>(m0[col + 1]) - 14));
+                                v = make_double2(R.value(2 * p, eu0 + dig_exp(m0[col]) - 14),
+                                                 R.value(2 * p + 1, eu0 + dig_exp(m0[col + 1]) - 14));
                             scr[p * DBM].d = v;
                         }
                         R.clear();
@@ -574,7 +578,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                             // rescale the sum so far to the second product's unit (its value below 2^-100 of the
                             // other's unit is lost, far under the digits left out); velocity gauge: minus the second
                             int x = 0;
-                            if (both && c0 + q < ncol) x = dig_shift(eu0 + dig_exp<S>(m0[c0 + q]), eu1 + dig_exp<S>(m1[c0 + q]));
+                            if (both && c0 + q < ncol) x = dig_shift(eu0 + dig_exp(m0[c0 + q]), eu1 + dig_exp(m1[c0 + q]));
                             const float sc = A.gauge ? -dig_pow2f(x) : dig_pow2f(x);
                             R.h[q] = __fmul_rn(R.h[q], sc);
                             R.l[q] = __fmul_rn(R.l[q], sc);
@@ -587,13 +591,13 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             if (!ok) break;
 #pragma unroll
             for (int p = 0; p < NC / 2; ++p) {
-                if constexpr (S == 8) {
+                if constexpr (dig_int(S)) {
                     const int col = c0 + 2 * p;
                     double2 v = make_double2(0.0, 0.0);
                     if (row < n && col < ncol) {
                         const int *m = A.xmax + (long long)(l >= 1 ? l - 1 : l + 1) * ncol + col;
                         const int e = (l >= 1 ? A.eu[(long long)(A.lmax + l - 1) * n + row] : A.eu[(long long)l * n + row]) - 14;
-                        v = make_double2(R.value(2 * p, e + dig_exp<S>(m[0])), R.value(2 * p + 1, e + dig_exp<S>(m[1])));
+                        v = make_double2(R.value(2 * p, e + dig_exp(m[0])), R.value(2 * p + 1, e + dig_exp(m[1])));
                         if (l >= 1 && A.gauge) v = make_double2(-v.x, -v.y);
                         if (both) {
                             const double2 w = scr[p * DBM].d;
@@ -615,7 +619,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         // a scheduler's pipe, so one group alone leaves that pipe idle.  The states
         // of a pulse are staged in shared memory by warp 2 (a load takes some 3500
         // cycles behind the operand tiles), D x is read one pulse ahead.
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_upd(BN)));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(dig_regs_upd(dig_wide(S, BN))));
         const int grp = (warp - 4 - DIG_DRAIN_WARPS) >> 2;
         const int r0 = (warp & 3) * 32 + lane;
         const int ncol = 2 * A.B;
@@ -649,8 +653,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                     // halves, bias 2048, bit 15: not finite); the maxima of column lane % 2 of the group's pulse lane / 2
                     const int pb = b0 + p32 + lane;
                     const double fv = pb < A.B ? __ldg(A.fval + pb) : 0.0;
-                    const int x0 = up && pb < A.B ? dig_pack<S>(A.xmax + (long long)(l + 1) * ncol + 2 * pb) : 0;
-                    const int x1 = dn && pb < A.B ? dig_pack<S>(A.xmax + (long long)(l - 1) * ncol + 2 * pb) : 0;
+                    const int x0 = up && pb < A.B ? dig_pack(A.xmax + (long long)(l + 1) * ncol + 2 * pb) : 0;
+                    const int x1 = dn && pb < A.B ? dig_pack(A.xmax + (long long)(l - 1) * ncol + 2 * pb) : 0;
                     int mine = 0;
                     const int pe = min(p32 + 32, np);
 #pragma unroll 1
@@ -675,7 +679,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                         double d[2];
 #pragma unroll
                         for (int w = 0; w < 2; ++w) {
-                            if constexpr (S == 8) {
+                            if constexpr (dig_int(S)) {
                                 d[w] = w ? o.d.y : o.d.x;
                             } else {
                                 const int e0 = eu0 + ((s0 >> (16 * w)) & 0x7fff), e1 = eu1 + ((s1 >> (16 * w)) & 0x7fff);

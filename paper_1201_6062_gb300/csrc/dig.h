@@ -8,9 +8,9 @@
 
 namespace tdse {
 
-// Digits per operand (8 bits each): 4 for FP32, 6 for float-float, 8 for FP64
+// Digits per operand (8 bits each): 7 for FP32 and float-float, 11 for FP64
 // contexts.  The error bounds are in dig.cuh.
-constexpr int dig_slices(int prec) { return prec == 1 ? 4 : (prec == 2 ? 6 : 8); }
+constexpr int dig_slices(int prec) { return prec == 0 ? 11 : 7; }
 
 // TMA descriptors: dipole digits [2 (U, U^T)][S][lmax][n][ldb] as (K, row,
 // plane) and state digits [S][2B][plane] as (column, pulse plane, digit).
@@ -39,9 +39,8 @@ struct DigTile { int cg, bn; };
 DigTile dig_tile(int slices, int n, int lmax, int B);
 size_t dig_scratch_bytes(DigTile t);
 cudaError_t launch_dig(int slices, DigTile t, const DigMaps &m, const DigArgs &A, cudaStream_t stream);
-const void *dig_fn4(int cg, int bn);
-const void *dig_fn6(int cg, int bn);
-const void *dig_fn8(int cg, int bn);
+const void *dig_fn7(int cg, int bn);
+const void *dig_fn11(int cg, int bn);
 
 // Dipole blocks in the storage format of `prec` -> digits and row exponents
 // (eu must hold 2*lmax*n ints; digits 2*S*lmax*n*ldb bf16, padding zeroed here).
