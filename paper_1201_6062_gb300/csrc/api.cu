@@ -152,10 +152,9 @@ struct tdse_ctx {
     tdse::TcMaps tc_maps{};
     // digit-sliced batches on the tensor cores (FP64 / FP32 / float-float contexts):
     // row exponents and digits of the dipole blocks (built by the first such
-    // batch), the maxima and digits of the states and the field values
-    DevBuf dgE, dgU, dgmax, dgX, dgF;
+    // batch), the maxima and digits of the states and the D x tiles of the CTAs
+    DevBuf dgE, dgU, dgmax, dgX, dgscr;
     bool dg_ready = false;
-    DevBuf dgscr;
     int dg_B = 0;                       // batch size the state digits / maps were built for
     tdse::DigTile dg_tile{};
     tdse::DigMaps dg_maps{};
@@ -474,30 +473,59 @@ static bool dig_wanted(const tdse_ctx *ctx, int B)
     return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
 }
 
+// Gives back the memory a context could do without (the digits of its dipole
+// blocks and of the states, which the slower kernels do not need; FP64: the
+// batched states too); false if it holds none.
+static bool shed(tdse_ctx *c)
+{
+    DevBuf *const optional[] = {&c->dgU, &c->dgE, &c->dgX, &c->dgmax, &c->dgscr, &c->bx, &c->bacc};
+    const int count = c->prec == TDSE_FP64 ? 7 : 5;
+    bool any = false;
+    for (int q = 0; q < count; ++q) any = any || optional[q]->p;
+    if (!any || cudaDeviceSynchronize() != cudaSuccess) return false;
+    for (int q = 0; q < count; ++q) optional[q]->release();
+    c->dg_ready = false;
+    c->dg_B = 0;
+    return true;
+}
+
 // Device storage, dipole digits and tensor maps of a digit-sliced batch; false
 // when they cannot be had (memory, or a stream under capture before the
-// digits exist): the caller then takes the FMA-pipe path.
-static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
+// digits exist): the caller then takes the pipe kernels' path, which finds the
+// memory as if there were no digits.
+static bool dig_prepare(tdse_ctx *ctx, int B, cudaStream_t s)
 {
     const int S = tdse::dig_slices(ctx->prec), L = ctx->lmax + 1, n = ctx->n;
     const int ldb = (n + 7) & ~7, nb = (n + 63) & ~63;
     const tdse::DigTile tile = tdse::dig_tile(S, n, ctx->lmax, B);
     const long long plane = (long long)L * nb;
-    const size_t ub = sizeof(__nv_bfloat16) * 2 * S * (size_t)ctx->lmax * n * ldb;
+    struct Need { DevBuf *buf; size_t bytes; bool optional; };
+    const size_t vb = sizeof(double2) * (size_t)B * ctx->N;
     const size_t xb = sizeof(__nv_bfloat16) * S * 2 * (size_t)B * plane;
+    const Need need[] = {
+        {&ctx->dgE, sizeof(int) * 2 * (size_t)ctx->lmax * n, true},
+        {&ctx->dgU, sizeof(__nv_bfloat16) * 2 * S * (size_t)ctx->lmax * n * ldb, true},
+        {&ctx->dgX, xb, true},
+        {&ctx->dgmax, sizeof(int) * 2 * 2 * (size_t)B * L, true},
+        {&ctx->dgscr, tdse::dig_scratch_bytes(tile), true},
+        {&ctx->bx, vb, ctx->prec == TDSE_FP64},
+        {&ctx->bacc, vb, ctx->prec == TDSE_FP64},
+    };
+    size_t extra = 0;
+    bool grown = false;
+    for (const Need &q : need)
+        if (q.buf->bytes < q.bytes) {
+            grown = true;
+            if (q.optional) extra += q.bytes;
+        }
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return false;
-    const bool grown = ctx->dgX.bytes < xb || ctx->bx.bytes < sizeof(double2) * (size_t)B * ctx->N ||
-                       ctx->dgF.bytes < sizeof(double) * 3 * (size_t)B * nsteps;
     if (cap != cudaStreamCaptureStatusNone && (!ctx->dg_ready || ctx->dg_B != B || grown)) return false;
-    bool ok = ctx->bx.ensure(sizeof(double2) * (size_t)B * ctx->N) == cudaSuccess &&
-              ctx->bacc.ensure(sizeof(double2) * (size_t)B * ctx->N) == cudaSuccess &&
-              ctx->dgmax.ensure(sizeof(int) * 2 * 2 * (size_t)B * L) == cudaSuccess &&
-              ctx->dgF.ensure(sizeof(double) * 3 * (size_t)B * nsteps) == cudaSuccess;
+    if (extra > 0 && !optional_room(extra)) return false;
+    bool ok = true;
+    for (const Need &q : need) ok = ok && q.buf->ensure(q.bytes) == cudaSuccess;
     if (ok && !ctx->dg_ready) {
-        ok = optional_room(ub) && ctx->dgE.ensure(sizeof(int) * 2 * (size_t)ctx->lmax * n) == cudaSuccess &&
-             ctx->dgU.ensure(ub) == cudaSuccess &&
-             tdse::launch_dig_u(ctx->prec, ctx->U.p, ctx->bstride, ctx->ld, n, ctx->lmax, ldb, ctx->dgE.as<int>(),
+        ok = tdse::launch_dig_u(ctx->prec, ctx->U.p, ctx->bstride, ctx->ld, n, ctx->lmax, ldb, ctx->dgE.as<int>(),
                                 ctx->dgU.as<__nv_bfloat16>(), s) == cudaSuccess;
         const cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)(2 * S * ctx->lmax)};
         const cuuint64_t strides[2] = {(cuuint64_t)ldb * 2, (cuuint64_t)n * ldb * 2};
@@ -507,8 +535,7 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
         ctx->launches += 3;
     }
     if (ok && ctx->dg_B != B) {
-        ok = ctx->dgX.ensure(xb) == cudaSuccess && ctx->dgscr.ensure(tdse::dig_scratch_bytes(tile)) == cudaSuccess &&
-             cudaMemsetAsync(ctx->dgX.p, 0, xb, s) == cudaSuccess;   // padding columns stay zero
+        ok = cudaMemsetAsync(ctx->dgX.p, 0, xb, s) == cudaSuccess;      // padding columns stay zero
         const cuuint64_t dims[3] = {(cuuint64_t)plane, (cuuint64_t)(2 * B), (cuuint64_t)S};
         const cuuint64_t strides[2] = {(cuuint64_t)plane * 2, (cuuint64_t)(2 * B) * plane * 2};
         const cuuint32_t box[3] = {64, (cuuint32_t)(tile.bn / tile.cg), 1};
@@ -519,25 +546,9 @@ static bool dig_prepare(tdse_ctx *ctx, int B, long nsteps, cudaStream_t s)
     if (!ok) {
         (void)cudaGetLastError();
         g_err.clear();
-        if (!ctx->dg_ready) { ctx->dgU.release(); ctx->dgE.release(); }
-        ctx->dgX.release();
-        ctx->dg_B = 0;
-        if (ctx->prec == TDSE_FP64) { ctx->bx.release(); ctx->bacc.release(); }      // (the pulse-by-pulse path has no use for them)
+        (void)shed(ctx);
     }
     return ok;
-}
-
-// Gives back the memory a context could do without (the digits of its dipole
-// blocks, which the slower kernels do not need); false if it holds none.
-static bool shed(tdse_ctx *c)
-{
-    if (!c->dgU.p || cudaDeviceSynchronize() != cudaSuccess) return false;
-    c->dgU.release();
-    c->dgE.release();
-    c->dgX.release();
-    c->dg_ready = false;
-    c->dg_B = 0;
-    return true;
 }
 
 // A call that may allocate: once more without the optional memory when there
@@ -559,9 +570,8 @@ static tdse_status propagate_batch_dig(tdse_ctx *ctx, double *c, const double *f
     int *xm = ctx->dgmax.as<int>();
     const size_t slot = (size_t)L * 2 * B;
     CUDA_TRY(cudaMemsetAsync(xm, 0, sizeof(int) * slot, s));
-    CUDA_TRY(tdse::launch_dig_field(field, (int)((long)sps * nsteps + 1), sps, nsteps, B, ctx->dgF.as<double>(), s));
     CUDA_TRY(tdse::launch_dig_max((const double2 *)c, n, ctx->lmax, B, xm, s));
-    ctx->launches += 2;
+    ctx->launches += 1;
     tdse::DigArgs A{};
     A.n = n;
     A.lmax = ctx->lmax;
@@ -570,6 +580,9 @@ static tdse_status propagate_batch_dig(tdse_ctx *ctx, double *c, const double *f
     A.N = ctx->N;
     A.E = ctx->E.as<double>();
     A.eu = ctx->dgE.as<int>();
+    A.field = field;
+    A.S = (int)((long)sps * nsteps + 1);
+    A.sps = sps;
     A.c = (double2 *)c;
     A.x = ctx->bx.as<double2>();
     A.acc = ctx->bacc.as<double2>();
@@ -582,10 +595,10 @@ static tdse_status propagate_batch_dig(tdse_ctx *ctx, double *c, const double *f
     long t = 0;
     for (long k = 0; k < nsteps; ++k) {
         for (int q = q0; q <= q1; ++q, ++t) {
-            const int h = scheme == TDSE_RK4 ? (q == 0 ? 0 : (q == 3 ? 2 : 1)) : (hold ? 1 : 0);
+            A.k = k;
+            A.h = scheme == TDSE_RK4 ? (q == 0 ? 0 : (q == 3 ? 2 : 1)) : (hold ? 1 : 0);
             A.stage = q;
             A.step = scheme == TDSE_RK4 ? (q == 3 ? dt / 6.0 : (q == 2 ? dt : 0.5 * dt)) : dt / (double)q;
-            A.fval = ctx->dgF.as<double>() + ((size_t)k * 3 + h) * B;
             A.xmax = xm + (t & 1) * slot;
             A.xmax_next = xm + ((t + 1) & 1) * slot;
             CUDA_TRY(tdse::launch_dig_x(S, q == q0 ? A.c : A.x, n, nb, ctx->lmax, B, A.xmax, A.xmax_next,
@@ -1358,7 +1371,7 @@ static tdse_status propagate_batch_once(tdse_ctx *ctx, double *c, const double *
         if (nsteps == 0) return TDSE_OK;
         return propagate_batch_tc(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, s);
     }
-    if (scheme != TDSE_LANCZOS && nsteps > 0 && dig_wanted(ctx, B) && dig_prepare(ctx, B, nsteps, s))
+    if (scheme != TDSE_LANCZOS && nsteps > 0 && dig_wanted(ctx, B) && dig_prepare(ctx, B, s))
         return propagate_batch_dig(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, s);
     if (ctx->prec == TDSE_DF32 && scheme != TDSE_LANCZOS) {
         if (nsteps == 0) return TDSE_OK;

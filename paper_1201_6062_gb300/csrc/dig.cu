@@ -223,23 +223,6 @@ cudaError_t launch_dig_x(int slices, const double2 *src, int n, int nb, int lmax
     return launch_pdl(fn, dim3((n + 511) / 512, lmax + 1, B), dim3(128), 0, s, args);
 }
 
-__global__ void dig_field_kernel(const double *__restrict__ field, int S, int sps, long long nsteps, int B,
-                                 double *__restrict__ fval)
-{
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nsteps * 3 * B) return;
-    const long long kh = q / B;
-    fval[q] = field_at(field + (q % B) * S, sps, kh / 3, (int)(kh % 3));
-}
-
-cudaError_t launch_dig_field(const double *field, int S, int sps, long long nsteps, int B, double *fval, cudaStream_t s)
-{
-    const long long tot = nsteps * 3 * B;
-    if (tot <= 0) return cudaSuccess;
-    dig_field_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(field, S, sps, nsteps, B, fval);
-    return cudaGetLastError();
-}
-
 // ----------------------------------------------------------------- launch --
 static int dig_sms()
 {

@@ -652,7 +652,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
                     // pulse b0 + p32 + lane: field value, exponents of the columns of the two products (two 16-bit
                     // halves, bias 2048, bit 15: not finite); the maxima of column lane % 2 of the group's pulse lane / 2
                     const int pb = b0 + p32 + lane;
-                    const double fv = pb < A.B ? __ldg(A.fval + pb) : 0.0;
+                    const double fv = pb < A.B ? field_at(A.field + (long long)pb * A.S, A.sps, A.k, A.h) : 0.0;
                     const int x0 = up && pb < A.B ? dig_pack(A.xmax + (long long)(l + 1) * ncol + 2 * pb) : 0;
                     const int x1 = dn && pb < A.B ? dig_pack(A.xmax + (long long)(l - 1) * ncol + 2 * pb) : 0;
                     int mine = 0;

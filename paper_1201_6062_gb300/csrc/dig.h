@@ -23,7 +23,9 @@ struct DigArgs {
     long long N;            // amplitudes per pulse
     const double *E;        // [N]
     const int *eu;          // [2][lmax][n]: exponents of the rows of U_l and U_l^T
-    const double *fval;     // this stage's field value per pulse [B]
+    const double *field;    // samples [B][S]; this stage's value is field_at(.., sps, k, h)
+    int S, sps, h;
+    long long k;
     double2 *c, *x, *acc;   // FP64 states [B][N]
     const int *xmax;        // [lmax+1][2B]: high word of max |x| per (block, plane), this stage's input
     int *xmax_next;         // the same of the next stage's input (atomicMax; cleared before the launch)
@@ -51,8 +53,5 @@ cudaError_t launch_dig_max(const double2 *src, int n, int lmax, int B, int *xmax
 // States src [B][N] -> digits [S][2B][plane], scaled by xmax; clears xmax_next.
 cudaError_t launch_dig_x(int slices, const double2 *src, int n, int nb, int lmax, int B, const int *xmax,
                          int *xmax_next, __nv_bfloat16 *digits, cudaStream_t stream);
-// fval[(k*3 + h)*B + b] = f_b(t_k + h dt/2).
-cudaError_t launch_dig_field(const double *field, int S, int sps, long long nsteps, int B, double *fval,
-                             cudaStream_t stream);
 
 }  // namespace tdse

@@ -224,3 +224,65 @@ def test_small_components_keep_their_digits(tdse_lib, prec, what):
         got = (c[b].cpu().numpy().reshape(x.shape).astype(np.clongdouble) - x) * 1j / np.longdouble(F)
         err = np.abs(got - ref).astype(np.float64)
         assert np.all(err <= own_bound(prec, n) * own), float((err / own).max())
+
+
+def run_batch(H, B, steps, dt=0.01):
+    N = H.N
+    c = torch.from_numpy(np.stack([inputs.random_state(N, b) for b in range(B)])).cuda()
+    H.propagate_batch(c, torch.full((B, steps + 1), 0.1, dtype=torch.float64, device="cuda"), B, dt, steps)
+    H.sync()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+def test_the_workspace_does_not_grow_with_the_steps(tdse_lib, prec):
+    lmax, n, B = 2, 100, 16
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, prec)
+    run_batch(H, B, 2)
+    used = tdse_lib.device_memory_in_use()
+    run_batch(H, B, 200)
+    assert tdse_lib.device_memory_in_use() == used
+    H.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+def test_no_workspace_of_digits_stays_where_the_other_path_serves(tdse_lib, prec):
+    """Under a cap that leaves the digits no room, a batch holds what the pipe kernels need and no more, so
+    that a cap of just that serves it (what the digits took first would be missing)."""
+    lmax, n, B = 2, 200, 64
+    N = (lmax + 1) * n
+    words = {"fp32": 2, "df32": 4, "fp64": 0}[prec]               # of four bytes, twice: the products' inputs
+    own = 2 * 16 * B * N + 2 * 4 * words * B * N + 3 * 2 * 4 * B if prec != "fp64" else 4096
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, prec)
+    used = tdse_lib.device_memory_in_use()
+    tdse_lib.set_device_memory_limit(used + own)
+    try:
+        run_batch(H, B, 2)
+        assert tdse_lib.device_memory_in_use() <= used + own
+    finally:
+        tdse_lib.set_device_memory_limit(0)
+    H.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+def test_other_calls_get_the_digits_memory(tdse_lib, prec):
+    """A call that runs out of memory while its context holds digits succeeds without them."""
+    lmax, n, B, steps = 2, 200, 64, 8
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, prec)
+    before = tdse_lib.device_memory_in_use()
+    c0 = torch.from_numpy(inputs.random_state(H.N, 1)).cuda()
+    F = torch.full((steps + 1,), 0.1, dtype=torch.float64, device="cuda")
+    w = torch.ones(H.N, dtype=torch.float64, device="cuda")
+    want = H.adjoint(c0, F, 0.01, steps, w)[0].clone()
+    need = tdse_lib.device_memory_in_use() - before
+    H.close()
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, prec)
+    run_batch(H, B, 2)
+    held = tdse_lib.device_memory_in_use()
+    tdse_lib.set_device_memory_limit(held + need // 2)
+    try:
+        got = H.adjoint(c0, F, 0.01, steps, w)[0]
+        assert torch.equal(got, want)
+        assert tdse_lib.device_memory_in_use() < held
+    finally:
+        tdse_lib.set_device_memory_limit(0)
+    H.close()
