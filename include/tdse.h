@@ -217,8 +217,10 @@ tdse_status tdse_populations(tdse_ctx *ctx, const double *c, int B, double *per_
  *           are exact; what is left out is below 2^-53 (FP32, DF32) or 2^-84
  *           of the largest dipole element of the row times the largest
  *           amplitude of the block, per product.  The digits of the blocks are
- *           made at a context's first batch and kept.  Where
- *           their memory cannot be had, or rows are short (n < 56) and pulses
+ *           made at a context's first batch and kept until another call of
+ *           the context runs out of memory (for good once a batch has been
+ *           captured into a graph, which replays on them).  Where their
+ *           memory cannot be had, or rows are short (n < 56) and pulses
  *           many, or FP64 pulses few: FP32 and DF32 on the FMA pipe (DF32:
  *           float-float), FP64 pulse by pulse on the single-system path (as
  *           does TDSE_LANCZOS on FP64 and DF32 contexts; FP32 and BF16X3

@@ -70,6 +70,8 @@ static std::atomic<long long> g_dev_limit{0};
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    DevBuf() = default;
+    DevBuf(DevBuf &&o) noexcept : p(o.p), bytes(o.bytes) { o.p = nullptr; o.bytes = 0; }
     ~DevBuf() { release(); }
     void release()
     {
@@ -156,6 +158,8 @@ struct tdse_ctx {
     DevBuf dgE, dgU, dgmax, dgX, dgscr;
     bool dg_ready = false;
     int dg_B = 0;                       // batch size the state digits / maps were built for
+    bool dg_captured = false;           // a caller's graph holds launches on this memory
+    std::vector<DevBuf> dg_kept;        // buffers outgrown since
     tdse::DigTile dg_tile{};
     tdse::DigMaps dg_maps{};
     int tc_persistent = 1;              // all stages of a batch in one launch (tdse_set_batch_persistent)
@@ -473,11 +477,21 @@ static bool dig_wanted(const tdse_ctx *ctx, int B)
     return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
 }
 
+// A batch's workspace.  Once a batch has been captured into a caller's graph,
+// a buffer that is outgrown stays: a replay still works on it.
+static cudaError_t batch_ensure(tdse_ctx *c, DevBuf &b, size_t nbytes)
+{
+    if (c->dg_captured && b.p && b.bytes < nbytes) c->dg_kept.push_back(std::move(b));
+    return b.ensure(nbytes);
+}
+
 // Gives back the memory a context could do without (the digits of its dipole
 // blocks and of the states, which the slower kernels do not need; FP64: the
-// batched states too); false if it holds none.
+// batched states too); false if it holds none, or if a caller's graph works on
+// it.
 static bool shed(tdse_ctx *c)
 {
+    if (c->dg_captured) return false;
     DevBuf *const optional[] = {&c->dgU, &c->dgE, &c->dgX, &c->dgmax, &c->dgscr, &c->bx, &c->bacc};
     const int count = c->prec == TDSE_FP64 ? 7 : 5;
     bool any = false;
@@ -523,7 +537,7 @@ static bool dig_prepare(tdse_ctx *ctx, int B, cudaStream_t s)
     if (cap != cudaStreamCaptureStatusNone && (!ctx->dg_ready || ctx->dg_B != B || grown)) return false;
     if (extra > 0 && !optional_room(extra)) return false;
     bool ok = true;
-    for (const Need &q : need) ok = ok && q.buf->ensure(q.bytes) == cudaSuccess;
+    for (const Need &q : need) ok = ok && batch_ensure(ctx, *q.buf, q.bytes) == cudaSuccess;
     if (ok && !ctx->dg_ready) {
         ok = tdse::launch_dig_u(ctx->prec, ctx->U.p, ctx->bstride, ctx->ld, n, ctx->lmax, ldb, ctx->dgE.as<int>(),
                                 ctx->dgU.as<__nv_bfloat16>(), s) == cudaSuccess;
@@ -546,8 +560,9 @@ static bool dig_prepare(tdse_ctx *ctx, int B, cudaStream_t s)
     if (!ok) {
         (void)cudaGetLastError();
         g_err.clear();
-        (void)shed(ctx);
+        if (!shed(ctx)) ctx->dg_B = 0;
     }
+    if (ok && cap != cudaStreamCaptureStatusNone) ctx->dg_captured = true;
     return ok;
 }
 
@@ -1301,8 +1316,8 @@ static tdse_status propagate_batch_df(tdse_ctx *ctx, double *c, const double *fi
 {
     const long long N = ctx->N;
     const long S = (long)sps * nsteps + 1;
-    CUDA_TRY(ctx->bx.ensure(sizeof(double2) * (size_t)B * N));
-    CUDA_TRY(ctx->bacc.ensure(sizeof(double2) * (size_t)B * N));
+    CUDA_TRY(batch_ensure(ctx, ctx->bx, sizeof(double2) * (size_t)B * N));
+    CUDA_TRY(batch_ensure(ctx, ctx->bacc, sizeof(double2) * (size_t)B * N));
     CUDA_TRY(ctx->bq.ensure(sizeof(float2) * 2 * 2 * (size_t)B * N));
     CUDA_TRY(ctx->bxmax.ensure(sizeof(int) * 3 * 2 * (size_t)B));
     CUDA_TRY(cudaMemsetAsync(ctx->bxmax.p, 0, sizeof(int) * 3 * 2 * (size_t)B, s));
@@ -1388,8 +1403,8 @@ static tdse_status propagate_batch_once(tdse_ctx *ctx, double *c, const double *
         return TDSE_OK;
     }
     if (nsteps == 0) return TDSE_OK;
-    CUDA_TRY(ctx->bx.ensure(sizeof(double2) * (size_t)B * N));
-    CUDA_TRY(ctx->bacc.ensure(sizeof(double2) * (size_t)B * N));
+    CUDA_TRY(batch_ensure(ctx, ctx->bx, sizeof(double2) * (size_t)B * N));
+    CUDA_TRY(batch_ensure(ctx, ctx->bacc, sizeof(double2) * (size_t)B * N));
     CUDA_TRY(ctx->bq.ensure(sizeof(float) * 2 * 2 * (size_t)B * N));
     float *q0 = ctx->bq.as<float>();
     float *q1 = q0 + 2 * (size_t)B * N;

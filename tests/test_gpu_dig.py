@@ -286,3 +286,42 @@ def test_other_calls_get_the_digits_memory(tdse_lib, prec):
     finally:
         tdse_lib.set_device_memory_limit(0)
     H.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
+def test_a_captured_batch_outlives_later_calls(tdse_lib, prec):
+    """A batch recorded in a caller's graph replays on the memory it was recorded with: after a larger batch
+    of the same context, after one of another tile and after a call that ran out of memory."""
+    lmax, n, B, steps, dt = 2, 200, 16, 2, 0.01
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, prec)
+    c0 = torch.from_numpy(np.stack([inputs.random_state(H.N, b) for b in range(B)])).cuda()
+    F = torch.full((B, steps + 1), 0.1, dtype=torch.float64, device="cuda")
+    c = c0.clone()
+    H.propagate_batch(c, F, B, dt, steps)
+    H.sync()
+    want = c.clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        H.propagate_batch(c, F, B, dt, steps)
+
+    def replay():
+        c.copy_(c0)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(c, want)
+
+    replay()
+    for other in (3, 200, 3):
+        run_batch(H, other, 1)
+        replay()
+    used = tdse_lib.device_memory_in_use()
+    tdse_lib.set_device_memory_limit(used + 1024)
+    try:
+        with pytest.raises(tdse_lib.TDSEError):
+            H.adjoint(c0[0], F[0], dt, steps, torch.ones(H.N, dtype=torch.float64, device="cuda"))
+        assert tdse_lib.device_memory_in_use() >= used
+    finally:
+        tdse_lib.set_device_memory_limit(0)
+    replay()
+    del g
+    H.close()
