@@ -221,10 +221,11 @@ tdse_status tdse_populations(tdse_ctx *ctx, const double *c, int B, double *per_
  *           the context runs out of memory (for good once a batch has been
  *           captured into a graph, which replays on them).  Where their
  *           memory cannot be had, or rows are short (n < 56) and pulses
- *           many, or FP64 pulses few: FP32 and DF32 on the FMA pipe (DF32:
- *           float-float), FP64 pulse by pulse on the single-system path (as
- *           does TDSE_LANCZOS on FP64 and DF32 contexts; FP32 and BF16X3
- *           contexts return ENOTSUP for it).
+ *           many (FP32 more than 4, DF32 more than 32), or FP64 pulses few
+ *           (fewer than 3 to 12, by the size of the blocks): FP32 and DF32 on
+ *           the FMA pipe (DF32: float-float), FP64 pulse by pulse on the
+ *           single-system path (as does TDSE_LANCZOS on FP64 and DF32
+ *           contexts; FP32 and BF16X3 contexts return ENOTSUP for it).
  *   BF16X3  tcgen05 tensor-core GEMM of bf16 hi/lo splits (3 products).
  *   c      device, complex [B][N], in/out.
  *   field  device, FP64 [B][samples_per_step*nsteps + 1].

@@ -466,15 +466,24 @@ static tdse_status propagate_batch_tc(tdse_ctx *ctx, double *c, const double *fi
 // ------------------------------------------- digit-sliced batches (dig.cuh) --
 // Whether a batch of B pulses runs as digit-sliced products on the tensor
 // cores.  Against the FMA-pipe GEMMs (FP32, float-float) they win at every
-// measured shape (lmax=15, n=1000, 256 pulses 502 against 3645 us a stage
-// float-float, 317 against 945 us FP32) but short rows with many pulses, where
-// most of a 128-row tile is padding (FP32, n=40, 200 pulses: 40 against 36 us;
-// n=56, 300: 38).  FP64 batches otherwise run pulse by pulse: a stage of lmax=7,
-// n=301 takes 24 us a pulse and 62 us for 6 pulses here.
+// measured shape (lmax=15, n=1000, 256 pulses 632 against 3637 us a stage
+// float-float, 628 against 945 us FP32) but short rows with many pulses, where
+// most of a 128-row tile is padding (lmax=9, n=48: FP32, 4, 16, 32, 300 pulses
+// 19.7, 25.8, 26.1, 40.4 against 24.4, 25.0, 25.9, 40.3, at n=40 25.7 against 24.1
+// for 16, at n=56 25.9 against 28.2; float-float 32 and 300 pulses 26.1 and 40.4
+// against 36.2 and 36.3).  FP64 batches otherwise run pulse by pulse, a system
+// that fits one cluster at 3-5 us a stage: the products pay from a number of
+// pulses on that falls with the size of the blocks.  Measured at lmax, n, us a
+// stage here and a pulse there: 3, 50 40 (12 pulses) and 4.0; 7, 64 39 (8) and 5.2;
+// 7, 100 59 (8) and 8.3; 7, 200 82 (6) and 14; 7, 301 96 (4) and 24; 15, 500 151
+// (4) and 45; 15, 1000 372 (3) and 148; 31, 2000 3095 (3) and 1041.
 static bool dig_wanted(const tdse_ctx *ctx, int B)
 {
     if (ctx->lmax < 1) return false;
-    return ctx->prec == TDSE_FP64 ? B >= 3 : ctx->n >= 56 || B <= 32;
+    if (ctx->prec == TDSE_FP32) return ctx->n >= 56 || B <= 4;
+    if (ctx->prec == TDSE_DF32) return ctx->n >= 56 || B <= 32;
+    const long long elems = (long long)ctx->lmax * ctx->n * ctx->n;
+    return B >= (elems < 50000 ? 12 : elems < 150000 ? 8 : elems < 500000 ? 6 : elems < 2000000 ? 5 : elems < 8000000 ? 4 : 3);
 }
 
 // A batch's workspace.  Once a batch has been captured into a caller's graph,

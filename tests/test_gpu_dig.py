@@ -183,7 +183,7 @@ def own_bound(prec, n):
 @pytest.mark.parametrize("what", ["dominant", "hydrogen"])
 def test_small_components_keep_their_digits(tdse_lib, prec, what):
     """Bound states: one amplitude near 1, the others of its block far below it."""
-    lmax, n, B = 3, 301, 4
+    lmax, n, B = 3, 301, 8
     rng = np.random.default_rng(9)
     x = np.zeros((lmax + 1, n), np.complex128)
     if what == "dominant":
@@ -324,4 +324,26 @@ def test_a_captured_batch_outlives_later_calls(tdse_lib, prec):
         tdse_lib.set_device_memory_limit(0)
     replay()
     del g
+    H.close()
+
+
+@pytest.mark.parametrize("lmax,n,few,many", [(3, 50, 11, 12), (7, 100, 7, 8), (3, 301, 5, 6)])
+def test_few_fp64_pulses_run_one_by_one(tdse_lib, lmax, n, few, many):
+    """Below the number of pulses from which the digit products pay, a stage of an FP64 batch takes no launch
+    of its own (the kernels of one system hold all stages); above, it takes two.  Both give the same states."""
+    steps, dt = 20, 0.01
+    E, U = inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8)
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, "fp64")
+    C = np.stack([inputs.random_state(H.N, b) for b in range(many)])
+    F = torch.full((many, steps + 1), 0.1, dtype=torch.float64, device="cuda")
+    out = []
+    for B in (few, many):
+        H.profile_read()
+        c = torch.from_numpy(C[:B].copy()).cuda()
+        H.propagate_batch(c, F[:B].clone(), B, dt, steps)
+        launches = H.profile_read()[2]
+        assert launches <= 4 * B + 4 if B == few else launches >= 8 * steps
+        out.append(c.cpu().numpy())
+    # 80 stages, each rounding once: the states agree to their FP64 rounding
+    assert np.linalg.norm(out[0] - out[1][:few]) <= 80 * 2.0 ** -52 * np.linalg.norm(out[0])
     H.close()
