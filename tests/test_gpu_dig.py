@@ -1,7 +1,9 @@
 """The digit-sliced batched products (csrc/dig.cuh) at the edges of their
-tiles: rows (128, 256), K rounds (64, 512), pulses per tile (16, 32, 64), end
-blocks, both gauges, graded and zero states, non-finite states, and the path
-that takes over when their storage cannot be had."""
+tiles: rows (128, 256), K rounds (64, 512), pulses per tile, end blocks, every
+tile shape with several tiles a CTA, both gauges, bound, graded, zero and
+non-finite states, and the paths and memory around them."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -68,7 +70,7 @@ def check(prec, lmax, n, U, C, k, gauge="length"):
         assert np.all(nrm <= NORM[prec] * np.linalg.norm(ref, axis=1) + 1e-300), (l, nrm / np.linalg.norm(ref, axis=1))
 
 
-SHAPES = [(1, 64, 1), (2, 65, 16), (1, 127, 17), (3, 128, 32), (1, 129, 33), (2, 200, 64), (1, 256, 65), (1, 257, 3),
+SHAPES = [(1, 64, 1), (2, 65, 16), (1, 127, 17), (3, 128, 32), (1, 129, 33), (2, 200, 64), (1, 256, 65), (1, 257, 9),
           (2, 513, 9), (1, 640, 40)]
 
 
@@ -78,6 +80,75 @@ def test_products_at_tile_edges(tdse_lib, prec, lmax, n, B):
     U, C = draw(prec, lmax, n, B, 11 * n + B)
     C *= 1e3                                      # the products, not c, set the size of the result
     check(prec, lmax, n, U * 1024, C, product(tdse_lib, prec, lmax, n, U * 1024, C))
+
+
+class Tile(ctypes.Structure):
+    _fields_ = [("cg", ctypes.c_int), ("bn", ctypes.c_int)]
+
+
+# (precisions, lmax, n, pulses): the tile (CTAs of 128 rows, pulse planes) the launch chooses, and more tiles than
+# CTAs or pairs, so that a CTA hands its scratch tile, state slots and accumulators on from one tile to the next
+WALKS = [(("fp32", "df32"), 90, 130, 16, (2, 32)), (("fp32", "df32"), 80, 130, 33, (2, 64)),
+         (("fp32", "df32"), 20, 200, 300, (2, 128)), (("fp32", "df32"), 80, 64, 33, (1, 32)),
+         (("fp32", "df32"), 40, 70, 130, (1, 64)), (("fp64",), 80, 130, 15, (2, 32)), (("fp64",), 80, 130, 33, (2, 64)),
+         (("fp64",), 90, 64, 33, (1, 32)), (("fp64",), 50, 70, 100, (1, 64))]
+WALKS = [(p,) + w[1:] for w in WALKS for p in w[0]]
+
+
+def assert_walk(T, prec, lmax, n, B, tile):
+    choose = T._lib._ZN4tdse8dig_tileEiiii
+    choose.restype, choose.argtypes = Tile, [ctypes.c_int] * 4
+    t = choose(DIGITS[prec], n, lmax, B)
+    assert (t.cg, t.bn) == tile
+    tiles = -(-n // (128 * t.cg)) * -(-2 * B // t.bn) * (lmax + 1)
+    assert tiles > torch.cuda.get_device_properties(0).multi_processor_count // t.cg
+
+
+@pytest.mark.parametrize("prec,lmax,n,B,tile", WALKS)
+def test_several_tiles_a_cta(tdse_lib, prec, lmax, n, B, tile):
+    assert_walk(tdse_lib, prec, lmax, n, B, tile)
+    for gauge in ("length", "velocity"):
+        U, C = draw(prec, lmax, n, B, n + B)
+        C *= 1e3
+        check(prec, lmax, n, U * 1024, C, product(tdse_lib, prec, lmax, n, U * 1024, C, gauge), gauge)
+
+
+@pytest.mark.parametrize("prec,lmax,n,B,tile", WALKS)
+@pytest.mark.parametrize("scheme", ["rk4", "taylor"])
+def test_steps_over_several_tiles(tdse_lib, prec, lmax, n, B, tile, scheme):
+    assert_walk(tdse_lib, prec, lmax, n, B, tile)
+    dt, order = 0.01, 4 if scheme == "rk4" else 3
+    U, C = draw(prec, lmax, n, B, n + B + 1)
+    C /= np.linalg.norm(C, axis=1)[:, None]
+    E = inputs.energies(lmax, n)
+    F = 0.05 + 0.01 * np.random.default_rng(7).random((B, 2))
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, prec)
+    c = torch.from_numpy(C.copy()).cuda()
+    H.propagate_batch(c, torch.from_numpy(F).cuda(), B, dt, 1, scheme, order=order)
+    H.sync()
+    H.close()
+
+    def g(y, f):
+        x = y.reshape(B, lmax + 1, n)
+        d = np.zeros_like(x)
+        d[:, :-1] += np.einsum("lij,blj->bli", U, x[:, 1:], optimize=True)
+        d[:, 1:] += np.einsum("lij,bli->blj", U, x[:, :-1], optimize=True)
+        return -1j * (E * y + f[:, None] * d.reshape(B, -1))
+
+    if scheme == "rk4":
+        fm = 0.5 * (F[:, 0] + F[:, 1])
+        k1 = g(C, F[:, 0])
+        k2 = g(C + 0.5 * dt * k1, fm)
+        k3 = g(C + 0.5 * dt * k2, fm)
+        ref = C + dt / 6.0 * (k1 + 2.0 * k2 + 2.0 * k3 + g(C + dt * k3, F[:, 1]))
+    else:
+        term = ref = C
+        for m in range(1, order + 1):
+            term = dt / m * g(term, F[:, 0])
+            ref = ref + term
+    # a step changes the state by dt (|E| + f |D|) of it at most; products as in NORM, FP64 rounding of the rest
+    err = np.linalg.norm(c.cpu().numpy() - ref, axis=1)
+    assert np.all(err <= 4 * (dt * 0.06 * 4 * NORM[prec] + 8 * 2.0 ** -53)), err.max()
 
 
 @pytest.mark.parametrize("prec", ["fp32", "df32", "fp64"])
