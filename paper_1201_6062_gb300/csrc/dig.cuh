@@ -295,7 +295,7 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag;
     __shared__ int issued[2], consumed;
-    __shared__ int st_issued, st_used[DIG_UPD_GROUPS];
+    __shared__ int st_issued;
     unsigned char *slots = smem + (size_t)NST * STAGE;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform)
@@ -324,7 +324,6 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         }
         mbar_init(&mma_drain, 1);
         st_issued = 0;
-        st_used[0] = st_used[1] = 0;
         abort_flag = 0;
         issued[0] = issued[1] = 0;
         consumed = 0;
@@ -720,7 +719,6 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
             __syncwarp();
             if (lane == 0) mbar_arrive(&d_empty);
         }
-        if ((warp & 3) == 0 && lane == 0) st_used[grp] = it0;
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) {
@@ -729,7 +727,8 @@ dig_kernel(const __grid_constant__ DigMaps M, const DigArgs A)
         volatile int never = 0;
         for (int q = consumed; rank == 0 && q < max(issued[0], issued[1]); ++q)
             mbar_wait_bounded(&full[q % NST], (uint32_t)((q / NST) & 1), &never, DIG_WAIT_NS);
-        for (int q = min(st_used[0], st_used[1]); q < st_issued; ++q)
+        // (a slot's earlier copies had landed when it was filled again, and a wait by parity would not see them)
+        for (int q = max(st_issued - DIG_NSU, 0); q < st_issued; ++q)
             mbar_wait_bounded(&st_full[q % DIG_NSU], (uint32_t)((q / DIG_NSU) & 1), &never, DIG_WAIT_NS);
         atomicOr(A.err, kErrTimeout);
     }

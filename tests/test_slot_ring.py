@@ -20,11 +20,13 @@ def constant(name):
     return int(re.search(r"\b%s = (\d+)" % name, DIG).group(1))
 
 
-def explore(slots, groups, tiles):
+def explore(slots, groups, tiles, first=None):
     """Every interleaving of a producer, copies in flight and `groups` consumers that take the items of a
     tile in turn (item p of a tile: group p % groups) and start a tile when all have finished the one
     before.  Returns the set of faults met: "early" (a wait returned although the copies of its item had
-    not landed) and "stuck" (nothing can move before all items are consumed)."""
+    not landed), "stuck" (nothing can move before all items are consumed) and "drain": had the kernel given
+    up here, waiting for items first(issued) to issued - 1 would miss copies in flight, or not return once
+    they have landed."""
     bounds = [0]
     for n in tiles:
         bounds.append(bounds[-1] + n)
@@ -44,6 +46,13 @@ def explore(slots, groups, tiles):
         # issued items; items in flight; completed `full` and `empty` phases per slot; items taken per group
         issued, flight, full, empty, taken = state
         moves = []
+        if first is not None:
+            landed = list(full)
+            for i in flight:
+                landed[i % slots] += 1
+            drained = range(first(issued), issued)
+            if any(i not in drained for i in flight) or any(landed[q % slots] % 2 == q // slots % 2 for q in drained):
+                faults.add("drain")
         if issued < bounds[-1]:
             s, k = issued % slots, issued // slots
             if k == 0 or empty[s] % 2 != (k - 1) % 2:           # parity wait for the release of item issued - slots
@@ -84,3 +93,11 @@ def test_the_model_sees_a_slot_that_changes_hands():
     assert "early" in explore(5, 2, (13,))
     assert explore(5, 1, (13,)) == set()
     assert explore(4, 2, (13,)) == set()
+
+
+def test_the_drain_after_giving_up_ends_with_the_last_copies():
+    S, G = constant("DIG_NSU"), constant("DIG_UPD_GROUPS")
+    assert re.search(r"for \(int q = max\(st_issued - DIG_NSU, 0\); q < st_issued; \+\+q\)", DIG)
+    assert explore(S, G, (5, 6, 3), lambda issued: max(issued - S, 0)) == set()
+    # from the start of the tile on, waits for copies that landed long ago would run into their limit
+    assert "drain" in explore(S, G, (13,), lambda issued: 0)
