@@ -101,10 +101,10 @@ struct DevBuf {
     template <class T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
-// Whether memory a call can do without (the digits of the dipole blocks for
-// the batched products) may be taken: at most an eighth of what the device and the
-// cap leave, so that allocations that are needed rarely meet it; one that does
-// gets it back (with_room).
+// Whether memory a call can do without (the digits of the batched products) may
+// be taken: at most an eighth of what the device and the cap leave, so that
+// allocations that are needed rarely meet it.  A later call of the same context
+// that does gets it back (with_room); other contexts and groups do not.
 static bool optional_room(size_t nbytes)
 {
     size_t free_b = 0, total = 0;
@@ -483,7 +483,8 @@ static bool dig_wanted(const tdse_ctx *ctx, int B)
     if (ctx->prec == TDSE_FP32) return ctx->n >= 56 || B <= 4;
     if (ctx->prec == TDSE_DF32) return ctx->n >= 56 || B <= 32;
     const long long elems = (long long)ctx->lmax * ctx->n * ctx->n;
-    return B >= (elems < 50000 ? 12 : elems < 150000 ? 8 : elems < 500000 ? 6 : elems < 2000000 ? 5 : elems < 8000000 ? 4 : 3);
+    if (elems < 500000) return B >= (elems < 50000 ? 12 : elems < 150000 ? 8 : 6);
+    return B >= (elems < 2000000 ? 5 : elems < 8000000 ? 4 : 3);
 }
 
 // A batch's workspace.  Once a batch has been captured into a caller's graph,
@@ -1019,7 +1020,7 @@ static tdse_status propagate_impl(tdse_ctx *ctx, double *c, const double *field,
 }
 
 static tdse_status propagate_once(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt,
-                           long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+                                  long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
 {
     g_err.clear();
     tdse_status st = check_prop_args(ctx, c, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold);
@@ -1032,14 +1033,17 @@ static tdse_status propagate_once(tdse_ctx *ctx, double *c, const double *field,
                           (cudaStream_t)stream);
 }
 
-tdse_status tdse_propagate(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+tdse_status tdse_propagate(tdse_ctx *ctx, double *c, const double *field, int samples_per_step, double dt, long nsteps,
+                           tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
 {
-    return with_room(ctx, [&] { return propagate_once(ctx, c, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
+    return with_room(ctx, [&] {
+        return propagate_once(ctx, c, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream);
+    });
 }
 
 static tdse_status propagate_rkf45_once(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1,
-                                 double dt0, double tol, double dt_min, double dt_max, long max_attempts,
-                                 tdse_rkf_stats *stats, void *stream)
+                                        double dt0, double tol, double dt_min, double dt_max, long max_attempts,
+                                        tdse_rkf_stats *stats, void *stream)
 {
     g_err.clear();
     if (!ctx || !c || !field) return fail(TDSE_EINVAL, "NULL argument");
@@ -1131,14 +1135,18 @@ static tdse_status propagate_rkf45_once(tdse_ctx *ctx, double *c, const tdse_fie
     return TDSE_OK;
 }
 
-tdse_status tdse_propagate_rkf45(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1, double dt0, double tol, double dt_min, double dt_max, long max_attempts, tdse_rkf_stats *stats, void *stream)
+tdse_status tdse_propagate_rkf45(tdse_ctx *ctx, double *c, const tdse_field_fn *field, double t0, double t1,
+                                 double dt0, double tol, double dt_min, double dt_max, long max_attempts,
+                                 tdse_rkf_stats *stats, void *stream)
 {
-    return with_room(ctx, [&] { return propagate_rkf45_once(ctx, c, field, t0, t1, dt0, tol, dt_min, dt_max, max_attempts, stats, stream); });
+    return with_room(ctx, [&] {
+        return propagate_rkf45_once(ctx, c, field, t0, t1, dt0, tol, dt_min, dt_max, max_attempts, stats, stream);
+    });
 }
 
 static tdse_status propagate_host_once(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step,
-                                double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
-                                void *stream)
+                                       double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
+                                       void *stream)
 {
     g_err.clear();
     if (!ctx || !c_host || !field_host) return fail(TDSE_EINVAL, "NULL argument");
@@ -1164,9 +1172,14 @@ static tdse_status propagate_host_once(tdse_ctx *ctx, double *c_host, const doub
     return tdse_sync(ctx, stream);
 }
 
-tdse_status tdse_propagate_host(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+tdse_status tdse_propagate_host(tdse_ctx *ctx, double *c_host, const double *field_host, int samples_per_step,
+                                double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
+                                void *stream)
 {
-    return with_room(ctx, [&] { return propagate_host_once(ctx, c_host, field_host, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
+    return with_room(ctx, [&] {
+        return propagate_host_once(ctx, c_host, field_host, samples_per_step, dt, nsteps, scheme, taylor_order,
+                                   taylor_hold, stream);
+    });
 }
 
 tdse_status tdse_set_gauge(tdse_ctx *ctx, tdse_gauge gauge)
@@ -1377,8 +1390,8 @@ static tdse_status propagate_batch_df(tdse_ctx *ctx, double *c, const double *fi
 }
 
 static tdse_status propagate_batch_once(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step,
-                                 double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
-                                 void *stream)
+                                        double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
+                                        void *stream)
 {
     g_err.clear();
     tdse_status st = check_prop_args(ctx, c, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold);
@@ -1455,9 +1468,13 @@ static tdse_status propagate_batch_once(tdse_ctx *ctx, double *c, const double *
     return TDSE_OK;
 }
 
-tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
+tdse_status tdse_propagate_batch(tdse_ctx *ctx, double *c, const double *field, int B, int samples_per_step, double dt,
+                                 long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, void *stream)
 {
-    return with_room(ctx, [&] { return propagate_batch_once(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, stream); });
+    return with_room(ctx, [&] {
+        return propagate_batch_once(ctx, c, field, B, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold,
+                                    stream);
+    });
 }
 
 // Field samples that a stage's field value depends on, with weights
@@ -1474,8 +1491,9 @@ static void field_deps(int sps, long k, int h, long long *i0, long long *i1, dou
 }
 
 static tdse_status adjoint_once(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt,
-                         long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, const double *weights,
-                         int checkpoint_every, double *grad_field, double *c_final, double *loss, void *stream)
+                                long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold,
+                                const double *weights, int checkpoint_every, double *grad_field, double *c_final,
+                                double *loss, void *stream)
 {
     g_err.clear();
     tdse_status st = check_prop_args(ctx, c0, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold);
@@ -1660,9 +1678,14 @@ static tdse_status adjoint_once(tdse_ctx *ctx, const double *c0, const double *f
     return TDSE_OK;
 }
 
-tdse_status tdse_adjoint(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt, long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, const double *weights, int checkpoint_every, double *grad_field, double *c_final, double *loss, void *stream)
+tdse_status tdse_adjoint(tdse_ctx *ctx, const double *c0, const double *field, int samples_per_step, double dt,
+                         long nsteps, tdse_scheme scheme, int taylor_order, int taylor_hold, const double *weights,
+                         int checkpoint_every, double *grad_field, double *c_final, double *loss, void *stream)
 {
-    return with_room(ctx, [&] { return adjoint_once(ctx, c0, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, weights, checkpoint_every, grad_field, c_final, loss, stream); });
+    return with_room(ctx, [&] {
+        return adjoint_once(ctx, c0, field, samples_per_step, dt, nsteps, scheme, taylor_order, taylor_hold, weights,
+                            checkpoint_every, grad_field, c_final, loss, stream);
+    });
 }
 
 // Systems whose rows take the same thread layout share one product launch.
