@@ -1257,7 +1257,10 @@ tdse_status tdse_populations(tdse_ctx *ctx, const double *c, int B, double *per_
     if (!aligned16(c)) return fail(TDSE_EINVAL, "c must be 16-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
     const int L = ctx->lmax + 1;
-    CUDA_TRY(ctx->part.ensure(sizeof(double) * 3 * (size_t)B * L));
+    const size_t pb = sizeof(double) * 3 * (size_t)B * L;
+    if (ctx->part.ensure(pb) == cudaErrorMemoryAllocation) (void)shed(ctx);
+    (void)cudaGetLastError();
+    CUDA_TRY(ctx->part.ensure(pb));
     CUDA_TRY(tdse::launch_pop_blocks((const double2 *)c, ctx->E.as<double>(), ctx->lmax, ctx->n, B, per_state, per_l,
                                      ctx->part.as<double>(), s));
     CUDA_TRY(tdse::launch_pop_totals(ctx->part.as<double>(), L, B, nullptr, bound, ionised, s));
@@ -1272,7 +1275,10 @@ tdse_status tdse_norm(tdse_ctx *ctx, const double *c, int B, double *out, void *
     if (!aligned16(c)) return fail(TDSE_EINVAL, "c must be 16-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
     const int L = ctx->lmax + 1;
-    CUDA_TRY(ctx->part.ensure(sizeof(double) * 3 * (size_t)B * L));
+    const size_t pb = sizeof(double) * 3 * (size_t)B * L;
+    if (ctx->part.ensure(pb) == cudaErrorMemoryAllocation) (void)shed(ctx);
+    (void)cudaGetLastError();
+    CUDA_TRY(ctx->part.ensure(pb));
     CUDA_TRY(tdse::launch_pop_blocks((const double2 *)c, ctx->E.as<double>(), ctx->lmax, ctx->n, B, nullptr, nullptr,
                                      ctx->part.as<double>(), s));
     CUDA_TRY(tdse::launch_pop_totals(ctx->part.as<double>(), L, B, out, nullptr, nullptr, s));

@@ -418,3 +418,18 @@ def test_few_fp64_pulses_run_one_by_one(tdse_lib, lmax, n, few, many):
     # 80 stages, each rounding once: the states agree to their FP64 rounding
     assert np.linalg.norm(out[0] - out[1][:few]) <= 80 * 2.0 ** -52 * np.linalg.norm(out[0])
     H.close()
+
+
+def test_observables_get_the_digits_memory(tdse_lib):
+    lmax, n, B = 2, 200, 64
+    H = tdse_lib.Hamiltonian(inputs.energies(lmax, n), inputs.dipoles(lmax, n, 8), lmax, n, "df32")
+    run_batch(H, B, 1)
+    c = torch.from_numpy(np.stack([inputs.random_state(H.N, b) for b in range(B)])).cuda()
+    held = tdse_lib.device_memory_in_use()
+    tdse_lib.set_device_memory_limit(held + 16)
+    try:
+        norms = H.norm(c, B).cpu().numpy()
+    finally:
+        tdse_lib.set_device_memory_limit(0)
+    assert np.allclose(norms, 1.0, rtol=0, atol=1e-12) and tdse_lib.device_memory_in_use() < held
+    H.close()
