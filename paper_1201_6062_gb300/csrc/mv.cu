@@ -263,21 +263,25 @@ cudaError_t launch_mv(int prec, const MvCfg &cfg, int grid, const SysDesc *sys, 
 // Per amplitude a = (m, i):  D x = R[a] (m < lmax) + sum of the column
 // partial slots of block m-1 (m >= 1), in slot order;  then H x = E x + f D x
 // and the stage / term update of the chosen scheme, all in FP64.
-// Four blocks of 64 amplitudes, two threads each, per entry of blk: bound by the
-// latency of the FP64 instructions, of which an SM completes one a warp in 16
-// cycles, so few amplitudes an SM.  FP32, lmax=28, n=108, us a stage with its
-// product: 12.7 with a thread an amplitude and 256 a block, 11.3 so; lmax=6,
-// n=300 12.0 and 10.2 (two threads each but 256 amplitudes a block: 11.6).
-template <class P>
-__global__ void __launch_bounds__(128, 8)                // (without the 8, 40 registers: the slots read one by one)
+// T / 2 amplitudes a block, two threads each, 512 / T blocks per entry of blk:
+// bound by the latency of the FP64 instructions, of which an SM completes one a
+// warp in 16 cycles, so few amplitudes an SM.  FP32, lmax=28, n=108, us a stage with
+// its product: 12.7 with a thread an amplitude and 256 a block, 11.3 so with T =
+// 128; lmax=6, n=300 12.0 and 10.2.  Registers: 64 read eight slots at a time; the
+// larger blocks take 48, since blocks that wait beside a product leave the next
+// product's CTA too few otherwise (lmax=15, n=1000 17.1 us a stage with T = 512,
+// 20.7 with 64 registers).
+template <class P, int T>
+__global__ void __maxnreg__(T == 128 ? 64 : 48)
 epi_kernel(const SysDesc *__restrict__ sys, const int2 *__restrict__ blk, EpiArgs A)
 {
     pdl_launch_dependents();
     // The plan, the descriptor, the energies and the slot ranges are the same
     // for every launch of a call: read them before waiting for the product.
-    const int2 bm = blk[blockIdx.x >> 2];
+    constexpr int PER = 512 / T;
+    const int2 bm = blk[blockIdx.x / PER];
     const SysDesc S = sys[bm.x];
-    const long long a = (long long)bm.y + (((blockIdx.x & 3) * 128 + threadIdx.x) >> 1);
+    const long long a = (long long)bm.y + (((blockIdx.x % PER) * T + threadIdx.x) >> 1);
     const int own = threadIdx.x & 1;
     const bool live = a < S.N;
     const EpiPre pre = live ? epi_pre(S, a) : EpiPre{};
@@ -355,24 +359,43 @@ cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaS
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+template <class P> static const void *epi_fn(int per)
+{
+    if (per == 4) return (const void *)epi_kernel<P, 128>;
+    return per == 2 ? (const void *)epi_kernel<P, 256> : (const void *)epi_kernel<P, 512>;
+}
+
 // early: start while the product still runs.  Not for groups of systems, whose
 // products (of several streams, or several CTAs an SM) lack the room that the
 // waiting blocks take (FP32, us for 4 steps: 12 systems 1087 early, 1019 not; 6
-// systems 460 and 420).
+// systems 460 and 420).  Blocks that start early are as small as leaves no more of
+// them than SMs: where some SMs hold two, the product's CTAs come late.  FP32, us a
+// stage with blocks of 64 / 128 / 256 amplitudes: lmax=15, n=500 (126 blocks of 64)
+// 9.9 / 10.3 / 11.6, lmax=20, n=500 (165) 14.7 / 11.3 / 12.5, lmax=15, n=1000 (250)
+// 20.6 / 15.7 / 17.1, lmax=31, n=700 (350) 20.6 / 21.1 / 18.3, lmax=31, n=2000 83.8 /
+// 83.6 / 83.2.
 cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream, bool early)
 {
     if (nblk <= 0) return cudaSuccess;
-    const void *fn = nullptr;
-    switch (prec) {
-    case 0: fn = (const void *)epi_kernel<PolF64>; break;
-    case 1: fn = (const void *)epi_kernel<PolF32>; break;
-    case 2: fn = (const void *)epi_kernel<PolDF32>; break;
-    default: return cudaErrorInvalidValue;
-    }
     if (a.mode == EPI_RK4) a.s = a.stage == 3 ? a.dt / 6.0 : (a.stage == 2 ? a.dt : 0.5 * a.dt);
     else if (a.mode == EPI_TAYLOR) a.s = a.dt / (double)a.stage;
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&a};
-    return launch_pdl(fn, dim3(4 * nblk), dim3(128), 0, stream, args, early);
+    int per = 4;                                             // blocks an entry of blk
+    if (early) {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        while (per > 1 && (long long)per * nblk > sms) per /= 2;
+    }
+    const void *fn = nullptr;
+    switch (prec) {
+    case 0: fn = epi_fn<PolF64>(per); break;
+    case 1: fn = epi_fn<PolF32>(per); break;
+    case 2: fn = epi_fn<PolDF32>(per); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return launch_pdl(fn, dim3(per * nblk), dim3(512 / per), 0, stream, args, early);
 }
 
 __global__ void bump_kernel(long long *kdev) { *kdev += 1; }

@@ -135,3 +135,32 @@ def test_products_queued_without_a_wait(tdse_lib, lmax, n, prec, tol):
         ref = oracle.hmatvec(lmax, n, E, U, 0.3, X[i])
         assert np.linalg.norm(y[i].cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
     H.close()
+
+
+# 256, 128 and 64 amplitudes a block of the update (fewer blocks than SMs where it starts early), the last one ragged
+@pytest.mark.parametrize("lmax,n", [(31, 653), (20, 487), (7, 301)])
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-14), ("df32", 1e-11), ("fp32", 2e-6)])
+def test_update_blocks(tdse_lib, lmax, n, prec, tol):
+    """One product and one RK4 step against plain FP64 arithmetic."""
+    U, c = random(lmax, n, 7)
+    c /= np.linalg.norm(c)
+    E, dt, f = inputs.energies(lmax, n), 0.01, 0.05
+
+    def hx(y):
+        x = y.reshape(lmax + 1, n)
+        d = np.zeros_like(x)
+        d[:-1] += np.einsum("lij,lj->li", U, x[1:], optimize=True)
+        d[1:] += np.einsum("lij,li->lj", U, x[:-1], optimize=True)
+        return E * y + f * d.reshape(-1)
+
+    H = tdse_lib.Hamiltonian(E, U, lmax, n, prec)
+    x = torch.from_numpy(c.copy()).cuda()
+    ref = hx(c)
+    assert np.linalg.norm(H.hmatvec(x, f).cpu().numpy() - ref) <= tol * np.linalg.norm(ref)
+    H.propagate(x, torch.full((2,), f, dtype=torch.float64, device="cuda"), dt, 1)
+    k1 = -1j * ref
+    k2 = -1j * hx(c + 0.5 * dt * k1)
+    k3 = -1j * hx(c + 0.5 * dt * k2)
+    ref = c + dt / 6.0 * (k1 + 2.0 * k2 + 2.0 * k3 - 1j * hx(c + dt * k3))
+    assert np.linalg.norm(x.cpu().numpy() - ref) <= tol
+    H.close()
