@@ -84,10 +84,12 @@ __global__ void __launch_bounds__(256) lz_init(const SysDesc *__restrict__ sys, 
 // The vector kernels are bound by the latency of loads and block sums and by the
 // FP64 pipe, which takes 16 cycles a warp instruction and SM.  So one thread takes
 // the root and the reciprocal (some 40 FP64 instructions, formerly in every warp),
-// and lz_orth requests its vectors before it sums the partials.  Product and both
-// kernels, us a Krylov vector: FP32, lmax=31, n=2000 116.4 -> 109.0; float-float,
-// lmax=15, n=500 46.4 -> 43.0 (with D x's slots eight at a time and its loads ahead
-// of the sum in lz_apply too: 113.1 and 50.1).
+// and with FP32 products lz_orth requests its vectors before it sums the partials.
+// Product and both kernels, us a Krylov vector, before and now: FP32, lmax=31,
+// n=2000 114.7 and 107.2, n=700 38.1 and 34.3; float-float, lmax=15, n=500 44.7 and
+// 41.1, lmax=31, n=700 54.9 and 54.6 (58.3 with the vectors requested first); FP64,
+// lmax=25, n=800 210.4 and 210.0 (214.2).  D x's slots eight at a time and its loads
+// ahead of the sum in lz_apply too took 50.1 at lmax=15, n=500.
 //
 // j = 0: x = v_0.  j > 0: b_j = |w| from the partials of lz_orth, x = v_j =
 // w / b_j (stored; zero after a breakdown), and the block products, taken of
@@ -149,14 +151,21 @@ __global__ void __launch_bounds__(256) lz_orth(const SysDesc *__restrict__ sys, 
     const SysDesc &S = sys[0];
     const long long a = (long long)blockIdx.x * 256 + threadIdx.x;
     const bool live = a < S.N;
+    // FP32 products: the vectors are requested before the sum.  Not beside FP64 and
+    // float-float ones, whose CTAs lack the registers that takes (42 against 32 a
+    // thread) and come late.
+    constexpr bool kAhead = sizeof(typename P::Elem) == 4;
     double2 x = make_double2(0.0, 0.0), ww = x, y = x;
-    if (live) {
+    const auto load = [&]() {
+        if (!live) return;
         x = vj[a];
         ww = w[a];
         if (j > 0) y = vjm1[a];
-    }
+    };
+    if constexpr (kAhead) load();
     const double beta = j > 0 ? scal[1 + 64 + j] : 0.0;      // b_j
     const double alpha = lz_sum_parts(parts_a, nparts, sh);
+    if constexpr (!kAhead) load();
     if (blockIdx.x == 0 && threadIdx.x == 0) scal[1 + j] = alpha;
     double v = 0.0;
     if (live) {
