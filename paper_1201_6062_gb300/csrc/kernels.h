@@ -124,6 +124,8 @@ struct EpiArgs {
 cudaError_t launch_bump(long long *kdev, cudaStream_t stream);
 cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream,
                        bool early = true);
+// Whether the updates of a group with this many entries of blk start early (launch_epi).
+bool epi_early(int nblk);
 
 // --- adjoint (adj.cu) ---
 // A pending scalar: the sum of parts[0..n) (fixed order) is added, times w0 and

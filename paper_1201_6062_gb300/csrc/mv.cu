@@ -359,33 +359,44 @@ cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaS
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
+static int epi_sms()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+    return sms;
+}
+
+bool epi_early(int nblk) { return 4LL * nblk <= epi_sms(); }
+
 template <class P> static const void *epi_fn(int per)
 {
     if (per == 4) return (const void *)epi_kernel<P, 128>;
     return per == 2 ? (const void *)epi_kernel<P, 256> : (const void *)epi_kernel<P, 512>;
 }
 
-// early: start while the product still runs.  Not for groups of systems, whose
-// products (of several streams, or several CTAs an SM) lack the room that the
-// waiting blocks take (FP32, us for 4 steps: 12 systems 1087 early, 1019 not; 6
-// systems 460 and 420).  Blocks that start early are as small as leaves no more of
-// them than SMs: where some SMs hold two, the product's CTAs come late.  FP32, us a
-// stage with blocks of 64 / 128 / 256 amplitudes: lmax=15, n=500 (126 blocks of 64)
-// 9.9 / 10.3 / 11.6, lmax=20, n=500 (165) 14.7 / 11.3 / 12.5, lmax=15, n=1000 (250)
-// 20.6 / 15.7 / 17.1, lmax=31, n=700 (350) 20.6 / 21.1 / 18.3, lmax=31, n=2000 83.8 /
-// 83.6 / 83.2.
-cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream, bool early)
+// early: start while the product still runs.  Blocks that do are as small as leaves
+// no more of them than SMs: where some SMs hold two, the product's CTAs come late.
+// FP32, us a stage with blocks of 64 / 128 / 256 amplitudes: lmax=15, n=500 (126
+// blocks of 64) 9.9 / 10.3 / 11.6, lmax=20, n=500 (165) 14.7 / 11.3 / 12.5, lmax=15,
+// n=1000 (250) 20.6 / 15.7 / 17.1, lmax=31, n=700 (350) 20.6 / 21.1 / 18.3, lmax=31,
+// n=2000 83.8 / 83.6 / 83.2.
+// Groups of systems, but small ones (epi_early), do not start early: their products
+// (of several streams, or several CTAs an SM) lack the room that many waiting blocks
+// take; 128 amplitudes a block then.  us a step, early with blocks of 64 / not early
+// with 64 / 128 amplitudes: FP32, 4 systems (some 80 blocks of 64) 56 / 61 / 64, 3
+// (some 200) 95 / 96 / 80, 12 (1100) 277 / 254 / 254; float-float, 5 (128) 95 / 141 /
+// 156, 16 (400) 196 / 186 / 186.
+cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream,
+                       bool early)
 {
     if (nblk <= 0) return cudaSuccess;
     if (a.mode == EPI_RK4) a.s = a.stage == 3 ? a.dt / 6.0 : (a.stage == 2 ? a.dt : 0.5 * a.dt);
     else if (a.mode == EPI_TAYLOR) a.s = a.dt / (double)a.stage;
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&a};
-    int per = 4;                                             // blocks an entry of blk
+    int per = early ? 4 : 2;                                 // blocks an entry of blk
     if (early) {
-        int dev = 0, sms = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
+        const int sms = epi_sms();
         while (per > 1 && (long long)per * nblk > sms) per /= 2;
     }
     const void *fn = nullptr;
