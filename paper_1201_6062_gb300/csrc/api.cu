@@ -1948,7 +1948,8 @@ static tdse_status group_step(tdse_group *g, int sps, double dt, cudaStream_t s,
     a.sps = sps;
     a.dt = dt;
     a.kdev = g->kdev.as<long long>();
-    const bool early = tdse::epi_early(g->plan.nblk);
+    bool early;
+    const int per = tdse::epi_group(g->plan.nblk, &early);
     if (fork) {
         // Each bucket runs its four stages (product, then its members' update)
         // on a stream of its own: a system's update needs only its own
@@ -1963,7 +1964,8 @@ static tdse_status group_step(tdse_group *g, int sps, double dt, cudaStream_t s,
                 a.stage = q;
                 tdse_status st = bucket_product(g, bk, bucket_cfg(bk), sb);
                 if (st != TDSE_OK) return st;
-                CUDA_TRY(tdse::launch_epi(g->prec, bk.nblk, bk.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, sb, early));
+                CUDA_TRY(tdse::launch_epi(g->prec, bk.nblk, bk.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, sb, early,
+                                          per));
             }
             CUDA_TRY(cudaEventRecord(fork->done[b], sb));
             CUDA_TRY(cudaStreamWaitEvent(s, fork->done[b], 0));
@@ -1973,7 +1975,8 @@ static tdse_status group_step(tdse_group *g, int sps, double dt, cudaStream_t s,
             a.stage = q;
             tdse_status st = group_product(g, s);
             if (st != TDSE_OK) return st;
-            CUDA_TRY(tdse::launch_epi(g->prec, g->plan.nblk, g->plan.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, s, early));
+            CUDA_TRY(tdse::launch_epi(g->prec, g->plan.nblk, g->plan.blk.as<int2>(), g->ddesc.as<SysDesc>(), a, s, early,
+                                      per));
         }
     }
     CUDA_TRY(tdse::launch_bump(g->kdev.as<long long>(), s));

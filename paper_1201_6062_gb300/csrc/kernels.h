@@ -123,9 +123,9 @@ struct EpiArgs {
 // *kdev += 1 (one thread): advances the step index of a captured step graph.
 cudaError_t launch_bump(long long *kdev, cudaStream_t stream);
 cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream,
-                       bool early = true);
-// Whether the updates of a group with this many entries of blk start early (launch_epi).
-bool epi_early(int nblk);
+                       bool early = true, int per = 0);
+// For the updates of a group with this many entries of blk: whether they start early, blocks an entry.
+int epi_group(int nblk, bool *early);
 
 // --- adjoint (adj.cu) ---
 // A pending scalar: the sum of parts[0..n) (fixed order) is added, times w0 and

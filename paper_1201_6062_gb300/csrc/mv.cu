@@ -367,7 +367,19 @@ static int epi_sms()
     return sms;
 }
 
-bool epi_early(int nblk) { return 4LL * nblk <= epi_sms(); }
+// The products of a group (of several streams, or several CTAs an SM) lack the room
+// that many waiting blocks take: early with small blocks for small groups, with 256
+// amplitudes a block for middling ones, else not early and 128 amplitudes a block.
+// us a step, early with 64 / early with 256 / not early with 128: FP32, 4 systems (20
+// entries of blk) 56 / 67 / 64, 3 (50) 95 / 82 / 80, 6 (52) 110 / 101 / 102, 12 (280)
+// 277 / 268 / 254; float-float, 5 (32) 95 / 98 / 156, 12 (64) 162 / 166 / 192, 16 (100)
+// 196 / 196 / 186.
+int epi_group(int nblk, bool *early)
+{
+    const long long sms = epi_sms();
+    *early = 2LL * nblk <= sms;
+    return 4LL * nblk <= sms ? 4 : (*early ? 1 : 2);
+}
 
 template <class P> static const void *epi_fn(int per)
 {
@@ -381,23 +393,17 @@ template <class P> static const void *epi_fn(int per)
 // blocks of 64) 9.9 / 10.3 / 11.6, lmax=20, n=500 (165) 14.7 / 11.3 / 12.5, lmax=15,
 // n=1000 (250) 20.6 / 15.7 / 17.1, lmax=31, n=700 (350) 20.6 / 21.1 / 18.3, lmax=31,
 // n=2000 83.8 / 83.6 / 83.2.
-// Groups of systems, but small ones (epi_early), do not start early: their products
-// (of several streams, or several CTAs an SM) lack the room that many waiting blocks
-// take; 128 amplitudes a block then.  us a step, early with blocks of 64 / not early
-// with 64 / 128 amplitudes: FP32, 4 systems (some 80 blocks of 64) 56 / 61 / 64, 3
-// (some 200) 95 / 96 / 80, 12 (1100) 277 / 254 / 254; float-float, 5 (128) 95 / 141 /
-// 156, 16 (400) 196 / 186 / 186.
+// per: blocks an entry of blk (4, 2 or 1), 0: by that rule.
 cudaError_t launch_epi(int prec, int nblk, const int2 *blk, const SysDesc *sys, EpiArgs a, cudaStream_t stream,
-                       bool early)
+                       bool early, int per)
 {
     if (nblk <= 0) return cudaSuccess;
     if (a.mode == EPI_RK4) a.s = a.stage == 3 ? a.dt / 6.0 : (a.stage == 2 ? a.dt : 0.5 * a.dt);
     else if (a.mode == EPI_TAYLOR) a.s = a.dt / (double)a.stage;
     void *args[] = {(void *)&sys, (void *)&blk, (void *)&a};
-    int per = early ? 4 : 2;                                 // blocks an entry of blk
-    if (early) {
+    if (per == 0) {
         const int sms = epi_sms();
-        while (per > 1 && (long long)per * nblk > sms) per /= 2;
+        for (per = 4; per > 1 && (long long)per * nblk > sms;) per /= 2;
     }
     const void *fn = nullptr;
     switch (prec) {
