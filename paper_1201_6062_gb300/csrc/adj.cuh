@@ -78,7 +78,7 @@ __device__ __forceinline__ double adj_amp(const SysDesc &S, long long a, const A
 // The same in halves (epi.cuh, per component): a thread assembles one
 // component of u = D g and updates the other one's cotangents; returns its
 // part of Im(conj(u) x).  lmax=15, n=500, FP64, 64 RK4 steps and gradient:
-// 23.5 -> 17.8 ms.
+// 36.6 -> 34.6 ms.
 enum AdjKind { AK_RK4_LAST, AK_RK4_MID, AK_RK4_FIRST, AK_TAYLOR };      // RK4 stage 3; 2, 1; 0
 
 struct AdjHalf {

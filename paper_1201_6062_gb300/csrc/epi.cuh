@@ -33,8 +33,8 @@ __device__ __forceinline__ EpiPre epi_pre(const SysDesc &S, long long a)
 // because the compiler evaluates short alternatives of a uniform branch side by
 // side and every FP64 instruction takes 64 cycles of its scheduler.  Bound by the
 // latency of those instructions and of the loads: a stage of the persistent
-// kernel 21.0 -> 18.7 us float-float and 30.9 -> 23.5 us FP64 at lmax=15, n=500,
-// 24.2 -> 16.9 us FP64 at lmax=7, n=301 (from one thread an amplitude).
+// kernel 21.0 -> 18.7 us float-float and 47.6 -> 44.7 us FP64 at lmax=15, n=500,
+// 27.2 -> 23.9 us FP64 at lmax=7, n=301 (from one thread an amplitude).
 enum EpiKind { EK_RK4_FIRST, EK_RK4_MID, EK_RK4_LAST, EK_TAYLOR, EK_HX, EK_MIHX };
 
 struct EpiHalf {
